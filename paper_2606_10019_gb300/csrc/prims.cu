@@ -6,6 +6,7 @@
 #include <cstring>
 
 #include "common.cuh"
+#include "csort.cuh"
 
 namespace gcvo {
 
@@ -175,13 +176,16 @@ gcvo_status scan_inclusive_max(int *data, int64_t n, void *scratch, cudaStream_t
 // RS_ITEMS * 32 consecutive items; per pass: digit histogram per tile
 // (digit-major layout), one inclusive scan over all (digit, tile) counts,
 // then a scatter in which each warp walks its tile in order, ranking equal
-// digits with __match_any_sync so that the order of equal keys is kept.
+// digits with ballots so that the order of equal keys is kept.  Up to
+// csort::MAX_N keys of at most csort::MAX_KEY_BITS bits the whole sort runs in
+// one cluster instead (csort.cuh), in one launch.
 // ---------------------------------------------------------------------------
 namespace {
 
 constexpr int RS_ITEMS = 16;
 constexpr int RS_TILE = 32 * RS_ITEMS;
 constexpr int RS_WARPS = 8;
+constexpr int RS_LOADS = 8;    // pairs a lane has in flight
 
 __global__ void rs_hist(const unsigned long long *keys, int64_t n, int shift, int n_tiles, int *hist) {
     __shared__ int cnt[RS_WARPS][256];
@@ -191,6 +195,7 @@ __global__ void rs_hist(const unsigned long long *keys, int64_t n, int shift, in
     int tile = blockIdx.x * RS_WARPS + w;
     if (tile < n_tiles) {
         int64_t base = (int64_t)tile * RS_TILE;
+#pragma unroll
         for (int it = 0; it < RS_ITEMS; ++it) {
             int64_t i = base + it * 32 + lane;
             if (i < n) atomicAdd(&cnt[w][(int)((keys[i] >> shift) & 255ull)], 1);
@@ -213,25 +218,103 @@ __global__ void rs_scatter(const unsigned long long *keys_in, const int *vals_in
     __syncwarp();
     int64_t base = (int64_t)tile * RS_TILE;
     unsigned lt = (1u << lane) - 1u;
-    for (int it = 0; it < RS_ITEMS; ++it) {
-        int64_t i = base + it * 32 + lane;
-        bool valid = i < n;
-        unsigned long long k = valid ? keys_in[i] : 0ull;
-        int d = valid ? (int)((k >> shift) & 255ull) : 256 + lane;
-        unsigned peers = __match_any_sync(0xffffffffu, d);
-        int leader = __ffs(peers) - 1;
-        int rank = __popc(peers & lt);
-        int b = 0;
-        if (valid && lane == leader) {
-            b = run[w][d];
-            run[w][d] = b + __popc(peers);
+#pragma unroll 1
+    for (int h = 0; h < RS_ITEMS; h += RS_LOADS) {
+        unsigned long long key[RS_LOADS];
+        int val[RS_LOADS];
+#pragma unroll
+        for (int q = 0; q < RS_LOADS; ++q) {
+            const int64_t i = base + (h + q) * 32 + lane;
+            key[q] = i < n ? keys_in[i] : 0ull;
+            val[q] = i < n ? vals_in[i] : 0;
         }
-        b = __shfl_sync(0xffffffffu, b, leader);
-        if (valid) {
-            keys_out[b + rank] = k;
-            vals_out[b + rank] = vals_in[i];
+#pragma unroll
+        for (int q = 0; q < RS_LOADS; ++q) {
+            const bool valid = base + (h + q) * 32 + lane < n;
+            const int d = (int)((key[q] >> shift) & 255ull);
+            const unsigned peers = csort::same_digit(d, __ballot_sync(0xffffffffu, valid));
+            const int rank = __popc(peers & lt);
+            int b = 0;
+            if (valid) b = run[w][d];
+            __syncwarp();
+            if (valid && rank == 0) run[w][d] = b + __popc(peers);
+            __syncwarp();
+            if (valid) {
+                keys_out[b + rank] = key[q];
+                vals_out[b + rank] = val[q];
+            }
         }
-        __syncwarp();
+    }
+}
+
+// The whole sort in one cluster (csort.cuh), in place.
+template <int ITEMS>
+__global__ void __launch_bounds__(csort::THREADS) k_cluster_sort(unsigned long long *keys, int *vals, int n, int bits) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    csort::Smem<ITEMS> &S = *reinterpret_cast<csort::Smem<ITEMS> *>(smem);
+    constexpr int TILE = csort::Smem<ITEMS>::TILE;
+    const int first = (int)csort::cluster_rank() * TILE;
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+        const int i = k * csort::THREADS + (int)threadIdx.x;
+        if (first + i < n) S.key[0][i] = keys[first + i] << csort::IDX_BITS | (unsigned)(first + i);
+    }
+    const int b = csort::sort<ITEMS>(S, n, bits);
+    unsigned long long key[ITEMS];
+    int val[ITEMS];
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+        const int i = k * csort::THREADS + (int)threadIdx.x;
+        if (first + i < n) {
+            key[k] = S.key[b][i];
+            val[k] = vals[key[k] & ((1u << csort::IDX_BITS) - 1u)];
+        }
+    }
+    csort::cluster_barrier(csort::cluster_blocks());   // every value read before any is replaced
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+        const int i = k * csort::THREADS + (int)threadIdx.x;
+        if (first + i < n) {
+            keys[first + i] = key[k] >> csort::IDX_BITS;
+            vals[first + i] = val[k];
+        }
+    }
+}
+
+template <int ITEMS>
+cudaError_t cluster_sort_attr() {
+    const cudaError_t e = cudaFuncSetAttribute(k_cluster_sort<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)sizeof(csort::Smem<ITEMS>));
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(k_cluster_sort<ITEMS>,
+                                                   cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+
+template <int ITEMS>
+gcvo_status cluster_sort_t(unsigned long long *keys, int *vals, int n, int bits, int blocks, cudaStream_t s) {
+    static const cudaError_t attr = cluster_sort_attr<ITEMS>();
+    GCVO_CUDA(attr);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(csort::THREADS);
+    cfg.dynamicSmemBytes = sizeof(csort::Smem<ITEMS>);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)blocks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    GCVO_CUDA(cudaLaunchKernelEx(&cfg, k_cluster_sort<ITEMS>, keys, vals, n, bits));
+    count_launches(1);
+    return GCVO_OK;
+}
+
+gcvo_status cluster_sort(unsigned long long *keys, int *vals, int n, int bits, int items, int blocks, cudaStream_t s) {
+    switch (items) {
+        case 1: return cluster_sort_t<1>(keys, vals, n, bits, blocks, s);
+        case 2: return cluster_sort_t<2>(keys, vals, n, bits, blocks, s);
+        default: return cluster_sort_t<4>(keys, vals, n, bits, blocks, s);
     }
 }
 
@@ -247,6 +330,9 @@ size_t radix_sort_scratch_bytes(int64_t n) {
 gcvo_status radix_sort_pairs(unsigned long long *keys, int *vals, int64_t n, int bits, void *scratch,
                              size_t scratch_bytes, cudaStream_t s) {
     if (n <= 1 || bits <= 0) return GCVO_OK;
+    int items, blocks;
+    csort::shape(n, items, blocks);
+    if (items && bits <= csort::MAX_KEY_BITS) return cluster_sort(keys, vals, (int)n, bits, items, blocks, s);
     if (scratch_bytes < radix_sort_scratch_bytes(n)) return GCVO_ERR_WORKSPACE;
     int n_tiles = (int)((n + RS_TILE - 1) / RS_TILE);
     auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
