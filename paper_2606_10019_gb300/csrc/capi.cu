@@ -712,9 +712,7 @@ std::vector<DevBuf *> ws_bufs(gcvo_ctx *c) {
                                &c->src_fx,    &c->t_fx,
                                &c->items,     &c->item_prob, &c->pack_tmp, &c->partial,   &c->partial2,
                                &c->probs,     &c->grids,     &c->evalout,  &c->logs,      &c->status_word,
-                               &c->knn_retry,  &c->knn_meta,  &c->knn_grid.ca, &c->grid_meta, &c->grid_tiles};
-    for (GridStore *g : {&c->knn_grid, &c->knn_grid2})
-        for (DevBuf *b : {&g->pos, &g->orig, &g->cell_start, &g->hkeys, &g->hval}) v.push_back(b);
+                               &c->knn_code,  &c->knn_pos,   &c->knn_cloud, &c->knn_meta, &c->grid_meta, &c->grid_tiles};
     return v;
 }
 
@@ -722,8 +720,6 @@ std::vector<size_t> ws_sizes(int64_t N, int64_t np, int64_t rows) {
     auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
     const size_t n = (size_t)std::max<int64_t>(N, 1);
     const size_t n64 = (n + 63) / 64 * 64;
-    size_t H = 64;
-    while (H < 2 * n) H <<= 1;
     const size_t small = al(np * sizeof(SrcDesc)) + al(np * sizeof(int)) * 7 + al(np * sizeof(int64_t)) +
                          al(sizeof(int)) * 4 + 256 + 4096;
     std::vector<size_t> v = {
@@ -745,15 +741,10 @@ std::vector<size_t> ws_sizes(int64_t N, int64_t np, int64_t rows) {
         np * sizeof(ProbDev), np * sizeof(GridDev), np * sizeof(EvalOut) + 256,
         (size_t)std::max<int64_t>(rows, 1) * sizeof(gcvo_iter_log),     // logs
         256,                                                            // status_word
-        2 * n * sizeof(int) + 256,                                      // knn_retry: two point lists
-        knn_meta_bytes((int64_t)n, (int)std::min<int64_t>(2 * np, (int64_t)n)),   // knn_meta
-        n * sizeof(float4),                                             // knn_grid.ca: gathered points
+        n * sizeof(unsigned long long), n * sizeof(float4), n * sizeof(int),   // knn_code, knn_pos, knn_cloud
+        knn_meta_bytes((int)std::min<int64_t>(2 * np, (int64_t)n)),     // knn_meta
         tgrid_meta_bytes((int)std::min<int64_t>(2 * np, (int64_t)n), (int64_t)n),   // grid_meta
         tgrid_tile_bytes(tgrid_max_tiles(1) + 2 * np)};                 // grid_tiles: one grid of 2^26 voxels
-    for (int g = 0; g < 2; ++g)
-        for (size_t b : {n * sizeof(float4), n * sizeof(int), (n + 1) * sizeof(int), H * sizeof(unsigned long long),
-                         H * sizeof(int)})
-            v.push_back(b);
     return v;
 }
 
@@ -837,13 +828,7 @@ gcvo_status gcvo_destroy(gcvo_ctx *ctx) {
                       &ctx->partial, &ctx->probs, &ctx->grids, &ctx->logs, &ctx->evalout, &ctx->status_word,
                       &ctx->items, &ctx->item_prob, &ctx->pack_tmp, &ctx->partial2};
     for (DevBuf *b : bufs) b->release();
-    for (GridStore *kg : {&ctx->knn_grid, &ctx->knn_grid2}) {
-        DevBuf *kb[] = {&kg->pos, &kg->ca, &kg->cb, &kg->plo, &kg->orig, &kg->cell_start, &kg->hkeys, &kg->hval,
-                        &kg->vox_first};
-        for (DevBuf *b : kb) b->release();
-    }
-    ctx->knn_retry.release();
-    ctx->knn_meta.release();
+    for (DevBuf *b : {&ctx->knn_code, &ctx->knn_pos, &ctx->knn_cloud, &ctx->knn_meta}) b->release();
     ctx->grid_meta.release();
     ctx->grid_tiles.release();
     ctx->clouds_stage.release();
@@ -983,9 +968,6 @@ gcvo_status gcvo_grid_destroy(gcvo_grid *grid) {
     s.plo.release();
     s.fx.release();
     s.orig.release();
-    s.cell_start.release();
-    s.hkeys.release();
-    s.hval.release();
     s.vox_first.release();
     delete grid;
     return GCVO_OK;

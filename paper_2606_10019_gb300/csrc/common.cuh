@@ -67,9 +67,8 @@ struct DevBuf {
 // from device memory).
 //
 // Points are sorted by voxel key.  pos[i] = (x - o, y - o, z - o, l0) for the
-// target grid (coordinates relative to the grid origin o, float32), and the
-// absolute coordinates for the internal kNN grid; ca[i] = (S00, S01, S02, S11),
-// cb[i] = (S12, S22, l1, l2).  Target grids also keep the rounding tails of
+// target grid (coordinates relative to the grid origin o, float32); ca[i] = (S00, S01, S02, S11),
+// cb[i] = (S12, S22, l1, l2).  The grids also keep the rounding tails of
 // the coordinates, plo[i] = (x - o) - pos[i].xyz (float), so that x - o =
 // pos + plo to about 2^-48 relative.  Voxel (cx, cy, cz) holds the points whose
 // coordinates c satisfy floor((c - corner) * inv_h) = (cx, cy, cz); its key is
@@ -83,13 +82,8 @@ struct GridDev {
     const float4 *plo;        // target grids: coordinate tails (x, y, z, 0)
     const float4 *fx;         // feature channels 3..6 (when feat_dim > 3)
     const int *orig;          // original index of each sorted point
-    const int *cell_start;    // n_cells + 1 offsets into the sorted points
-    const unsigned long long *hkeys;  // open-addressing table of voxel keys
-    const int *hval;          // voxel index of each table slot
-    const int *vox_first;     // target grids: first sorted point of every voxel, dense (+1 entry)
-    unsigned long long hmask; // table size - 1 (power of two)
-    unsigned long long key_base;   // batched kNN grids: offset of this cloud's voxel keys (0 otherwise)
-    double origin[3];         // o (target grid) or 0 (kNN grid), double
+    const int *vox_first;     // first sorted point of every voxel, dense (+1 entry)
+    double origin[3];         // o, double
     float corner[3];          // lowest voxel corner, in the coordinates of pos
     float h, inv_h;
     int dims[3];
@@ -99,30 +93,6 @@ struct GridDev {
     int feat_dim;
     int kernel_mode;
 };
-
-static constexpr unsigned long long EMPTY_KEY = ~0ull;
-
-__host__ __device__ inline unsigned long long hash_key(unsigned long long k) {
-    // splitmix64 finaliser
-    k ^= k >> 30;
-    k *= 0xbf58476d1ce4e5b9ull;
-    k ^= k >> 27;
-    k *= 0x94d049bb133111ebull;
-    k ^= k >> 31;
-    return k;
-}
-
-// Voxel index of `key`, or -1 when the voxel holds no point.
-__device__ inline int grid_lookup(const GridDev &g, unsigned long long key) {
-    unsigned long long s = hash_key(key) & g.hmask;
-    for (int probe = 0; probe <= (int)g.hmask; ++probe) {
-        unsigned long long k = __ldg(g.hkeys + s);
-        if (k == key) return __ldg(g.hval + s);
-        if (k == EMPTY_KEY) return -1;
-        s = (s + 1) & g.hmask;
-    }
-    return -1;
-}
 
 // ---------------------------------------------------------------------------
 // Primitives (prims.cu).
@@ -174,11 +144,11 @@ __host__ __device__ inline float sym3_min_eig(float a00, float a01, float a02, f
 }
 
 // ---------------------------------------------------------------------------
-// Grids (grid.cu).
+// Grids.
 // ---------------------------------------------------------------------------
 struct GridStore {
     GridDev d{};
-    DevBuf pos, ca, cb, plo, fx, orig, cell_start, hkeys, hval, vox_first;
+    DevBuf pos, ca, cb, plo, fx, orig, vox_first;
 };
 
 // Target grids of a batch of clouds in one set of launches (tgrid.cu):
@@ -197,8 +167,8 @@ size_t tgrid_meta_bytes(int n_clouds, int64_t n_points);
 size_t tgrid_tile_bytes(int64_t n_tiles);
 int64_t tgrid_max_tiles(int n_clouds);
 
-// kNN covariances of a batch of clouds in one set of launches: cloud k has
-// n[k] points at xyz[k] (3 x n SoA, device) and its own parameters kp[k];
+// kNN covariances of a batch of clouds in one set of launches (knn.cu):
+// cloud k has n[k] points at xyz[k] (3 x n SoA, device) and its own parameters kp[k];
 // Sigma goes to cov[k] (6 x n SoA, device).
 struct KnnJob {
     const float *xyz;
@@ -207,7 +177,7 @@ struct KnnJob {
     const gcvo_kernel_params *kp;
 };
 gcvo_status knn_covariances(gcvo_ctx *ctx, int n_clouds, const KnnJob *jobs);
-size_t knn_meta_bytes(int64_t n_points, int n_clouds);
+size_t knn_meta_bytes(int n_clouds);
 
 }  // namespace gcvo
 
@@ -231,13 +201,12 @@ struct gcvo_ctx {
     gcvo::DevBuf t_pos, t_ca, t_cb, t_lo, t_fx;      // the same at the current pose (k_transform)
     gcvo::DevBuf partial, probs, grids, logs, evalout, status_word, items, item_prob, pack_tmp;
     gcvo::DevBuf partial2;                           // second partial row of the G-CVO-E pass
-    gcvo::GridStore knn_grid, knn_grid2;             // reused by gcvo_estimate_covariances
-    gcvo::DevBuf knn_meta;                           // its per-cloud descriptors and grids
+    // covariances: Morton-sorted clouds (codes, points, cloud of each) and per-cloud descriptors
+    gcvo::DevBuf knn_code, knn_pos, knn_cloud, knn_meta;
     gcvo::DevBuf grid_meta, grid_tiles;              // target-grid builds: per-cloud data, scan tiles
     // gcvo_register_clouds: staged host clouds, covariances and target grids
     gcvo::DevBuf clouds_stage, clouds_cov;
     std::vector<gcvo_grid *> clouds_grids;
-    gcvo::DevBuf knn_retry;
     void *host_pinned = nullptr;
     size_t host_pinned_bytes = 0;
     int sm_count = 0;
