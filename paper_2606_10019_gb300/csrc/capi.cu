@@ -393,6 +393,7 @@ gcvo_status choose_schedule(gcvo_ctx *ctx, const Prepared &P, IterBufs &b) {
             for (auto &e : ev) cudaEventDestroy(e);
             if (st != GCVO_OK) return st;
             ctx->tuned.emplace_back(key, sched);
+            GCVO_CUDA(cudaMemsetAsync(b.work, 0, sizeof(int), ctx->stream));
         }
     }
     if (packed != sched) GCVO_TRY(pack(ctx, P, sched));
@@ -462,7 +463,8 @@ gcvo_status iter_bufs(gcvo_ctx *ctx, const Prepared &P, IterBufs &b, gcvo_iter_l
     f.chunk = chunk;
     f.chunk_cnt = chunk_cnt;
     f.n_chunks = work + 2;   // written by pack_items
-    f.reduce_blocks = std::max(1, ctx->sm_count) * 8;
+    f.reduce_blocks = (int)std::min<int64_t>((int64_t)n_chunk_rows, (int64_t)std::max(1, ctx->sm_count) * 8);
+    f.work = work;
     f.evalout = ctx->evalout.as<EvalOut>();
     f.logs = dlogs;
     f.n_active = n_active;
@@ -516,11 +518,11 @@ gcvo_status prof_end(gcvo_ctx *ctx, cudaStream_t s, bool capturing, long long sl
     return GCVO_OK;
 }
 
-// One pair pass on stream s (the work counter is reset first); evaluation
-// and G-CVO-E passes are timed when profiling.
+// One pair pass on stream s (the work counter is zero: prepare cleared it, and
+// every finalize clears it again); evaluation and G-CVO-E passes are timed when
+// profiling.
 gcvo_status launch_pair_pass(gcvo_ctx *ctx, const Prepared &P, IterBufs &b, int mode, cudaStream_t s,
                              bool capturing = false) {
-    GCVO_CUDA(cudaMemsetAsync(b.work, 0, sizeof(int), s));
     long long slot = -1;
     if (mode == PAIR_EVAL || mode == PAIR_EXACT) GCVO_TRY(prof_begin(ctx, s, capturing, 0, &slot));
     const int grid = mode == PAIR_EVAL ? b.grid : pair_grid(ctx, P, mode, b.sub);

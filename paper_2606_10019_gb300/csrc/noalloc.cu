@@ -118,6 +118,7 @@ __global__ void k_na_setup(NaSetup a, unsigned char *base) {
     P->w1 = a.n_items;
     P->c0 = 0;
     P->c1 = (a.n_items + FIN_CHUNK - 1) / FIN_CHUNK;
+    P->done = 0;
     P->lo = 1;   // r from double-float positions (no eigenvalue bounds here)
     const int le = words[2];
     const float lam_src = __int_as_float(le >= 0 ? le : le ^ 0x7fffffff);
@@ -251,7 +252,8 @@ extern "C" gcvo_status gcvo_eval_static(const gcvo_grid *target, const float *sr
     int grid = std::max(1, std::min(n_items, std::max(1, per_sm) * sm));
     GCVO_CUDA(launch_pair(pa, PAIR_EVAL, iso, fd, NA_SUB, grid, s));
     fa.mode = FIN_EVAL;
-    fa.reduce_blocks = std::max(1, sm) * 8;
+    fa.reduce_blocks = std::min((n_items + FIN_CHUNK - 1) / FIN_CHUNK, std::max(1, sm) * 8);
+    fa.work = words;
     GCVO_CUDA(launch_finalize(fa, s));
     EvalOut e;
     unsigned st = 0;

@@ -1,12 +1,12 @@
 // The FP64 side of the per-iteration hot path of Algorithm 1, the transform
 // of the source points, and the source packing done once per call:
-//   k_fin_reduce -- FP64 sums of the item partials over chunks of FIN_CHUNK
+//   k_finalize  -- FP64 sums of the item partials over chunks of FIN_CHUNK
 //                  work items of one problem (all SMs, whatever the batch);
-//   k_fin_step  -- one warp per problem: the sum of its chunk rows, change
-//                  of frame, connection term (Eq. 12), the 6x6 solve of
-//                  Eq. (13) (or the G-CVO-E Newton step with the exact
-//                  Hessian) and the update T <- T exp(xi); the split pose
-//                  constants the transform reads.
+//                  the block that adds a problem's last chunk takes its
+//                  step: change of frame, connection term (Eq. 12), the
+//                  6x6 solve of Eq. (13) (or the G-CVO-E Newton step with
+//                  the exact Hessian), the update T <- T exp(xi) and the
+//                  split pose constants the transform reads;
 //   k_transform -- every source point of an active problem moved into the
 //                  target grid's frame at the current pose (Algorithm 1,
 //                  T^-1 z): p = R^T (z - t) - o in double-float arithmetic,
@@ -24,237 +24,150 @@ namespace gcvo {
 namespace {
 
 // ---------------------------------------------------------------------------
-// FP64 finalize: the device-side math of the per-problem step (k_fin_step).
+// FP64 finalize: the per-problem step, on one warp.
+//
+// The step is a few hundred FP64 operations with little to share between
+// problems, on a GPU that finishes 2 FP64 results per SM and cycle: a warp
+// instruction costs the same for one lane as for 32, so what counts is the
+// number of FP64 instructions in line.  One lane working through it alone
+// took about 1300 of them, 43 us per iteration.  Here the lanes hold the
+// entries of the matrices (a 6 x 6 entry, or a column in the solve), which
+// leaves about 200; the exponential's coefficients are short series, one
+// lane each.
 // ---------------------------------------------------------------------------
 
-__device__ void hat3d(const double w[3], double W[9]) {
-    W[0] = 0;     W[1] = -w[2]; W[2] = w[1];
-    W[3] = w[2];  W[4] = 0;     W[5] = -w[0];
-    W[6] = -w[1]; W[7] = w[0];  W[8] = 0;
+// Entry (r, c) of w^.
+__device__ __forceinline__ double hat_at(const double w[3], int r, int c) {
+    const double v = r + c == 1 ? w[2] : r + c == 2 ? w[1] : w[0];
+    return r == c ? 0.0 : ((c - r + 3) % 3 == 1 ? -v : v);
 }
 
-// exp of a twist (omega, v): Rodrigues rotation and V-matrix translation,
-// with series coefficients for small angles.
-__device__ void exp_twist(const double xi[6], double Rout[9], double tout[3]) {
-    double th2 = xi[0] * xi[0] + xi[1] * xi[1] + xi[2] * xi[2];
-    double th = sqrt(th2);
-    double A, B, C;
-    if (th < 1e-4) {
-        A = 1.0 - th2 / 6.0 + th2 * th2 / 120.0;
-        B = 0.5 - th2 / 24.0 + th2 * th2 / 720.0;
-        C = 1.0 / 6.0 - th2 / 120.0 + th2 * th2 / 5040.0;
-    } else {
-        double s, c;
-        sincos(th, &s, &c);
-        A = s / th;
-        B = (1.0 - c) / th2;
-        C = (th - s) / (th2 * th);
+// Entry (r, c) of Gamma (Eq. 12), [[-1/2 g_w^, 0], [-g_v^, 0]].
+__device__ __forceinline__ double gamma_at(const double g[6], int r, int c) {
+    if (c > 2) return 0.0;
+    return r < 3 ? -0.5 * hat_at(g, r, c) : -hat_at(g + 3, r - 3, c);
+}
+
+// out = B^T N B for B = [[I, 0], [-o^, I]] (6 x 6, row-major in shared
+// memory; tmp is scratch): the change from the grid-origin frame to the
+// caller's, with p = p_o + o and J = J_o B.  sym: N is symmetric, and the
+// result is made so exactly.
+__device__ void change_frame(const double *N, const double o[3], double *tmp, double *out, bool sym, int lane) {
+    for (int e = lane; e < 36; e += 32) {
+        const int r = e / 6, c = e % 6;
+        double v = N[e];
+        if (c < 3)
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                if (k != c) v -= N[6 * r + 3 + k] * hat_at(o, k, c);
+        tmp[e] = v;
     }
-    double W[9], W2[9];
-    hat3d(xi, W);
-    for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c) W2[3 * r + c] = W[3 * r] * W[c] + W[3 * r + 1] * W[3 + c] + W[3 * r + 2] * W[6 + c];
-    for (int k = 0; k < 9; ++k) {
-        double I = (k % 4 == 0) ? 1.0 : 0.0;
-        Rout[k] = I + A * W[k] + B * W2[k];
-    }
-    for (int r = 0; r < 3; ++r) {
-        double s = 0;
-        for (int c = 0; c < 3; ++c) {
-            double I = r == c ? 1.0 : 0.0;
-            s += (I + B * W[3 * r + c] + C * W2[3 * r + c]) * xi[3 + c];
+    __syncwarp();
+    for (int e = lane; e < 36; e += 32) {
+        int r = e / 6, c = e % 6;
+        if (sym && r > c) {
+            const int t = r;
+            r = c;
+            c = t;
         }
-        tout[r] = s;
+        double v = tmp[6 * r + c];
+        if (r < 3)
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                if (k != r) v += hat_at(o, r, k) * tmp[6 * (3 + k) + c];
+        out[e] = v;
     }
+    __syncwarp();
 }
 
-// Solve A x = b (6x6, row-major) by LU with partial pivoting.  Returns 0,
-// or 1 when a pivot is exactly zero.
-__device__ int solve_lu6(const double Ain[36], const double b[6], double x[6]) {
-    double A[42];
-    for (int r = 0; r < 6; ++r) {
-        for (int c = 0; c < 6; ++c) A[7 * r + c] = Ain[6 * r + c];
-        A[7 * r + 6] = b[r];
-    }
-    for (int c = 0; c < 6; ++c) {
-        int piv = c;
-        for (int r = c + 1; r < 6; ++r)
-            if (fabs(A[7 * r + c]) > fabs(A[7 * piv + c])) piv = r;
-        if (A[7 * piv + c] == 0.0) return 1;
-        if (piv != c)
-            for (int k = 0; k < 7; ++k) {
-                double tmp = A[7 * c + k];
-                A[7 * c + k] = A[7 * piv + k];
-                A[7 * piv + k] = tmp;
+// Solves A x = b (A 6 x 6 row-major, b: shared memory) by Gauss-Jordan
+// elimination with partial pivoting: lane j < 6 holds column j, lane 6 the
+// right-hand side; x[k] ends in shared memory.  Returns 0, or 1 when a pivot
+// is exactly zero (the same in every lane).
+__device__ int solve6(const double *A, const double *b, double *x, int lane) {
+    const unsigned FULL = 0xffffffffu;
+    double col[6];
+#pragma unroll
+    for (int r = 0; r < 6; ++r) col[r] = lane < 6 ? A[6 * r + lane] : lane == 6 ? b[r] : 0.0;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        // the row of column k's largest entry, by its high word
+        int piv = k, top = __double2hiint(col[k]) & 0x7fffffff;
+#pragma unroll
+        for (int r = k + 1; r < 6; ++r) {
+            const int m = __double2hiint(col[r]) & 0x7fffffff;
+            if (m > top) {
+                top = m;
+                piv = r;
             }
-        for (int r = c + 1; r < 6; ++r) {
-            double f = A[7 * r + c] / A[7 * c + c];
-            for (int k = c; k < 7; ++k) A[7 * r + k] -= f * A[7 * c + k];
         }
+        piv = __shfl_sync(FULL, piv, k);
+#pragma unroll
+        for (int r = k + 1; r < 6; ++r)
+            if (r == piv) {
+                const double t = col[k];
+                col[k] = col[r];
+                col[r] = t;
+            }
+        const double p = __shfl_sync(FULL, col[k], k);
+        if (p == 0.0) return 1;
+        double f[6];
+#pragma unroll
+        for (int r = 0; r < 6; ++r) f[r] = __shfl_sync(FULL, col[r], k);
+        col[k] *= 1.0 / p;
+#pragma unroll
+        for (int r = 0; r < 6; ++r)
+            if (r != k) col[r] -= f[r] * col[k];
     }
-    for (int r = 5; r >= 0; --r) {
-        double sm = A[7 * r + 6];
-        for (int k = r + 1; k < 6; ++k) sm -= A[7 * r + k] * x[k];
-        x[r] = sm / A[7 * r + r];
-    }
+    if (lane == 6)
+#pragma unroll
+        for (int r = 0; r < 6; ++r) x[r] = col[r];
+    __syncwarp();
     return 0;
 }
 
-// Gamma of Eq. (12) as a 6x6 row-major matrix: [[-1/2 g_w^, 0], [-g_v^, 0]].
-__device__ void gamma6(const double g[6], double Gam[36]) {
-#pragma unroll
-    for (int k = 0; k < 36; ++k) Gam[k] = 0.0;
-    Gam[1] = 0.5 * g[2];   Gam[2] = -0.5 * g[1];
-    Gam[6] = -0.5 * g[2];  Gam[8] = 0.5 * g[0];
-    Gam[12] = 0.5 * g[1];  Gam[13] = -0.5 * g[0];
-    Gam[19] = g[5];  Gam[20] = -g[4];
-    Gam[24] = -g[5]; Gam[26] = g[3];
-    Gam[30] = g[4];  Gam[31] = -g[3];
-}
+// 1 / m! for m = 0 .. 23.
+__constant__ double INV_FACT[24] = {1.0,
+                                    1.0,
+                                    1.0 / 2,
+                                    1.0 / 6,
+                                    1.0 / 24,
+                                    1.0 / 120,
+                                    1.0 / 720,
+                                    1.0 / 5040,
+                                    1.0 / 40320,
+                                    1.0 / 362880,
+                                    1.0 / 3628800,
+                                    1.0 / 39916800,
+                                    1.0 / 479001600,
+                                    1.0 / 6227020800.0,
+                                    1.0 / 87178291200.0,
+                                    1.0 / 1307674368000.0,
+                                    1.0 / 20922789888000.0,
+                                    1.0 / 355687428096000.0,
+                                    1.0 / 6402373705728000.0,
+                                    1.0 / 121645100408832000.0,
+                                    1.0 / 2432902008176640000.0,
+                                    1.0 / 51090942171709440000.0,
+                                    1.0 / 1124000727777607680000.0,
+                                    1.0 / 25852016738884976640000.0};
 
-// Solve (M - Gamma) xi = g (Eq. 13).  M is symmetric positive definite for a
-// problem with overlap; Gamma (Eq. 12) has non-zero entries only in its first
-// three columns, Gamma = Gc E^T with Gc = [-1/2 g_omega^; -g_v^] (6x3) and
-// E = [I3; 0].  With the Cholesky factor of M, y = M^-1 g and Z = M^-1 Gc,
-// the Sherman-Morrison-Woodbury identity gives
-//   xi = y + Z (I3 - E^T Z)^-1 E^T y.
-// Falls back to partial-pivot LU of M - Gamma when M is not positive
-// definite.  Returns 0, or 1 when both fail.
-__device__ int solve_gn(const double M[36], const double g[6], double xi[6]) {
-    double Gc[18];
+// The coefficients of exp at the squared angle x = theta^2: lane 0 gets
+// sin(theta) / theta, lane 1 (1 - cos(theta)) / theta^2, lane 2 (theta -
+// sin(theta)) / theta^3: sum_k (-x)^k / (2 k + 1 + lane)!.  Up to a radian
+// eleven terms leave less than 1e-19; larger steps take the closed forms.
+__device__ double exp_coefficient(double x, int lane) {
+    if (x <= 1.0) {
+        const int m = 1 + min(lane, 2);
+        double s = INV_FACT[20 + m];
 #pragma unroll
-    for (int r = 0; r < 18; ++r) Gc[r] = 0.0;
-    // Gc = [-1/2 g_omega^ ; -g_v^]
-    Gc[1] = 0.5 * g[2];  Gc[2] = -0.5 * g[1];
-    Gc[3] = -0.5 * g[2]; Gc[5] = 0.5 * g[0];
-    Gc[6] = 0.5 * g[1];  Gc[7] = -0.5 * g[0];
-    Gc[10] = g[5];  Gc[11] = -g[4];
-    Gc[12] = -g[5]; Gc[14] = g[3];
-    Gc[15] = g[4];  Gc[16] = -g[3];
-    // Cholesky M = L L^T (inverse diagonal kept)
-    double L[36], id[6];
-    bool spd = true;
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-#pragma unroll
-        for (int j = 0; j <= i; ++j) {
-            double sm = M[6 * i + j];
-#pragma unroll
-            for (int k = 0; k < j; ++k) sm -= L[6 * i + k] * L[6 * j + k];
-            if (i == j) {
-                spd = spd && (sm > 0.0);
-                double r = sqrt(fmax(sm, 1e-300));
-                L[6 * i + i] = r;
-                id[i] = 1.0 / r;
-            } else {
-                L[6 * i + j] = sm * id[j];
-            }
-        }
+        for (int k = 9; k >= 0; --k) s = INV_FACT[2 * k + m] - x * s;
+        return s;
     }
-    if (spd) {
-        // X = M^-1 [g, Gc] (6 x 4)
-        double X[24];
-#pragma unroll
-        for (int r = 0; r < 6; ++r) {
-            X[4 * r] = g[r];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) X[4 * r + 1 + c] = Gc[3 * r + c];
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-#pragma unroll
-            for (int i = 0; i < 6; ++i) {
-                double sm = X[4 * i + c];
-#pragma unroll
-                for (int k = 0; k < i; ++k) sm -= L[6 * i + k] * X[4 * k + c];
-                X[4 * i + c] = sm * id[i];
-            }
-#pragma unroll
-            for (int i = 5; i >= 0; --i) {
-                double sm = X[4 * i + c];
-#pragma unroll
-                for (int k = i + 1; k < 6; ++k) sm -= L[6 * k + i] * X[4 * k + c];
-                X[4 * i + c] = sm * id[i];
-            }
-        }
-        // K = I3 - E^T Z, w = K^-1 E^T y (Cramer), xi = y + Z w
-        double K[9];
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) K[3 * r + c] = (r == c ? 1.0 : 0.0) - X[4 * r + 1 + c];
-        double c00 = K[4] * K[8] - K[5] * K[7], c01 = K[5] * K[6] - K[3] * K[8], c02 = K[3] * K[7] - K[4] * K[6];
-        double detK = K[0] * c00 + K[1] * c01 + K[2] * c02;
-        double kn = 0.0;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) kn = fmax(kn, fabs(K[k]));
-        if (fabs(detK) > 1e-12 * kn * kn * kn) {
-            double idet = 1.0 / detK;
-            double y0 = X[0], y1 = X[4], y2 = X[8];
-            // inverse of K by its adjugate
-            double w0 = (c00 * y0 + (K[2] * K[7] - K[1] * K[8]) * y1 + (K[1] * K[5] - K[2] * K[4]) * y2) * idet;
-            double w1 = (c01 * y0 + (K[0] * K[8] - K[2] * K[6]) * y1 + (K[2] * K[3] - K[0] * K[5]) * y2) * idet;
-            double w2 = (c02 * y0 + (K[1] * K[6] - K[0] * K[7]) * y1 + (K[0] * K[4] - K[1] * K[3]) * y2) * idet;
-#pragma unroll
-            for (int r = 0; r < 6; ++r) xi[r] = X[4 * r] + X[4 * r + 1] * w0 + X[4 * r + 2] * w1 + X[4 * r + 3] * w2;
-            return 0;
-        }
-    }
-    // LU with partial pivoting of M - Gamma (Gamma = Gc in the first 3 columns)
-    double A[36];
-    for (int r = 0; r < 6; ++r)
-        for (int c = 0; c < 6; ++c) A[6 * r + c] = M[6 * r + c] - (c < 3 ? Gc[3 * r + c] : 0.0);
-    return solve_lu6(A, g, xi);
-}
-
-// G-CVO-E: D(g) in the caller's frame from the grid-frame sums of the exact
-// pass.  Per source point, with y = Sigma_ij^-1 r summed over its targets,
-// S_y = sum w y, S_B = sum w (y u^T + K) and P = p^ (tile.cu, pair_exact),
-// the pass leaves C = sum_points (-S_y^ P + P S_B) in tot[28..36] and
-// sum_points S_B in tot[37..45], row-major.  Qm is B^T (Q - M)_o B, already
-// moved by the code that moves M; the rest is N_o = [[C, S_y^], [S_B, 0]]
-// with S_y summed over all points = -g_v, and D = Qm - B^T N_o B for
-// B = [[I, 0], [-o^, I]].
-__device__ void exact_derivative(const double *tot, const double Qm[36], const double o[3], double D[36]) {
-    double N[36];
-#pragma unroll
-    for (int k = 0; k < 36; ++k) N[k] = 0.0;
-    const double s0 = -tot[4], s1 = -tot[5], s2 = -tot[6];   // S_y
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            N[6 * r + c] = tot[28 + 3 * r + c];
-            N[6 * (r + 3) + c] = tot[37 + 3 * r + c];
-        }
-    N[4] = -s2;  N[5] = s1;
-    N[9] = s2;   N[11] = -s0;
-    N[15] = -s1; N[16] = s0;
-    double O[9];
-    hat3d(o, O);
-    // X = N B: columns 0..2 get -N[:, 3:6] o^
-    double X[36];
-#pragma unroll
-    for (int r = 0; r < 6; ++r)
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            double v = N[6 * r + c];
-            if (c < 3)
-#pragma unroll
-                for (int k = 0; k < 3; ++k) v -= N[6 * r + 3 + k] * O[3 * k + c];
-            X[6 * r + c] = v;
-        }
-    // B^T X: rows 0..2 get +o^ X[3:6, :]  (B^T = [[I, o^], [0, I]])
-#pragma unroll
-    for (int r = 0; r < 6; ++r)
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            double v = X[6 * r + c];
-            if (r < 3)
-#pragma unroll
-                for (int k = 0; k < 3; ++k) v += O[3 * r + k] * X[6 * (3 + k) + c];
-            D[6 * r + c] = Qm[6 * r + c] - v;
-        }
+    const double th = sqrt(x);
+    double sn, cs;
+    sincos(th, &sn, &cs);
+    return lane == 0 ? sn / th : lane == 1 ? (1.0 - cs) / x : (th - sn) / (x * th);
 }
 
 // Smallest positive real root of the cubic d3 t^3 + d2 t^2 + d1 t + d0
@@ -307,266 +220,242 @@ __device__ double smallest_pos_root(double d3, double d2, double d1, double d0) 
     return best;
 }
 
-__device__ inline void set_inactive(ProbDev *P, int st, int *n_active) {
+constexpr int FIN_THREADS = 256;   // 8 warps: item g of a chunk goes to warp g % 8
+
+// Shared memory of one block of k_finalize.
+struct FinShared {
+    double red[FIN_THREADS / 32][64];
+    long long cred[FIN_THREADS / 32][4];
+    double tot[64];
+    long long ctot[4];
+    double N[36], tmp[36], M[36], D[36], A[36];
+    double g[6], xi[6], T[12], dT[12];
+    int last;
+};
+
+// The split constants of the transform at the pose T (shared memory): R as
+// float head and tail, and c = R^T t + o (o the grid origin, in memory)
+// likewise.
+__device__ void refresh_pose(const double *T, const double *o, ProbDev *P, int lane) {
+    if (lane >= 12) return;
+    double v;
+    if (lane < 9) {
+        v = T[lane];
+    } else {
+        const int k = lane - 9;
+        v = T[k] * T[9] + T[3 + k] * T[10] + T[6 + k] * T[11] + o[k];
+    }
+    const float h = (float)v, l = (float)(v - (double)h);
+    if (lane < 9) {
+        P->Rh[lane] = h;
+        P->Rl[lane] = l;
+    } else {
+        P->ch[lane - 9] = h;
+        P->cl[lane - 9] = l;
+    }
+}
+
+__device__ __forceinline__ void set_inactive(ProbDev *P, int st, int *n_active) {
     P->status = st;
     atomicSub(n_active, 1);
 }
 
-__device__ inline void apply_step(ProbDev *P, const double xi[6], gcvo_iter_log *lg, const FinalizeArgs &a,
-                                  int it) {
+// T <- T exp(xi) with xi and T in S; the log row, the stop test, and the
+// transform constants of a problem that stays active.
+__device__ void apply_step(const FinalizeArgs &a, ProbDev *P, FinShared &S, const double *o, gcvo_iter_log *lg, int it,
+                           int lane) {
+    const unsigned FULL = 0xffffffffu;
+    const double *w = S.xi, *v = S.xi + 3;
+    const double x = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
+    const double co = exp_coefficient(x, lane);
+    const double A = __shfl_sync(FULL, co, 0), B = __shfl_sync(FULL, co, 1), C = __shfl_sync(FULL, co, 2);
+    // w^ w^ = w w^T - x I
+    if (lane < 9) {
+        const int r = lane / 3, c = lane % 3;
+        const double W2 = w[r] * w[c] - (r == c ? x : 0.0);
+        S.dT[lane] = (r == c ? 1.0 : 0.0) + A * hat_at(w, r, c) + B * W2;
+    } else if (lane < 12) {
+        const int r = lane - 9, r1 = (r + 1) % 3, r2 = (r + 2) % 3;
+        const double wv = w[0] * v[0] + w[1] * v[1] + w[2] * v[2];
+        S.dT[lane] = v[r] + B * (w[r1] * v[r2] - w[r2] * v[r1]) + C * (w[r] * wv - x * v[r]);
+    }
+    __syncwarp();
+    double tn = 0.0;
+    if (lane < 9) {
+        const int r = lane / 3, c = lane % 3;
+        tn = S.T[3 * r] * S.dT[c] + S.T[3 * r + 1] * S.dT[3 + c] + S.T[3 * r + 2] * S.dT[6 + c];
+    } else if (lane < 12) {
+        const int r = lane - 9;
+        tn = S.T[3 * r] * S.dT[9] + S.T[3 * r + 1] * S.dT[10] + S.T[3 * r + 2] * S.dT[11] + S.T[lane];
+    }
+    __syncwarp();
+    if (lane < 12) {
+        S.T[lane] = tn;
+        P->T[lane] = tn;
+    }
+    __syncwarp();
+    refresh_pose(S.T, o, P, lane);
     double l1 = 0.0;
 #pragma unroll
-    for (int k = 0; k < 6; ++k) l1 += fabs(xi[k]);
-    double dR[9], dt[3];
-    exp_twist(xi, dR, dt);
-    double Rn[9], tn[3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-            Rn[3 * r + c] = P->T[3 * r] * dR[c] + P->T[3 * r + 1] * dR[3 + c] + P->T[3 * r + 2] * dR[6 + c];
-        tn[r] = P->T[3 * r] * dt[0] + P->T[3 * r + 1] * dt[1] + P->T[3 * r + 2] * dt[2] + P->T[9 + r];
+    for (int k = 0; k < 6; ++k) l1 += fabs(S.xi[k]);
+    if (lg && lane < 6) lg->xi[lane] = S.xi[lane];
+    if (lane == 0) {
+        if (lg) lg->xi_l1 = l1;
+        P->iter = it + 1;
+        if (!(l1 == l1)) set_inactive(P, -(int)GCVO_ERR_NONFINITE, a.n_active);
+        else if (l1 < a.eps_tol) set_inactive(P, 1, a.n_active);
+        else if (it + 1 >= a.k_max) set_inactive(P, 2, a.n_active);
     }
-#pragma unroll
-    for (int k = 0; k < 9; ++k) P->T[k] = Rn[k];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) P->T[9 + k] = tn[k];
-    if (lg) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) lg->xi[k] = xi[k];
-        lg->xi_l1 = l1;
-    }
-    P->iter = it + 1;
-    if (!(l1 == l1)) set_inactive(P, -(int)GCVO_ERR_NONFINITE, a.n_active);
-    else if (l1 < a.eps_tol) set_inactive(P, 1, a.n_active);
-    else if (it + 1 >= a.k_max) set_inactive(P, 2, a.n_active);
 }
 
-// The per-problem FP64 step (one thread): returns 1 when the pose changed
-// and the problem stays active, so the transform constants must be refreshed.
-__device__ int finalize_thread0(const FinalizeArgs &a, int prob, ProbDev *P, const double *tot,
-                                const long long *ctot) {
+// The per-problem step of one warp from the slot sums S.tot and S.ctot.
+__device__ void fin_step(const FinalizeArgs &a, int prob, ProbDev *P, FinShared &S, int lane) {
+    const unsigned FULL = 0xffffffffu;
     const GridDev *G = a.grids + prob;
-    const double o0 = G->origin[0], o1 = G->origin[1], o2 = G->origin[2];
+    const double o[3] = {G->origin[0], G->origin[1], G->origin[2]};
     const int it = P->iter;
     gcvo_iter_log *lg = a.logs ? a.logs + (size_t)prob * a.k_max + it : nullptr;
+    const double *tot = S.tot;
+    if (lane < 12) S.T[lane] = P->T[lane];
+    __syncwarp();
 
     if (a.mode == FIN_LINESEARCH) {
         // G(t) ~ sum_k c_k t^k along xi = g (Eq. 9).  c_1 = dG/dt(0) = <g, g>
         // exactly; it is taken from the FP64 gradient rather than the FP32
         // pair sums, which cancel towards zero near the optimum.
-        double c1 = 0.0;
+        if (lane == 0) {
+            double c1 = 0.0;
 #pragma unroll
-        for (int k = 0; k < 6; ++k) c1 += P->dir[k] * P->dir[k];
-        double c2 = tot[2], c3 = tot[3], c4 = tot[4];
-        double ts = smallest_pos_root(4.0 * c4, 3.0 * c3, 2.0 * c2, c1);
-        double mu = ts > a.mu0 ? ts : a.mu0;
-        double xi[6];
+            for (int k = 0; k < 6; ++k) c1 += P->dir[k] * P->dir[k];
+            const double ts = smallest_pos_root(4.0 * tot[4], 3.0 * tot[3], 2.0 * tot[2], c1);
+            const double mu = ts > a.mu0 ? ts : a.mu0;
 #pragma unroll
-        for (int k = 0; k < 6; ++k) xi[k] = mu * P->dir[k];
-        apply_step(P, xi, lg, a, it);
-        return P->status == 0;
+            for (int k = 0; k < 6; ++k) S.xi[k] = mu * P->dir[k];
+        }
+        __syncwarp();
+        apply_step(a, P, S, G->origin, lg, it, lane);
+        return;
     }
 
-    // f, g, M in the grid-origin frame (p relative to o), moved to the
-    // caller's frame: with p = p_o + o, J = J_o B for B = [[I, 0], [-o^, I]],
-    // so g = B^T g_o and M = B^T M_o B.  In 3x3 blocks (A, Bm, C of M_o and
-    // O = o^, X = Bm O): M_ww = A - X - X^T - O C O, M_wv = Bm + O C, M_vv = C,
-    // g_w = g_ow + o x g_ov, g_v = g_ov.
-    double f = tot[0];
-    double A[9], Bm[9], C[9];
-    {
-        int q = 7;
-        double U[36];
-#pragma unroll
-        for (int r = 0; r < 6; ++r)
-#pragma unroll
-            for (int c = r; c < 6; ++c) {
-                U[6 * r + c] = tot[q];
-                U[6 * c + r] = tot[q];
-                ++q;
-            }
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                A[3 * r + c] = U[6 * r + c];
-                Bm[3 * r + c] = U[6 * r + 3 + c];
-                C[3 * r + c] = U[6 * (r + 3) + 3 + c];
-            }
+    // f, g and M (G-CVO-E: Q - M) in the grid-origin frame (p relative to
+    // o), moved to the caller's: g = B^T g_o, M = B^T M_o B (change_frame)
+    const double f = tot[0];
+    for (int e = lane; e < 36; e += 32) {
+        const int r = min(e / 6, e % 6), c = max(e / 6, e % 6);
+        S.N[e] = tot[7 + r * 6 - r * (r - 1) / 2 + (c - r)];
     }
-    double X[9], CO[9], OCO[9], OC[9];
+    if (lane < 6) {
+        double v = tot[1 + lane];
+        if (lane < 3)
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        X[3 * r + 0] = Bm[3 * r + 1] * o2 - Bm[3 * r + 2] * o1;
-        X[3 * r + 1] = -Bm[3 * r + 0] * o2 + Bm[3 * r + 2] * o0;
-        X[3 * r + 2] = Bm[3 * r + 0] * o1 - Bm[3 * r + 1] * o0;
-        CO[3 * r + 0] = C[3 * r + 1] * o2 - C[3 * r + 2] * o1;
-        CO[3 * r + 1] = -C[3 * r + 0] * o2 + C[3 * r + 2] * o0;
-        CO[3 * r + 2] = C[3 * r + 0] * o1 - C[3 * r + 1] * o0;
+            for (int k = 0; k < 3; ++k)
+                if (k != lane) v += hat_at(o, lane, k) * tot[4 + k];
+        S.g[lane] = v;
     }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        OCO[c] = -o2 * CO[3 + c] + o1 * CO[6 + c];
-        OCO[3 + c] = o2 * CO[c] - o0 * CO[6 + c];
-        OCO[6 + c] = -o1 * CO[c] + o0 * CO[3 + c];
-        OC[c] = -o2 * C[3 + c] + o1 * C[6 + c];
-        OC[3 + c] = o2 * C[c] - o0 * C[6 + c];
-        OC[6 + c] = -o1 * C[c] + o0 * C[3 + c];
-    }
-    double M[36];
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            M[6 * r + c] = A[3 * r + c] - X[3 * r + c] - X[3 * c + r] - OCO[3 * r + c];
-            double wv = Bm[3 * r + c] + OC[3 * r + c];
-            M[6 * r + 3 + c] = wv;
-            M[6 * (c + 3) + r] = wv;
-            M[6 * (r + 3) + 3 + c] = C[3 * r + c];
-        }
-    double g[6];
-    {
-        double gw0 = tot[1], gw1 = tot[2], gw2 = tot[3], gv0 = tot[4], gv1 = tot[5], gv2 = tot[6];
-        g[0] = gw0 + (o1 * gv2 - o2 * gv1);
-        g[1] = gw1 + (o2 * gv0 - o0 * gv2);
-        g[2] = gw2 + (o0 * gv1 - o1 * gv0);
-        g[3] = gv0;
-        g[4] = gv1;
-        g[5] = gv2;
-    }
-    bool finite = isfinite(f);
-#pragma unroll
-    for (int k = 0; k < 6; ++k) finite = finite && isfinite(g[k]);
-#pragma unroll
-    for (int k = 0; k < 36; ++k) finite = finite && isfinite(M[k]);
-    // G-CVO-E: M above holds B^T (Q - M)_o B; D(g) replaces -M
+    __syncwarp();
+    change_frame(S.N, o, S.tmp, S.M, true, lane);
     const bool exact = a.mode == FIN_EXACT || a.mode == FIN_EXACT_EVAL;
-    double D[36];
     if (exact) {
-        const double o[3] = {o0, o1, o2};
-        exact_derivative(tot, M, o, D);
-#pragma unroll
-        for (int k = 0; k < 36; ++k) finite = finite && isfinite(D[k]);
+        // D(g) in the caller's frame from the grid-frame sums of the exact
+        // pass.  Per source point, with y = Sigma_ij^-1 r summed over its
+        // targets, S_y = sum w y, S_B = sum w (y u^T + K) and P = p^
+        // (tile.cu, pair_exact), the pass leaves C = sum_points (-S_y^ P + P
+        // S_B) in tot[28..36] and sum_points S_B in tot[37..45], row-major.
+        // M holds B^T (Q - M)_o B; the rest is N_o = [[C, S_y^], [S_B, 0]] with
+        // S_y summed over all points = -g_v, and D = M - B^T N_o B.
+        const double sy[3] = {-tot[4], -tot[5], -tot[6]};
+        for (int e = lane; e < 36; e += 32) {
+            const int r = e / 6, c = e % 6;
+            S.N[e] = c < 3 ? (r < 3 ? tot[28 + 3 * r + c] : tot[37 + 3 * (r - 3) + c]) : r < 3 ? hat_at(sy, r, c - 3) : 0.0;
+        }
+        __syncwarp();
+        change_frame(S.N, o, S.tmp, S.D, false, lane);
+        for (int e = lane; e < 36; e += 32) S.D[e] = S.M[e] - S.D[e];
+        __syncwarp();
     }
+    bool finite = isfinite(f) && (lane >= 6 || isfinite(S.g[lane]));
+    for (int e = lane; e < 36; e += 32) finite = finite && isfinite(S.M[e]) && (!exact || isfinite(S.D[e]));
+    finite = __all_sync(FULL, finite);
 
     if (lg) {
-        lg->f = f;
-#pragma unroll
-        for (int k = 0; k < 6; ++k) lg->g[k] = g[k];
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) lg->T[4 * r + c] = P->T[3 * r + c];
-            lg->T[4 * r + 3] = P->T[9 + r];
+        if (lane < 6) lg->g[lane] = S.g[lane];
+        if (lane < 16) lg->T[lane] = lane < 12 ? (lane % 4 < 3 ? S.T[3 * (lane / 4) + lane % 4] : S.T[9 + lane / 4]) : lane == 15 ? 1.0 : 0.0;
+        if (lane == 0) {
+            lg->f = f;
+            lg->n_pairs = S.ctot[0];
+            lg->n_kept = S.ctot[1];
         }
-        lg->T[12] = lg->T[13] = lg->T[14] = 0.0;
-        lg->T[15] = 1.0;
-        lg->n_pairs = ctot[0];
-        lg->n_kept = ctot[1];
     }
-
     if (a.mode == FIN_EVAL || a.mode == FIN_EXACT_EVAL) {
         // H_GN = -M + Gamma (Eq. 12); G-CVO-E: H_E = D(g) + Gamma, M <- D(g)
         EvalOut *e = a.evalout + prob;
-        e->f = f;
-#pragma unroll
-        for (int k = 0; k < 6; ++k) e->g[k] = g[k];
-        double Gam[36];
-        gamma6(g, Gam);
-#pragma unroll
-        for (int k = 0; k < 36; ++k) {
-            e->M[k] = exact ? D[k] : M[k];
-            e->H[k] = (exact ? D[k] : -M[k]) + Gam[k];
+        if (lane < 6) e->g[lane] = S.g[lane];
+        for (int k = lane; k < 36; k += 32) {
+            const double m = exact ? S.D[k] : S.M[k];
+            e->M[k] = m;
+            e->H[k] = (exact ? m : -m) + gamma_at(S.g, k / 6, k % 6);
         }
-        e->n_pairs = ctot[0];
-        e->n_kept = ctot[1];
-        e->n_cand = ctot[2];
-        return 0;
+        if (lane == 0) {
+            e->f = f;
+            e->n_pairs = S.ctot[0];
+            e->n_kept = S.ctot[1];
+            e->n_cand = S.ctot[2];
+        }
+        return;
     }
     if (!finite) {
-        set_inactive(P, -(int)GCVO_ERR_NONFINITE, a.n_active);
-        return 0;
+        if (lane == 0) set_inactive(P, -(int)GCVO_ERR_NONFINITE, a.n_active);
+        return;
     }
-    if (ctot[1] == 0 || !(f > 0.0)) {
-        set_inactive(P, -(int)GCVO_ERR_NO_OVERLAP, a.n_active);
-        return 0;
+    if (S.ctot[1] == 0 || !(f > 0.0)) {
+        if (lane == 0) set_inactive(P, -(int)GCVO_ERR_NO_OVERLAP, a.n_active);
+        return;
     }
     if (a.mode == FIN_GRAD) {
         // G-CVO-1: the line search runs along xi = g (Eq. 9); in the
         // grid-origin frame that direction has v' = omega x o + v.
+        if (lane < 6) {
+            P->dir[lane] = S.g[lane];
+            double d = S.g[lane];
+            if (lane > 2)
 #pragma unroll
-        for (int k = 0; k < 6; ++k) P->dir[k] = g[k];
-        P->dir32[0] = (float)g[0];
-        P->dir32[1] = (float)g[1];
-        P->dir32[2] = (float)g[2];
-        P->dir32[3] = (float)(g[1] * o2 - g[2] * o1 + g[3]);
-        P->dir32[4] = (float)(g[2] * o0 - g[0] * o2 + g[4]);
-        P->dir32[5] = (float)(g[0] * o1 - g[1] * o0 + g[5]);
-        return 0;
-    }
-    double xi[6];
-    if (exact) {
-        // G-CVO-E: Newton step xi = -H_E^-1 g, H_E = D(g) + Gamma (Eq. 12)
-        double Gam[36], nH[36];
-        gamma6(g, Gam);
-#pragma unroll
-        for (int k = 0; k < 36; ++k) nH[k] = -(D[k] + Gam[k]);
-        if (solve_lu6(nH, g, xi) != 0) {
-            set_inactive(P, -(int)GCVO_ERR_SINGULAR, a.n_active);
-            return 0;
+                for (int k = 0; k < 3; ++k)
+                    if (k != lane - 3) d -= hat_at(o, lane - 3, k) * S.g[k];   // omega x o = -o x omega
+            P->dir32[lane] = (float)d;
         }
-        apply_step(P, xi, lg, a, it);
-        return P->status == 0;
+        return;
     }
-    // G-CVO-2 step, Eq. (13)
-    if (solve_gn(M, g, xi) != 0) {
-        set_inactive(P, -(int)GCVO_ERR_SINGULAR, a.n_active);
-        return 0;
+    // G-CVO-2 step (M - Gamma) xi = g, Eq. (13); G-CVO-E: Newton step xi =
+    // -H_E^-1 g, H_E = D(g) + Gamma (Eq. 12)
+    for (int e = lane; e < 36; e += 32) {
+        const double gm = gamma_at(S.g, e / 6, e % 6);
+        S.A[e] = exact ? -(S.D[e] + gm) : S.M[e] - gm;
     }
-    apply_step(P, xi, lg, a, it);
-    return P->status == 0;
+    __syncwarp();
+    if (solve6(S.A, S.g, S.xi, lane) != 0) {
+        if (lane == 0) set_inactive(P, -(int)GCVO_ERR_SINGULAR, a.n_active);
+        return;
+    }
+    apply_step(a, P, S, G->origin, lg, it, lane);
 }
-
-// The split constants of the transform at the pose P->T: R as float head
-// and tail, and c = R^T t + o (o the grid origin) likewise.
-__device__ void refresh_pose(const FinalizeArgs &a, int prob, ProbDev *P) {
-    const GridDev *G = a.grids + prob;
-    double c[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-        c[k] = P->T[k] * P->T[9] + P->T[3 + k] * P->T[10] + P->T[6 + k] * P->T[11] + G->origin[k];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const float h = (float)P->T[k];
-        P->Rh[k] = h;
-        P->Rl[k] = (float)(P->T[k] - (double)h);
-    }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const float h = (float)c[k];
-        P->ch[k] = h;
-        P->cl[k] = (float)(c[k] - (double)h);
-    }
-}
-
-constexpr int FIN_RED_THREADS = 256;   // 8 warps: item g goes to warp g % 8
-// problems per block of k_fin_step: one, so that problems spread over the
-// SMs and their serial FP64 steps do not share one SM's FP64 units
-constexpr int FIN_STEP_WARPS = 1;
 
 // The chunk rows: per chunk, per slot, a compensated FP32 sum of the (hi, lo)
 // partials over each warp's items (8 loads in flight per warp), the warps
 // added in FP64 in a fixed order; the pair counts likewise.  A persistent
 // grid walks the chunks; the problem of chunk c is the last one with c0 <= c.
-__global__ void __launch_bounds__(FIN_RED_THREADS) k_fin_reduce(FinalizeArgs a) {
-    __shared__ double red[FIN_RED_THREADS / 32][64];
-    __shared__ long long cred[FIN_RED_THREADS / 32][4];
+// The block that finishes a problem's last chunk adds its rows in chunk
+// order and takes the step.  As two launches, the step on one lane, they
+// were 22 + 46 us of the 85 us that an iteration took at 2,000 source points;
+// a registration of 22 iterations went from 1989 to 1132 us.
+__global__ void __launch_bounds__(FIN_THREADS) k_finalize(FinalizeArgs a) {
+    __shared__ FinShared S;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     // the G-CVO-E pass leaves slots 32..45 in a second partial row per item
     // (its slots 46..63 are never written, and their sums never read)
     const int rows = (a.mode == FIN_EXACT || a.mode == FIN_EXACT_EVAL) ? 2 : 1;
     const int nch = *a.n_chunks;
+    // the pair pass is done with its work counter: ready for the next one
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.work = 0;
     for (int c = blockIdx.x; c < nch; c += gridDim.x) {
         int lo = 0, hi = a.n_problems - 1;
         while (lo < hi) {
@@ -574,15 +463,18 @@ __global__ void __launch_bounds__(FIN_RED_THREADS) k_fin_reduce(FinalizeArgs a) 
             if (a.probs[mid].c0 <= c) lo = mid;
             else hi = mid - 1;
         }
-        const ProbDev *P = a.probs + lo;
-        if (P->status != 0) continue;   // the same for the whole block
-        const int i0 = P->w0 + (c - P->c0) * FIN_CHUNK, i1 = min(P->w1, i0 + FIN_CHUNK);
+        ProbDev *P = a.probs + lo;
+        // the same for the whole block: the status only changes in the step
+        // that follows the problem's last chunk
+        if (P->status != 0) continue;
+        const int c0 = P->c0, c1 = P->c1;
+        const int i0 = P->w0 + (c - c0) * FIN_CHUNK, i1 = min(P->w1, i0 + FIN_CHUNK);
         for (int row = 0; row < rows; ++row) {
             const float *src = row == 0 ? a.part : a.part2;
             float H = 0.f, Lo = 0.f;
             long long cacc = 0;
 #pragma unroll 8
-            for (int g = i0 + w; g < i1; g += FIN_RED_THREADS / 32) {
+            for (int g = i0 + w; g < i1; g += FIN_THREADS / 32) {
                 const float *p = src + (size_t)g * 64;
                 const float h = p[lane], l = p[32 + lane];
                 const float sm = H + h;
@@ -592,54 +484,70 @@ __global__ void __launch_bounds__(FIN_RED_THREADS) k_fin_reduce(FinalizeArgs a) 
                 Lo += l + err;
                 if (row == 0 && lane < 3) cacc += a.counts[(size_t)g * 4 + lane];
             }
-            red[w][32 * row + lane] = (double)H + (double)Lo;
-            if (row == 0 && lane < 4) cred[w][lane] = cacc;
+            S.red[w][32 * row + lane] = (double)H + (double)Lo;
+            if (row == 0 && lane < 4) S.cred[w][lane] = cacc;
         }
         __syncthreads();
         if (threadIdx.x < 32 * rows) {
             double sm = 0.0;
 #pragma unroll
-            for (int q = 0; q < FIN_RED_THREADS / 32; ++q) sm += red[q][threadIdx.x];
-            a.chunk[(size_t)c * 64 + threadIdx.x] = sm;
+            for (int q = 0; q < FIN_THREADS / 32; ++q) sm += S.red[q][threadIdx.x];
+            S.tot[threadIdx.x] = sm;
+            if (c1 - c0 > 1) a.chunk[(size_t)c * 64 + threadIdx.x] = sm;
         }
         if (threadIdx.x < 4) {
             long long cs = 0;
 #pragma unroll
-            for (int q = 0; q < FIN_RED_THREADS / 32; ++q) cs += cred[q][threadIdx.x];
-            a.chunk_cnt[(size_t)c * 4 + threadIdx.x] = cs;
+            for (int q = 0; q < FIN_THREADS / 32; ++q) cs += S.cred[q][threadIdx.x];
+            S.ctot[threadIdx.x] = cs;
+            if (c1 - c0 > 1) a.chunk_cnt[(size_t)c * 4 + threadIdx.x] = cs;
         }
+        if (c1 - c0 > 1) {
+            __threadfence();   // the row before the count of finished chunks
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                S.last = atomicAdd(&P->done, 1) == c1 - c0 - 1;
+                if (S.last) P->done = 0;
+            }
+            __syncthreads();
+            if (!S.last) continue;
+            __threadfence();   // the other chunks' rows after the count
+            // warp w takes every eighth row; the warps are added in order
+            for (int row = 0; row < rows; ++row) {
+                double sm = 0.0;
+                for (int q = c0 + w; q < c1; q += FIN_THREADS / 32) sm += __ldcg(a.chunk + (size_t)q * 64 + 32 * row + lane);
+                S.red[w][32 * row + lane] = sm;
+            }
+            if (lane < 4) {
+                long long cs = 0;
+                for (int q = c0 + w; q < c1; q += FIN_THREADS / 32) cs += __ldcg(a.chunk_cnt + (size_t)q * 4 + lane);
+                S.cred[w][lane] = cs;
+            }
+            __syncthreads();
+            if (threadIdx.x < 32 * rows) {
+                double sm = 0.0;
+#pragma unroll
+                for (int q = 0; q < FIN_THREADS / 32; ++q) sm += S.red[q][threadIdx.x];
+                S.tot[threadIdx.x] = sm;
+            }
+            if (threadIdx.x < 4) {
+                long long cs = 0;
+#pragma unroll
+                for (int q = 0; q < FIN_THREADS / 32; ++q) cs += S.cred[q][threadIdx.x];
+                S.ctot[threadIdx.x] = cs;
+            }
+        }
+        __syncthreads();
+        if (w == 0) fin_step(a, lo, P, S, lane);
         __syncthreads();
     }
 }
 
-// One warp per problem: the sums over its chunk rows in chunk order (FP64),
-// then the per-problem FP64 step on lane 0.
-__global__ void __launch_bounds__(FIN_STEP_WARPS * 32) k_fin_step(FinalizeArgs a) {
-    __shared__ double tot[FIN_STEP_WARPS][64];
-    __shared__ long long ctot[FIN_STEP_WARPS][4];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int prob = blockIdx.x * FIN_STEP_WARPS + w;
-    if (prob >= a.n_problems) return;
-    ProbDev *P = a.probs + prob;
-    if (P->status != 0) return;
-    if (a.mode == FIN_POSE) {
-        if (lane == 0) refresh_pose(a, prob, P);
-        return;
-    }
-    const int rows = (a.mode == FIN_EXACT || a.mode == FIN_EXACT_EVAL) ? 2 : 1;
-    const int c0 = P->c0, c1 = P->c1;
-    for (int row = 0; row < rows; ++row) {
-        double sm = 0.0;
-        for (int c = c0; c < c1; ++c) sm += a.chunk[(size_t)c * 64 + 32 * row + lane];
-        tot[w][32 * row + lane] = sm;
-    }
-    if (lane < 4) {
-        long long cs = 0;
-        for (int c = c0; c < c1; ++c) cs += a.chunk_cnt[(size_t)c * 4 + lane];
-        ctot[w][lane] = cs;
-    }
-    __syncwarp();
-    if (lane == 0 && finalize_thread0(a, prob, P, tot[w], ctot[w])) refresh_pose(a, prob, P);
+// The transform constants of every problem's initial pose, one warp each.
+__global__ void __launch_bounds__(32) k_fin_pose(FinalizeArgs a) {
+    const int prob = blockIdx.x;
+    const GridDev *G = a.grids + prob;
+    refresh_pose(a.probs[prob].T, G->origin, a.probs + prob, threadIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -802,11 +710,8 @@ __global__ void k_transform(TransformArgs a) {
 // Host launchers.
 // ---------------------------------------------------------------------------
 cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t s) {
-    if (a.mode != FIN_POSE) {
-        k_fin_reduce<<<(unsigned)(a.reduce_blocks > 0 ? a.reduce_blocks : 1024), FIN_RED_THREADS, 0, s>>>(a);
-        count_launches(1);
-    }
-    k_fin_step<<<(unsigned)((a.n_problems + FIN_STEP_WARPS - 1) / FIN_STEP_WARPS), FIN_STEP_WARPS * 32, 0, s>>>(a);
+    if (a.mode == FIN_POSE) k_fin_pose<<<(unsigned)a.n_problems, 32, 0, s>>>(a);
+    else k_finalize<<<(unsigned)(a.reduce_blocks > 0 ? a.reduce_blocks : 1024), FIN_THREADS, 0, s>>>(a);
     count_launches(1);
     return cudaGetLastError();
 }

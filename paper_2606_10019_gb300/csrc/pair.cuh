@@ -44,6 +44,7 @@ struct ProbDev {
     int iter;
     int w0, w1;        // range of packed work items
     int c0, c1;        // range of finalize chunks (FIN_CHUNK work items each)
+    int done;          // chunks of the running finalize that are summed (0 between launches)
     int lo;            // 1: the pair passes form r from double-float positions
     float rho2;        // Euclidean pre-test radius squared
     float c2;          // cutoff squared
@@ -72,17 +73,18 @@ struct PairArgs {
     float *part;               // n_items x 64 (hi[32], lo[32])
     float *part2;              // PAIR_EXACT: slots 32.. in a second n_items x 64
     long long *counts;         // n_items x 4
-    int *work;                 // dynamic item counter (zeroed before launch)
+    int *work;                 // dynamic item counter (zero before launch)
     unsigned *status_word;
     int ls_literal;
 };
 
-// The finalize runs in two launches: k_fin_reduce sums the work items of
-// every chunk (FIN_CHUNK consecutive items of one problem) into one FP64 row,
-// then k_fin_step, one warp per problem, adds its chunks' rows in order and
-// takes the FP64 step.  The chunk rows depend only on the problem's own
-// items, so a problem's result does not depend on the rest of the batch.
-constexpr int FIN_CHUNK = 256;
+// The finalize sums the work items of every chunk (FIN_CHUNK consecutive
+// items of one problem) into one FP64 row; the block that finishes a
+// problem's last chunk adds its rows in order and takes the FP64 step.  The
+// chunk rows depend only on the problem's own items, so a problem's result
+// does not depend on the rest of the batch.  128 items are 16 per warp, two
+// rounds of loads; 20,000 source points still make 20 to 40 chunks.
+constexpr int FIN_CHUNK = 128;
 
 // Bytes of the chunk rows for at most n_items work items over np problems.
 inline size_t fin_chunk_bytes(int64_t n_items, int np) {
@@ -99,7 +101,8 @@ struct FinalizeArgs {
     double *chunk;             // per chunk: 64 FP64 slot sums
     long long *chunk_cnt;      // per chunk: 4 count sums
     const int *n_chunks;       // chunks of all problems (written when items are packed)
-    int reduce_blocks;         // grid of k_fin_reduce (a few blocks per SM)
+    int reduce_blocks;         // grid of k_finalize (at most a few blocks per SM)
+    int *work;                 // the pair pass's item counter, zeroed for the next one
     EvalOut *evalout;
     gcvo_iter_log *logs;
     int *n_active;
