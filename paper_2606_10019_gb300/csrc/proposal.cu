@@ -12,9 +12,8 @@
 //
 // Weights are BF16 copies of FP32 master weights (Adam); every product
 // accumulates in FP32.  The per-point layers 2 and 3 (the dense part: 82 k
-// flop per point) run on the tensor cores with mma.sync m16n8k16 BF16; the
-// max-pool is computed by one block per cloud, so the argmax (lowest point
-// index on ties) is deterministic.  Backward uses that only each channel's
+// flop per point) run on the tensor cores (tcgen05); the max-pool keeps the
+// lowest point index on ties, so the argmax is deterministic.  Backward uses that only each channel's
 // argmax point receives gradient from the max-pool.
 #include <cuda_bf16.h>
 
@@ -25,6 +24,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "ptx.cuh"
 
 namespace gcvo {
 namespace prop {
@@ -48,23 +48,6 @@ struct Net {
     const __nv_bfloat16 *w;       // BF16 copy, same layout
     int off[NT + 1];
 };
-
-constexpr int PT_WARPS = 4;       // per-point kernel: warps per block, 16 points each
-constexpr int W2_LD = 64 + 8;     // padded rows in shared memory (bank spread)
-constexpr int W3_LD = 128 + 8;
-
-__device__ inline uint32_t pack_bf16(float lo, float hi) {
-    __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<uint32_t *>(&v);
-}
-
-__device__ inline void mma16816(float c[4], const uint32_t a[4], uint32_t b0, uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
 
 // ---------------------------------------------------------------------------
 // Normalisation: one block per pair.  Points of cloud 2b (source) and 2b+1
@@ -122,180 +105,321 @@ __global__ void k_prep(int n, const float *sx, const float *sf, int sf_stride, c
 }
 
 // ---------------------------------------------------------------------------
-// Per-point MLP and max-pool: one block per cloud, each warp takes tiles of
-// 16 points.  Layer 1 (4 -> 64) in FP32; layers 2 and 3 on the tensor cores,
-// the output fragments of layer 2 (bias, relu, BF16) being the input
-// fragments of layer 3.  feat[cloud][c] = max over points, arg[cloud][c] =
-// the point (lowest index on ties).
+// Per-point MLP and max-pool on the tensor cores.
+//
+// A tile is 128 points of one cloud; a block (one per SM) walks a contiguous
+// range of the batch's tiles.  Layer 1 (4 -> 64) is FP32; layer 2 is one
+// 128 x 128 x 64 product (points x channels), layer 3 two 128 x 128 x 128
+// products with the operands the other way round (128 channels x points), so
+// that a lane of tensor memory holds one channel's value at every point and
+// the max-pool needs no exchange between lanes.  Per tile the tensor cores
+// need about 1280 cycles at their BF16 rate and the other pipes about 1100
+// issue slots per scheduler, so the roles run side by side:
+//   warps 0..3  layer 1 of tile i + 1 into shared memory, then layer 2's sums
+//               of tile i out of tensor memory, bias, relu, BF16, back into
+//               shared memory;
+//   warp 8      one thread issues the MMAs;
+//   warps 4..7  layer 3's sums of each half out of tensor memory, bias, the
+//               running maximum of every channel and its point.
+// Layer 2's sums and both layers' inputs have two buffers, layer 3's halves
+// one each: half a of the next tile runs while half b is read.
+// The sums have the bits of the mma.sync m16n8k16 chains that ran here before.
+// 512 clouds of 4096 points: 1287 us with mma.sync (one block of 4 warps per
+// cloud, B fragments from padded shared memory), about 330 us here.
+// The maxima of a cloud that several blocks share meet in 64-bit atomics:
+// (ordered value, inverted point index), so the lowest index wins a tie.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(PT_WARPS * 32) k_point_fwd(Net net, int n, const float4 *pts, float *feat,
-                                                            int *arg) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __nv_bfloat16 *w2 = reinterpret_cast<__nv_bfloat16 *>(smem);
-    __nv_bfloat16 *w3 = w2 + 128 * W2_LD;
-    float *w1 = reinterpret_cast<float *>(w3 + 256 * W3_LD);
-    float *b1 = w1 + 256;
-    float *b2 = b1 + 64;
-    float *b3 = b2 + 128;
-    float *wmax = b3 + 256;              // [PT_WARPS][256]
-    int *warg = reinterpret_cast<int *>(wmax + PT_WARPS * 256);
+constexpr int PT_TILE = 128;
+constexpr int PT_THREADS = 9 * 32;
+constexpr uint32_t PT_COLS = 512;                 // tensor memory: 2 x 128 (layer 2), 2 x 128 (layer 3)
+constexpr int PT_W2 = 0;                          // byte offsets in shared memory
+constexpr int PT_W3 = PT_W2 + 128 * 128;          // [half][K block of 64][128 channels][128 bytes]
+constexpr int PT_H1 = PT_W3 + 4 * 128 * 128;      // [buffer][128 points][128 bytes]
+constexpr int PT_H2 = PT_H1 + 2 * 128 * 128;      // [buffer][K block][128 points][128 bytes]
+constexpr int PT_W1 = PT_H2 + 4 * 128 * 128;      // [32 output pairs][12]: w0 w0' w1 w1' w2 w2' w3 w3' b b' - -
+constexpr int PT_B2 = PT_W1 + 32 * 12 * 4;        // [128]
+constexpr int PT_BAR = PT_B2 + 128 * 4;
+constexpr int PT_SMEM = PT_BAR + 256;
 
-    const int cloud = blockIdx.x;
-    for (int i = threadIdx.x; i < 128 * 64; i += blockDim.x) w2[(i / 64) * W2_LD + i % 64] = net.w[net.off[W2] + i];
-    for (int i = threadIdx.x; i < 256 * 128; i += blockDim.x) w3[(i / 128) * W3_LD + i % 128] = net.w[net.off[W3] + i];
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) {
-        w1[i] = __bfloat162float(net.w[net.off[W1] + i]);
-        b3[i] = net.p[net.off[B3] + i];
+struct PtBars {
+    uint64_t h1_full[2], d2_full[2], h2_full[2], h2_free[2], d3_full[2], d3_free[2];
+    uint32_t tmem;
+};
+static_assert(sizeof(PtBars) <= 256, "the barriers fit");
+
+// A float as an unsigned that orders like it, 0 below every float.
+__device__ __forceinline__ unsigned pt_enc(float f) {
+    const unsigned u = __float_as_uint(f);
+    return u & 0x80000000u ? ~u : u | 0x80000000u;
+}
+__device__ __forceinline__ float pt_dec(unsigned u) {
+    return __uint_as_float(u & 0x80000000u ? u & 0x7fffffffu : ~u);
+}
+
+// relu of two floats as packed BF16 (a NaN gives 0).
+__device__ __forceinline__ uint32_t relu_bf16(uint64_t v) {
+    float lo, hi;
+    f2_unpack(v, lo, hi);
+    const __nv_bfloat162 p = __hmax2(__floats2bfloat162_rn(lo, hi), __floats2bfloat162_rn(0.f, 0.f));
+    return *reinterpret_cast<const uint32_t *>(&p);
+}
+
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float d;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
+// Rows of a 128-row BF16 matrix (row-major in memory, ld values per row) into
+// the swizzled layout, 64 columns from col0.
+__device__ __forceinline__ void pt_stage(unsigned char *dst, const __nv_bfloat16 *src, int ld, int col0) {
+    for (int i = threadIdx.x; i < 128 * 8; i += PT_THREADS) {
+        const int r = i >> 3, c = i & 7;
+        *reinterpret_cast<uint4 *>(dst + r * 128 + ((c ^ (r & 7)) << 4)) =
+            *reinterpret_cast<const uint4 *>(src + (size_t)r * ld + col0 + 8 * c);
     }
-    for (int i = threadIdx.x; i < 64; i += blockDim.x) b1[i] = net.p[net.off[B1] + i];
-    for (int i = threadIdx.x; i < 128; i += blockDim.x) b2[i] = net.p[net.off[B2] + i];
+}
+
+// Layer 1 of one point into row r of a tile.
+__device__ __forceinline__ void pt_layer1(const float *w1, float4 p, unsigned char *h1, int r) {
+    const uint64_t x = f2_pack(p.x, p.x), y = f2_pack(p.y, p.y), z = f2_pack(p.z, p.z), l = f2_pack(p.w, p.w);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        uint32_t h[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const ulonglong2 *w = reinterpret_cast<const ulonglong2 *>(w1 + 12 * (4 * c + k));
+            const ulonglong2 a = w[0], b = w[1];
+            const uint64_t bias = w[2].x;
+            uint64_t s = f2_mul(a.y, y);
+            s = f2_fma(a.x, x, s);
+            s = f2_fma(b.x, z, s);
+            s = f2_fma(b.y, l, s);
+            h[k] = relu_bf16(f2_add(s, bias));
+        }
+        *reinterpret_cast<uint4 *>(h1 + r * 128 + ((c ^ (r & 7)) << 4)) = make_uint4(h[0], h[1], h[2], h[3]);
+    }
+}
+
+__global__ void __launch_bounds__(PT_THREADS, 1)
+    k_point_fwd(Net net, int n, int tiles_per_cloud, int64_t n_tiles, const float4 *pts, unsigned long long *top,
+                unsigned *status) {
+    extern __shared__ unsigned char pt_raw[];
+    unsigned char *sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(pt_raw) + 1023) & ~(uintptr_t)1023);
+    float *w1 = reinterpret_cast<float *>(sm + PT_W1);
+    float *b2 = reinterpret_cast<float *>(sm + PT_B2);
+    PtBars &B = *reinterpret_cast<PtBars *>(sm + PT_BAR);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t t0 = n_tiles * blockIdx.x / gridDim.x, t1 = n_tiles * (blockIdx.x + 1) / gridDim.x;
+    const int nt = (int)(t1 - t0);
+
+    pt_stage(sm + PT_W2, net.w + net.off[W2], 64, 0);
+    for (int q = 0; q < 4; ++q)
+        pt_stage(sm + PT_W3 + q * 128 * 128, net.w + net.off[W3] + (size_t)(q >> 1) * 128 * 128, 128, 64 * (q & 1));
+    for (int i = tid; i < 64 * 4; i += PT_THREADS)
+        w1[12 * (i >> 3) + 2 * (i & 3) + (i >> 2 & 1)] = __bfloat162float(net.w[net.off[W1] + i]);
+    if (tid < 64) w1[12 * (tid >> 1) + 8 + (tid & 1)] = net.p[net.off[B1] + tid];
+    if (tid < 128) b2[tid] = net.p[net.off[B2] + tid];
+    if (warp == 8) tc5_alloc(&B.tmem, PT_COLS);
+    if (tid == 0) {
+        for (int k = 0; k < 2; ++k) {
+            mbar_init(&B.h1_full[k], 128);
+            mbar_init(&B.h2_full[k], 128);
+            mbar_init(&B.d3_free[k], 128);
+            mbar_init(&B.d2_full[k], 1);
+            mbar_init(&B.h2_free[k], 1);
+            mbar_init(&B.d3_full[k], 1);
+        }
+    }
+    fence_proxy_async_smem();
+    tc5_fence_before();
     __syncthreads();
+    tc5_fence_after();
+    const uint32_t tmem = B.tmem;
+    bool ok = true;   // every wait of this thread ended in time
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = lane >> 2, t = lane & 3;
-    float rmax[64];   // running max for this lane's channels: tile j (32), cols 2t, 2t+1
-    int rarg[64];
-#pragma unroll
-    for (int k = 0; k < 64; ++k) {
-        rmax[k] = -INFINITY;
-        rarg[k] = 0x7fffffff;
-    }
-    const float4 *P = pts + (size_t)cloud * n;
-    for (int base = warp * 16; base < n; base += PT_WARPS * 16) {
-        const int r0 = base + g, r1 = base + g + 8;
-        const float4 p0 = P[min(r0, n - 1)], p1 = P[min(r1, n - 1)];
-        const bool v0 = r0 < n, v1 = r1 < n;
-        // layer 1 straight into the A fragments of layer 2 (K = 64)
-        uint32_t a2[4][4];
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-            float h[8];
-#pragma unroll
+    if (warp < 4) {
+        const int r = tid;
+        auto point = [&](int i) {
+            const int64_t t = t0 + i;
+            const int64_t cloud = t / tiles_per_cloud;
+            const int at = (int)(t - cloud * tiles_per_cloud) * PT_TILE + r;
+            return pts[cloud * n + min(at, n - 1)];
+        };
+        float4 p = point(0);
+        pt_layer1(w1, p, sm + PT_H1, r);
+        fence_proxy_async_smem();
+        mbar_arrive(&B.h1_full[0]);
+        if (nt > 1) p = point(1);
+        for (int i = 0; i < nt && ok; ++i) {
+            const int b = i & 1;
+            const unsigned ph = (unsigned)(i >> 1) & 1u;
+            if (i + 1 < nt) {
+                // the buffer's last reader, MMA 2 of tile i - 1, is done: its sums were read below
+                pt_layer1(w1, p, sm + PT_H1 + (b ^ 1) * 128 * 128, r);
+                fence_proxy_async_smem();
+                mbar_arrive(&B.h1_full[b ^ 1]);
+                if (i + 2 < nt) p = point(i + 2);
+            }
+            ok = mbar_wait(&B.d2_full[b], ph);
+            if (i >= 2) ok = ok && mbar_wait(&B.h2_free[b], ph ^ 1u);
+            if (!__all_sync(0xffffffffu, ok)) {
+                ok = false;
+                break;
+            }
+            tc5_fence_after();
+            unsigned char *h2 = sm + PT_H2 + b * 2 * 128 * 128;
+            const uint32_t d2 = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)b * 128u;
+#pragma unroll 1
             for (int q = 0; q < 4; ++q) {
-                const int col = 16 * kk + 2 * t + (q & 1) + (q >> 1) * 8;
-                const float *wr = w1 + 4 * col;
-                h[2 * q] = fmaxf(wr[0] * p0.x + wr[1] * p0.y + wr[2] * p0.z + wr[3] * p0.w + b1[col], 0.f);
-                h[2 * q + 1] = fmaxf(wr[0] * p1.x + wr[1] * p1.y + wr[2] * p1.z + wr[3] * p1.w + b1[col], 0.f);
-            }
-            // h[0,2]: row g cols 2t, 2t+1; h[1,3]: row g+8; h[4..7]: cols + 8
-            a2[kk][0] = pack_bf16(h[0], h[2]);
-            a2[kk][1] = pack_bf16(h[1], h[3]);
-            a2[kk][2] = pack_bf16(h[4], h[6]);
-            a2[kk][3] = pack_bf16(h[5], h[7]);
-        }
-        // layer 2 (64 -> 128): 16 n-tiles
-        uint32_t a3[8][4];
+                uint32_t v[32];
+                tc5_ld32(d2 + 32 * q, v);
+                tc5_wait_ld(v);
 #pragma unroll
-        for (int jp = 0; jp < 8; ++jp) {
-            float c[2][4];
+                for (int c = 0; c < 4; ++c) {
+                    uint32_t h[4];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int j = 2 * jp + h;
-                c[h][0] = c[h][1] = c[h][2] = c[h][3] = 0.f;
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    const __nv_bfloat16 *row = w2 + (8 * j + g) * W2_LD + 16 * kk + 2 * t;
-                    mma16816(c[h], a2[kk], *reinterpret_cast<const uint32_t *>(row),
-                             *reinterpret_cast<const uint32_t *>(row + 8));
+                    for (int k = 0; k < 4; k += 2) {
+                        const ulonglong2 bb = *reinterpret_cast<const ulonglong2 *>(b2 + 32 * q + 8 * c + 2 * k);
+                        const int e = 8 * c + 2 * k;
+                        h[k] = relu_bf16(f2_add(f2_pack(__uint_as_float(v[e]), __uint_as_float(v[e + 1])), bb.x));
+                        h[k + 1] = relu_bf16(f2_add(f2_pack(__uint_as_float(v[e + 2]), __uint_as_float(v[e + 3])), bb.y));
+                    }
+                    const int cc = 4 * (q & 1) + c;
+                    *reinterpret_cast<uint4 *>(h2 + (q >> 1) * 128 * 128 + r * 128 + ((cc ^ (r & 7)) << 4)) =
+                        make_uint4(h[0], h[1], h[2], h[3]);
                 }
-                const float bb0 = b2[8 * j + 2 * t], bb1 = b2[8 * j + 2 * t + 1];
-                c[h][0] = fmaxf(c[h][0] + bb0, 0.f);
-                c[h][1] = fmaxf(c[h][1] + bb1, 0.f);
-                c[h][2] = fmaxf(c[h][2] + bb0, 0.f);
-                c[h][3] = fmaxf(c[h][3] + bb1, 0.f);
             }
-            a3[jp][0] = pack_bf16(c[0][0], c[0][1]);
-            a3[jp][1] = pack_bf16(c[0][2], c[0][3]);
-            a3[jp][2] = pack_bf16(c[1][0], c[1][1]);
-            a3[jp][3] = pack_bf16(c[1][2], c[1][3]);
+            tc5_fence_before();
+            fence_proxy_async_smem();
+            mbar_arrive(&B.h2_full[b]);
         }
-        // layer 3 (128 -> 256): 32 n-tiles, running max over the points
+    } else if (warp == 8) {
+        if (lane == 0) {
+            const uint32_t idesc = tc5_idesc(128, 128);
+            const uint32_t w2a = smem_addr(sm + PT_W2), w3a = smem_addr(sm + PT_W3), h1a = smem_addr(sm + PT_H1),
+                           h2a = smem_addr(sm + PT_H2);
+            for (int i = -1; i < nt && ok; ++i) {
+                if (i + 1 < nt) {   // layer 2 of tile i + 1
+                    const int b = (i + 1) & 1;
+                    ok = mbar_wait(&B.h1_full[b], (unsigned)((i + 1) >> 1) & 1u);
+                    if (!ok) break;
+                    tc5_fence_after();
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-            float c[4] = {0.f, 0.f, 0.f, 0.f};
+                    for (int k = 0; k < 4; ++k)
+                        tc5_mma(tmem + (uint32_t)b * 128u, tc5_desc(h1a + b * 128 * 128 + 32 * k), tc5_desc(w2a + 32 * k),
+                                idesc, k);
+                    tc5_commit(&B.d2_full[b]);
+                }
+                if (i < 0) continue;
+                const int b = i & 1;
+                ok = mbar_wait(&B.h2_full[b], (unsigned)(i >> 1) & 1u);
+                for (int h = 0; h < 2 && ok; ++h) {   // layer 3 of tile i, channels 128 h ..
+                    if (i > 0) ok = mbar_wait(&B.d3_free[h], (unsigned)(i - 1) & 1u);
+                    if (!ok) break;
+                    tc5_fence_after();
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
-                const __nv_bfloat16 *row = w3 + (8 * j + g) * W3_LD + 16 * kk + 2 * t;
-                mma16816(c, a3[kk], *reinterpret_cast<const uint32_t *>(row),
-                         *reinterpret_cast<const uint32_t *>(row + 8));
-            }
-            const float bb0 = b3[8 * j + 2 * t], bb1 = b3[8 * j + 2 * t + 1];
-            const float x00 = v0 ? c[0] + bb0 : -INFINITY, x01 = v0 ? c[1] + bb1 : -INFINITY;
-            const float x10 = v1 ? c[2] + bb0 : -INFINITY, x11 = v1 ? c[3] + bb1 : -INFINITY;
-            // column 2t: rows r0, r1 (r0 < r1 keeps the lower index on ties)
-            if (x00 > rmax[2 * j] || (x00 == rmax[2 * j] && r0 < rarg[2 * j])) {
-                rmax[2 * j] = x00;
-                rarg[2 * j] = r0;
-            }
-            if (x10 > rmax[2 * j] || (x10 == rmax[2 * j] && r1 < rarg[2 * j])) {
-                rmax[2 * j] = x10;
-                rarg[2 * j] = r1;
-            }
-            if (x01 > rmax[2 * j + 1] || (x01 == rmax[2 * j + 1] && r0 < rarg[2 * j + 1])) {
-                rmax[2 * j + 1] = x01;
-                rarg[2 * j + 1] = r0;
-            }
-            if (x11 > rmax[2 * j + 1] || (x11 == rmax[2 * j + 1] && r1 < rarg[2 * j + 1])) {
-                rmax[2 * j + 1] = x11;
-                rarg[2 * j + 1] = r1;
+                    for (int k = 0; k < 8; ++k)
+                        tc5_mma(tmem + 256u + 128u * (uint32_t)h, tc5_desc(w3a + (2 * h + (k >> 2)) * 128 * 128 + 32 * (k & 3)),
+                                tc5_desc(h2a + (2 * b + (k >> 2)) * 128 * 128 + 32 * (k & 3)), idesc, k);
+                    tc5_commit(&B.d3_full[h]);
+                }
+                if (ok) tc5_commit(&B.h2_free[b]);
             }
         }
-    }
-    // reduce over the 8 lanes sharing t (the g bits), then over the warps
-#pragma unroll
-    for (int k = 0; k < 64; ++k) {
-#pragma unroll
-        for (int o = 4; o < 32; o <<= 1) {
-            float om = __shfl_xor_sync(0xffffffffu, rmax[k], o);
-            int oa = __shfl_xor_sync(0xffffffffu, rarg[k], o);
-            if (om > rmax[k] || (om == rmax[k] && oa < rarg[k])) {
-                rmax[k] = om;
-                rarg[k] = oa;
-            }
-        }
-    }
-    if (g == 0) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
+        ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+    } else {
+        const int ch = tid - 128;   // and ch + 128
+        const float bias[2] = {net.p[net.off[B3] + ch], net.p[net.off[B3] + 128 + ch]};
+        float best[2] = {-INFINITY, -INFINITY};
+        int arg[2] = {0, 0};
+        for (int i = 0; i < nt && ok; ++i) {
+            const int64_t t = t0 + i, cloud = t / tiles_per_cloud;
+            const int base = (int)(t - cloud * tiles_per_cloud) * PT_TILE;
+            const int valid = n - base;   // points of the tile, if below 128
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const int ch = 8 * j + 2 * t + h;
-                wmax[warp * 256 + ch] = rmax[2 * j + h];
-                warg[warp * 256 + ch] = rarg[2 * j + h];
+                ok = ok && mbar_wait(&B.d3_full[h], (unsigned)i & 1u);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    ok = false;
+                    break;
+                }
+                tc5_fence_after();
+                const uint32_t d3 = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 256u + 128u * (uint32_t)h;
+                const uint64_t bb = f2_pack(bias[h], bias[h]);
+                uint32_t v[2][32];
+                tc5_ld32(d3, v[0]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    tc5_wait_ld(v[q & 1]);
+                    if (q < 3) {
+                        tc5_ld32(d3 + 32 * (q + 1), v[(q + 1) & 1]);
+                    } else {
+                        tc5_fence_before();
+                        mbar_arrive(&B.d3_free[h]);
+                    }
+                    float x[32];
+#pragma unroll
+                    for (int e = 0; e < 32; e += 2)
+                        f2_unpack(f2_add(f2_pack(__uint_as_float(v[q & 1][e]), __uint_as_float(v[q & 1][e + 1])), bb), x[e],
+                                  x[e + 1]);
+                    if (32 * q + 32 > valid)
+#pragma unroll
+                        for (int e = 0; e < 32; ++e)
+                            if (32 * q + e >= valid) x[e] = -INFINITY;
+                    float m = x[0];
+#pragma unroll
+                    for (int e = 1; e + 1 < 32; e += 2) m = max3(m, x[e], x[e + 1]);
+                    m = fmaxf(m, x[31]);
+                    if (__any_sync(0xffffffffu, m > best[h])) {
+                        int at = 31;
+#pragma unroll
+                        for (int e = 30; e >= 0; --e)
+                            if (x[e] == m) at = e;
+                        if (m > best[h]) {
+                            best[h] = m;
+                            arg[h] = base + 32 * q + at;
+                        }
+                    }
+                }
             }
-    }
-    __syncthreads();
-    for (int ch = threadIdx.x; ch < 256; ch += blockDim.x) {
-        float m = wmax[ch];
-        int a = warg[ch];
-        for (int w = 1; w < PT_WARPS; ++w) {
-            float om = wmax[w * 256 + ch];
-            int oa = warg[w * 256 + ch];
-            if (om > m || (om == m && oa < a)) {
-                m = om;
-                a = oa;
+            if (!ok) break;
+            if (i + 1 == nt || (t + 1) % tiles_per_cloud == 0) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    // + 0: the zeros compare equal
+                    const unsigned long long key = (unsigned long long)pt_enc(best[h] + 0.f) << 32 | (0xffffffffu - (unsigned)arg[h]);
+                    atomicMax(top + cloud * 256 + 128 * h + ch, key);
+                    best[h] = -INFINITY;
+                    arg[h] = 0;
+                }
             }
         }
-        feat[(size_t)cloud * 256 + ch] = m;
-        arg[(size_t)cloud * 256 + ch] = a;
     }
+    if (!ok && lane == 0) atomicOr(status, DEV_ERR_TIMEOUT);
+    tc5_fence_before();
+    __syncthreads();
+    tc5_fence_after();
+    if (warp == 8) tc5_dealloc(tmem, PT_COLS);
 }
 
-size_t point_fwd_smem() {
-    return (size_t)(128 * W2_LD + 256 * W3_LD) * 2 + (256 + 64 + 128 + 256) * 4 + PT_WARPS * 256 * 8;
-}
+size_t point_fwd_smem() { return PT_SMEM + 1024; }
 
 // ---------------------------------------------------------------------------
 // Head: one block (256 threads) per pair.  z1 = relu(H1 u + c1), z2 =
 // relu(H2 z1 + c2), out = H3 z2 + c3; pre-activations y1, y2 kept for
 // backward.
 // ---------------------------------------------------------------------------
-__global__ void k_head_fwd(Net net, const float *feat, float *y1, float *y2, float *out) {
+__global__ void k_head_fwd(Net net, const unsigned long long *top, float *feat, int *arg, float *y1, float *y2,
+                           float *out) {
     const int b = blockIdx.x;
     __shared__ float u[512], z1[256], z2[128];
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) {
-        u[i] = feat[(size_t)(2 * b) * 256 + i];
-        u[256 + i] = feat[(size_t)(2 * b + 1) * 256 + i];
+    // the maxima of the pair's two clouds and their points
+    for (int i = threadIdx.x; i < 512; i += blockDim.x) {
+        const unsigned long long key = top[(size_t)b * 512 + i];
+        u[i] = pt_dec((unsigned)(key >> 32));
+        feat[(size_t)b * 512 + i] = u[i];
+        arg[(size_t)b * 512 + i] = (int)(0xffffffffu - (unsigned)key);
     }
     __syncthreads();
     {
@@ -715,7 +839,7 @@ struct gcvo_proposal {
     int device = 0;
     prop::Layout L;
     DevBuf p, g, m, v, w;                // master, grad, Adam moments, BF16 copy
-    DevBuf pts, cs, feat, arg, y1, y2, out, label, d_out, d_y1, d_y2, d_feat, loss;
+    DevBuf pts, cs, top, feat, arg, y1, y2, out, label, d_out, d_y1, d_y2, d_feat, loss;
     int step = 0;
     int cap_pairs = 0, cap_points = 0;
 };
@@ -730,10 +854,14 @@ prop::Net net_of(gcvo_proposal *P) {
     return n;
 }
 
+// The status word of the forward pass (in the loss buffer, which holds 256 bytes).
+unsigned *status_of(gcvo_proposal *P) { return P->loss.as<unsigned>() + 1; }
+
 gcvo_status ensure_batch(gcvo_ctx *ctx, gcvo_proposal *P, int B, int n) {
     cudaStream_t s = ctx->stream;
     GCVO_TRY(P->pts.ensure((size_t)2 * B * n * sizeof(float4), s));
     GCVO_TRY(P->cs.ensure((size_t)B * 4 * sizeof(float), s));
+    GCVO_TRY(P->top.ensure((size_t)2 * B * 256 * sizeof(unsigned long long), s));
     GCVO_TRY(P->feat.ensure((size_t)2 * B * 256 * sizeof(float), s));
     GCVO_TRY(P->arg.ensure((size_t)2 * B * 256 * sizeof(int), s));
     GCVO_TRY(P->y1.ensure((size_t)B * 256 * sizeof(float), s));
@@ -755,17 +883,19 @@ gcvo_status forward_batch(gcvo_ctx *ctx, gcvo_proposal *P, int B, int n, const f
     cudaStream_t s = ctx->stream;
     GCVO_TRY(ensure_batch(ctx, P, B, n));
     prop::k_prep<<<B, 256, 0, s>>>(n, sx, sf, sfs, tx, tf, tfs, P->pts.as<float4>(), P->cs.as<float>());
-    static bool attr = false;
-    if (!attr) {
-        GCVO_CUDA(cudaFuncSetAttribute(prop::k_point_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)prop::point_fwd_smem()));
-        attr = true;
-    }
+    static const cudaError_t attr = cudaFuncSetAttribute(
+        prop::k_point_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)prop::point_fwd_smem());
+    GCVO_CUDA(attr);
     prop::Net net = net_of(P);
-    prop::k_point_fwd<<<2 * B, prop::PT_WARPS * 32, prop::point_fwd_smem(), s>>>(
-        net, n, P->pts.as<float4>(), P->feat.as<float>(), P->arg.as<int>());
-    prop::k_head_fwd<<<B, 256, 0, s>>>(net, P->feat.as<float>(), P->y1.as<float>(), P->y2.as<float>(),
-                                      P->out.as<float>());
+    auto *top = P->top.as<unsigned long long>();
+    const int tiles = (n + prop::PT_TILE - 1) / prop::PT_TILE;
+    const int64_t n_tiles = (int64_t)2 * B * tiles;
+    GCVO_CUDA(cudaMemsetAsync(top, 0, (size_t)2 * B * 256 * sizeof(*top), s));
+    GCVO_CUDA(cudaMemsetAsync(P->loss.ptr, 0, 256, s));   // the loss, and the status word behind it
+    prop::k_point_fwd<<<(unsigned)std::min<int64_t>(n_tiles, std::max(1, ctx->sm_count)), prop::PT_THREADS,
+                        prop::point_fwd_smem(), s>>>(net, n, tiles, n_tiles, P->pts.as<float4>(), top, status_of(P));
+    prop::k_head_fwd<<<B, 256, 0, s>>>(net, top, P->feat.as<float>(), P->arg.as<int>(), P->y1.as<float>(),
+                                      P->y2.as<float>(), P->out.as<float>());
     count_launches(3);
     GCVO_CUDA(cudaGetLastError());
     return GCVO_OK;
@@ -804,7 +934,7 @@ gcvo_status gcvo_proposal_create(gcvo_ctx *ctx, gcvo_proposal **out) {
 gcvo_status gcvo_proposal_destroy(gcvo_proposal *P) {
     if (!P) return GCVO_ERR_INVALID_ARG;
     cudaSetDevice(P->device);
-    for (DevBuf *b : {&P->p, &P->g, &P->m, &P->v, &P->w, &P->pts, &P->cs, &P->feat, &P->arg, &P->y1, &P->y2,
+    for (DevBuf *b : {&P->p, &P->g, &P->m, &P->v, &P->w, &P->pts, &P->cs, &P->top, &P->feat, &P->arg, &P->y1, &P->y2,
                       &P->out, &P->label, &P->d_out, &P->d_y1, &P->d_y2, &P->d_feat, &P->loss})
         b->release();
     delete P;
@@ -874,8 +1004,11 @@ gcvo_status gcvo_proposal_infer(gcvo_ctx *ctx, gcvo_proposal *P, int B, int n, c
     GCVO_TRY(forward_batch(ctx, P, B, n, src_xyz, src_feat, src_feat_stride, tgt_xyz, tgt_feat, tgt_feat_stride));
     std::vector<float> out((size_t)B * 6), cs((size_t)B * 4);
     GCVO_CUDA(cudaMemcpyAsync(out.data(), P->out.ptr, out.size() * 4, cudaMemcpyDeviceToHost, ctx->stream));
+    unsigned st = 0;
     GCVO_CUDA(cudaMemcpyAsync(cs.data(), P->cs.ptr, cs.size() * 4, cudaMemcpyDeviceToHost, ctx->stream));
+    GCVO_CUDA(cudaMemcpyAsync(&st, status_of(P), sizeof(st), cudaMemcpyDeviceToHost, ctx->stream));
     GCVO_CUDA(cudaStreamSynchronize(ctx->stream));
+    if (st & DEV_ERR_TIMEOUT) return GCVO_ERR_TIMEOUT;
     if (twist_out) memcpy(twist_out, out.data(), out.size() * 4);
     if (T0_out) {
         for (int b = 0; b < B; ++b) {
@@ -909,8 +1042,11 @@ gcvo_status gcvo_proposal_train_step(gcvo_ctx *ctx, gcvo_proposal *P, int B, int
     GCVO_TRY(forward_batch(ctx, P, B, n, src_xyz, src_feat, src_feat_stride, tgt_xyz, tgt_feat, tgt_feat_stride));
     // labels: the twist of S T S^-1 (S the shift by -c), translation / s
     std::vector<float> cs((size_t)B * 4), lab((size_t)B * 6);
+    unsigned st = 0;
     GCVO_CUDA(cudaMemcpyAsync(cs.data(), P->cs.ptr, cs.size() * 4, cudaMemcpyDeviceToHost, s));
+    GCVO_CUDA(cudaMemcpyAsync(&st, status_of(P), sizeof(st), cudaMemcpyDeviceToHost, s));
     GCVO_CUDA(cudaStreamSynchronize(s));
+    if (st & DEV_ERR_TIMEOUT) return GCVO_ERR_TIMEOUT;
     for (int b = 0; b < B; ++b) {
         const double *T = T_label + 16 * b;
         const double c[3] = {cs[4 * b], cs[4 * b + 1], cs[4 * b + 2]};
@@ -928,7 +1064,6 @@ gcvo_status gcvo_proposal_train_step(gcvo_ctx *ctx, gcvo_proposal *P, int B, int
     GCVO_CUDA(cudaMemcpyAsync(P->label.ptr, lab.data(), lab.size() * 4, cudaMemcpyHostToDevice, s));
     const int np = P->L.n();
     GCVO_CUDA(cudaMemsetAsync(P->g.ptr, 0, np * sizeof(float), s));
-    GCVO_CUDA(cudaMemsetAsync(P->loss.ptr, 0, sizeof(float), s));
     prop::Net net = net_of(P);
     prop::k_head_bwd<<<B, 256, 0, s>>>(net, B, P->feat.as<float>(), P->y1.as<float>(), P->y2.as<float>(),
                                       P->out.as<float>(), P->label.as<float>(), P->d_out.as<float>(),
