@@ -115,22 +115,25 @@ __global__ void k_prep(int n, const float *sx, const float *sf, int sf_stride, c
 // the max-pool needs no exchange between lanes.  Per tile the tensor cores
 // need about 1280 cycles at their BF16 rate and the other pipes about 1100
 // issue slots per scheduler, so the roles run side by side:
-//   warps 0..3  layer 1 of tile i + 1 into shared memory, then layer 2's sums
-//               of tile i out of tensor memory, bias, relu, BF16, back into
-//               shared memory;
-//   warp 8      one thread issues the MMAs;
-//   warps 4..7  layer 3's sums of each half out of tensor memory, bias, the
-//               running maximum of every channel and its point.
-// Layer 2's sums and both layers' inputs have two buffers, layer 3's halves
-// one each: half a of the next tile runs while half b is read.
+//   warps 0..7  in two groups, one for the even and one for the odd tiles:
+//               layer 1 into shared memory, then layer 2's sums out of tensor
+//               memory, bias, relu, BF16, back into shared memory;
+//   warps 8..15 in two groups, one for each half of layer 3's channels: the
+//               sums out of tensor memory, bias, the running maximum of every
+//               channel and its point;
+//   warp 16     one thread issues the MMAs.
+// Each front group has its own buffers, each half of layer 3 its own sums: the
+// next tile's first half runs while this one's second is read.  With one
+// group of each kind, 2 warps per scheduler, the roles' dependent chains left
+// two thirds of the issue slots empty (290 us; tensor pipe 26% busy).
 // The sums have the bits of the mma.sync m16n8k16 chains that ran here before.
 // 512 clouds of 4096 points: 1287 us with mma.sync (one block of 4 warps per
-// cloud, B fragments from padded shared memory), about 330 us here.
+// cloud, B fragments from padded shared memory), about 215 us here.
 // The maxima of a cloud that several blocks share meet in 64-bit atomics:
 // (ordered value, inverted point index), so the lowest index wins a tie.
 // ---------------------------------------------------------------------------
 constexpr int PT_TILE = 128;
-constexpr int PT_THREADS = 9 * 32;
+constexpr int PT_THREADS = 17 * 32;
 constexpr uint32_t PT_COLS = 512;                 // tensor memory: 2 x 128 (layer 2), 2 x 128 (layer 3)
 constexpr int PT_W2 = 0;                          // byte offsets in shared memory
 constexpr int PT_W3 = PT_W2 + 128 * 128;          // [half][K block of 64][128 channels][128 bytes]
@@ -183,7 +186,7 @@ __device__ __forceinline__ void pt_stage(unsigned char *dst, const __nv_bfloat16
 // Layer 1 of one point into row r of a tile.
 __device__ __forceinline__ void pt_layer1(const float *w1, float4 p, unsigned char *h1, int r) {
     const uint64_t x = f2_pack(p.x, p.x), y = f2_pack(p.y, p.y), z = f2_pack(p.z, p.z), l = f2_pack(p.w, p.w);
-#pragma unroll
+#pragma unroll 4
     for (int c = 0; c < 8; ++c) {
         uint32_t h[4];
 #pragma unroll
@@ -220,7 +223,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1)
         w1[12 * (i >> 3) + 2 * (i & 3) + (i >> 2 & 1)] = __bfloat162float(net.w[net.off[W1] + i]);
     if (tid < 64) w1[12 * (tid >> 1) + 8 + (tid & 1)] = net.p[net.off[B1] + tid];
     if (tid < 128) b2[tid] = net.p[net.off[B2] + tid];
-    if (warp == 8) tc5_alloc(&B.tmem, PT_COLS);
+    if (warp == 16) tc5_alloc(&B.tmem, PT_COLS);
     if (tid == 0) {
         for (int k = 0; k < 2; ++k) {
             mbar_init(&B.h1_full[k], 128);
@@ -238,29 +241,24 @@ __global__ void __launch_bounds__(PT_THREADS, 1)
     const uint32_t tmem = B.tmem;
     bool ok = true;   // every wait of this thread ended in time
 
-    if (warp < 4) {
-        const int r = tid;
+    if (warp < 8) {
+        const int r = tid & 127, b = warp >> 2;   // row of the tile, group
         auto point = [&](int i) {
             const int64_t t = t0 + i;
             const int64_t cloud = t / tiles_per_cloud;
             const int at = (int)(t - cloud * tiles_per_cloud) * PT_TILE + r;
             return pts[cloud * n + min(at, n - 1)];
         };
-        float4 p = point(0);
-        pt_layer1(w1, p, sm + PT_H1, r);
-        fence_proxy_async_smem();
-        mbar_arrive(&B.h1_full[0]);
-        if (nt > 1) p = point(1);
-        for (int i = 0; i < nt && ok; ++i) {
-            const int b = i & 1;
+        unsigned char *h1 = sm + PT_H1 + b * 128 * 128, *h2 = sm + PT_H2 + b * 2 * 128 * 128;
+        const uint32_t d2 = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)b * 128u;
+        float4 p = point(min(b, nt - 1));
+        for (int i = b; i < nt && ok; i += 2) {
             const unsigned ph = (unsigned)(i >> 1) & 1u;
-            if (i + 1 < nt) {
-                // the buffer's last reader, MMA 2 of tile i - 1, is done: its sums were read below
-                pt_layer1(w1, p, sm + PT_H1 + (b ^ 1) * 128 * 128, r);
-                fence_proxy_async_smem();
-                mbar_arrive(&B.h1_full[b ^ 1]);
-                if (i + 2 < nt) p = point(i + 2);
-            }
+            // h1's last reader, the group's last layer-2 product, is done: its sums were read below
+            pt_layer1(w1, p, h1, r);
+            fence_proxy_async_smem();
+            mbar_arrive(&B.h1_full[b]);
+            if (i + 2 < nt) p = point(i + 2);
             ok = mbar_wait(&B.d2_full[b], ph);
             if (i >= 2) ok = ok && mbar_wait(&B.h2_free[b], ph ^ 1u);
             if (!__all_sync(0xffffffffu, ok)) {
@@ -268,8 +266,6 @@ __global__ void __launch_bounds__(PT_THREADS, 1)
                 break;
             }
             tc5_fence_after();
-            unsigned char *h2 = sm + PT_H2 + b * 2 * 128 * 128;
-            const uint32_t d2 = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)b * 128u;
 #pragma unroll 1
             for (int q = 0; q < 4; ++q) {
                 uint32_t v[32];
@@ -294,7 +290,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1)
             fence_proxy_async_smem();
             mbar_arrive(&B.h2_full[b]);
         }
-    } else if (warp == 8) {
+    } else if (warp == 16) {
         if (lane == 0) {
             const uint32_t idesc = tc5_idesc(128, 128);
             const uint32_t w2a = smem_addr(sm + PT_W2), w3a = smem_addr(sm + PT_W3), h1a = smem_addr(sm + PT_H1),
@@ -329,70 +325,66 @@ __global__ void __launch_bounds__(PT_THREADS, 1)
         }
         ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
     } else {
-        const int ch = tid - 128;   // and ch + 128
-        const float bias[2] = {net.p[net.off[B3] + ch], net.p[net.off[B3] + 128 + ch]};
-        float best[2] = {-INFINITY, -INFINITY};
-        int arg[2] = {0, 0};
+        const int h = (warp >> 2) - 2, ch = tid - 256;   // half, channel
+        const uint32_t d3 = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 256u + 128u * (uint32_t)h;
+        const float bias = net.p[net.off[B3] + ch];
+        const uint64_t bb = f2_pack(bias, bias);
+        float best = -INFINITY;
+        int arg = 0;
         for (int i = 0; i < nt && ok; ++i) {
             const int64_t t = t0 + i, cloud = t / tiles_per_cloud;
             const int base = (int)(t - cloud * tiles_per_cloud) * PT_TILE;
             const int valid = n - base;   // points of the tile, if below 128
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                ok = ok && mbar_wait(&B.d3_full[h], (unsigned)i & 1u);
-                if (!__all_sync(0xffffffffu, ok)) {
-                    ok = false;
-                    break;
+            ok = mbar_wait(&B.d3_full[h], (unsigned)i & 1u);
+            if (!__all_sync(0xffffffffu, ok)) {
+                ok = false;
+                break;
+            }
+            tc5_fence_after();
+#pragma unroll 1
+            for (int q = 0; q < 4; ++q) {
+                uint32_t v[32];
+                tc5_ld32(d3 + 32 * q, v);
+                tc5_wait_ld(v);
+                if (q == 3) {
+                    tc5_fence_before();
+                    mbar_arrive(&B.d3_free[h]);
                 }
-                tc5_fence_after();
-                const uint32_t d3 = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 256u + 128u * (uint32_t)h;
-                const uint64_t bb = f2_pack(bias[h], bias[h]);
-                uint32_t v[2][32];
-                tc5_ld32(d3, v[0]);
+                float x[32];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    tc5_wait_ld(v[q & 1]);
-                    if (q < 3) {
-                        tc5_ld32(d3 + 32 * (q + 1), v[(q + 1) & 1]);
-                    } else {
-                        tc5_fence_before();
-                        mbar_arrive(&B.d3_free[h]);
-                    }
-                    float x[32];
+                for (int e = 0; e < 32; e += 2)
+                    f2_unpack(f2_add(f2_pack(__uint_as_float(v[e]), __uint_as_float(v[e + 1])), bb), x[e], x[e + 1]);
+                if (32 * q + 32 > valid)
 #pragma unroll
-                    for (int e = 0; e < 32; e += 2)
-                        f2_unpack(f2_add(f2_pack(__uint_as_float(v[q & 1][e]), __uint_as_float(v[q & 1][e + 1])), bb), x[e],
-                                  x[e + 1]);
-                    if (32 * q + 32 > valid)
+                    for (int e = 0; e < 32; ++e)
+                        if (32 * q + e >= valid) x[e] = -INFINITY;
+                float m[4];
 #pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            if (32 * q + e >= valid) x[e] = -INFINITY;
-                    float m = x[0];
+                for (int e = 0; e < 4; ++e) m[e] = max3(x[e], x[e + 4], x[e + 8]);
 #pragma unroll
-                    for (int e = 1; e + 1 < 32; e += 2) m = max3(m, x[e], x[e + 1]);
-                    m = fmaxf(m, x[31]);
-                    if (__any_sync(0xffffffffu, m > best[h])) {
-                        int at = 31;
+                for (int e = 12; e < 28; e += 8)
 #pragma unroll
-                        for (int e = 30; e >= 0; --e)
-                            if (x[e] == m) at = e;
-                        if (m > best[h]) {
-                            best[h] = m;
-                            arg[h] = base + 32 * q + at;
-                        }
+                    for (int k = 0; k < 4; ++k) m[k] = max3(m[k], x[e + k], x[e + 4 + k]);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) m[k] = fmaxf(m[k], x[28 + k]);
+                const float top4 = max3(fmaxf(m[0], m[1]), m[2], m[3]);
+                if (__any_sync(0xffffffffu, top4 > best)) {
+                    int at = 31;
+#pragma unroll
+                    for (int e = 30; e >= 0; --e)
+                        if (x[e] == top4) at = e;
+                    if (top4 > best) {
+                        best = top4;
+                        arg = base + 32 * q + at;
                     }
                 }
             }
-            if (!ok) break;
             if (i + 1 == nt || (t + 1) % tiles_per_cloud == 0) {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    // + 0: the zeros compare equal
-                    const unsigned long long key = (unsigned long long)pt_enc(best[h] + 0.f) << 32 | (0xffffffffu - (unsigned)arg[h]);
-                    atomicMax(top + cloud * 256 + 128 * h + ch, key);
-                    best[h] = -INFINITY;
-                    arg[h] = 0;
-                }
+                // + 0: the zeros compare equal
+                const unsigned long long key = (unsigned long long)pt_enc(best + 0.f) << 32 | (0xffffffffu - (unsigned)arg);
+                atomicMax(top + cloud * 256 + ch, key);
+                best = -INFINITY;
+                arg = 0;
             }
         }
     }
@@ -400,7 +392,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1)
     tc5_fence_before();
     __syncthreads();
     tc5_fence_after();
-    if (warp == 8) tc5_dealloc(tmem, PT_COLS);
+    if (warp == 16) tc5_dealloc(tmem, PT_COLS);
 }
 
 size_t point_fwd_smem() { return PT_SMEM + 1024; }
