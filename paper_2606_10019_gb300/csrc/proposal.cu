@@ -52,55 +52,197 @@ struct Net {
 // ---------------------------------------------------------------------------
 // Normalisation: one block per pair.  Points of cloud 2b (source) and 2b+1
 // (target) are written as float4 (x', y', z', l).
+//
+// Centroid and RMS radius are FP64 values; a thread's sums run in pairs of
+// floats (TwoSum and exact products by FMA, about 2^-48 relative) and only the
+// block's few partial sums in FP64, on one thread each: FP64 on every thread,
+// at 2 results per SM and cycle, was most of this kernel (256 pairs of 4096
+// points: 67 us, now about 27).
 // ---------------------------------------------------------------------------
-__global__ void k_prep(int n, const float *sx, const float *sf, int sf_stride, const float *tx, const float *tf,
-                       int tf_stride, float4 *pts, float *cs) {
+constexpr int PREP_THREADS = 512;
+
+// (s, e) += v, s + e the sum to about twice float's precision.
+__device__ __forceinline__ void acc2(float &s, float &e, float v) {
+    const float t = __fadd_rn(s, v), bb = __fsub_rn(t, s);
+    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(v, bb)));
+    s = t;
+}
+
+// The block's sum of every thread's (h, l) for K values, in FP64 to thread k.
+template <int K>
+__device__ double prep_block_sum(float (&h)[K], float (&l)[K], float2 (*red)[3]) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const float hh = __shfl_xor_sync(0xffffffffu, h[k], o), ll = __shfl_xor_sync(0xffffffffu, l[k], o);
+            acc2(h[k], l[k], hh);
+            l[k] = __fadd_rn(l[k], ll);
+        }
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int k = 0; k < K; ++k) red[threadIdx.x >> 5][k] = make_float2(h[k], l[k]);
+    __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x < K)
+        for (int q = 0; q < PREP_THREADS / 32; ++q)
+            s += (double)red[q][threadIdx.x].x + (double)red[q][threadIdx.x].y;
+    return s;
+}
+
+// The block's sum of one double per thread, to every thread (only for values
+// beyond float's range).
+__device__ double prep_block_sum64(double v, double *red) {
+    __syncthreads();
+    if (threadIdx.x == 0) *red = 0.0;
+    __syncthreads();
+    atomicAdd(red, v);
+    __syncthreads();
+    return *red;
+}
+
+// log of a rigid transform: rotation vector from the skew part of R (with
+// the symmetric part near pi), translation through the inverse V matrix.
+__device__ void se3_log(const double T[16], double xi[6]) {
+    const double R[9] = {T[0], T[1], T[2], T[4], T[5], T[6], T[8], T[9], T[10]};
+    const double cth = fmin(1.0, fmax(-1.0, (R[0] + R[4] + R[8] - 1.0) / 2.0));
+    double th = acos(cth);
+    double w[3];
+    if (th < 1e-6) {
+        w[0] = (R[7] - R[5]) / 2;
+        w[1] = (R[2] - R[6]) / 2;
+        w[2] = (R[3] - R[1]) / 2;
+    } else if (M_PI - th < 1e-4) {
+        // axis from the diagonal of (R + I) / 2 = n n^T
+        const double d[3] = {sqrt(fmax(0.0, (R[0] + 1) / 2)), sqrt(fmax(0.0, (R[4] + 1) / 2)),
+                             sqrt(fmax(0.0, (R[8] + 1) / 2))};
+        const int k = d[0] >= d[1] && d[0] >= d[2] ? 0 : (d[1] >= d[2] ? 1 : 2);
+        double nrm[3];
+        for (int j = 0; j < 3; ++j) nrm[j] = j == k ? d[k] : (R[3 * k + j] + R[3 * j + k]) / (4 * d[k]);
+        const double s = 1.0 / sqrt(nrm[0] * nrm[0] + nrm[1] * nrm[1] + nrm[2] * nrm[2]);
+        for (int j = 0; j < 3; ++j) w[j] = nrm[j] * s * th;
+    } else {
+        const double f = th / (2 * sin(th));
+        w[0] = (R[7] - R[5]) * f;
+        w[1] = (R[2] - R[6]) * f;
+        w[2] = (R[3] - R[1]) * f;
+    }
+    // V^-1 t = (I - 1/2 W + (1/th^2)(1 - A / (2B)) W^2) t
+    const double th2 = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
+    th = sqrt(th2);
+    double D;
+    if (th < 1e-4) {
+        D = 1.0 / 12 + th2 / 720;
+    } else {
+        double sn, cn;
+        sincos(th, &sn, &cn);
+        D = (1 - sn / th / (2 * ((1 - cn) / th2))) / th2;
+    }
+    // W t = w x t, W^2 t = w (w . t) - th^2 t
+    const double t[3] = {T[3], T[7], T[11]};
+    const double wt = w[0] * t[0] + w[1] * t[1] + w[2] * t[2];
+    const double Wt[3] = {w[1] * t[2] - w[2] * t[1], w[2] * t[0] - w[0] * t[2], w[0] * t[1] - w[1] * t[0]};
+    for (int k = 0; k < 3; ++k) {
+        xi[k] = w[k];
+        xi[3 + k] = t[k] - 0.5 * Wt[k] + D * (w[k] * wt - th2 * t[k]);
+    }
+}
+
+// T_label, label: with labels (training), the twist of S T S^-1 (S the shift
+// by -c), translation / s, of the pair's pose; one thread has it ready while
+// the others write the points, and no host waits for c and s.
+__global__ void __launch_bounds__(PREP_THREADS)
+    k_prep(int n, const float *sx, const float *sf, int sf_stride, const float *tx, const float *tf, int tf_stride,
+           float4 *pts, float *cs, const double *T_label, float *label) {
+    __shared__ float2 red[PREP_THREADS / 32][3];
+    __shared__ double c64[3], r64, wide;
+    __shared__ float ch[3], cl[3], is;
     const int b = blockIdx.x;
     const float *t = tx + (size_t)b * 3 * n;
     const float *s = sx + (size_t)b * 3 * n;
-    __shared__ double red[4][256];
-    double a0 = 0, a1 = 0, a2 = 0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        a0 += t[i];
-        a1 += t[n + i];
-        a2 += t[2 * n + i];
-    }
-    red[0][threadIdx.x] = a0;
-    red[1][threadIdx.x] = a1;
-    red[2][threadIdx.x] = a2;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o)
-            for (int k = 0; k < 3; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + o];
+    {
+        float h[3] = {0.f, 0.f, 0.f}, l[3] = {0.f, 0.f, 0.f};
+#pragma unroll 4
+        for (int i = threadIdx.x; i < n; i += PREP_THREADS)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) acc2(h[a], l[a], t[(size_t)a * n + i]);
+        const double sum = prep_block_sum<3>(h, l, red);
+        if (threadIdx.x < 3) c64[threadIdx.x] = sum / n;
+        __syncthreads();
+        for (int a = 0; a < 3; ++a)
+            if (!isfinite(c64[a])) {
+                double v = 0.0;
+                for (int i = threadIdx.x; i < n; i += PREP_THREADS) v += t[(size_t)a * n + i];
+                v = prep_block_sum64(v, &wide);
+                if (threadIdx.x == 0) c64[a] = v / n;
+                __syncthreads();
+            }
+        if (threadIdx.x < 3) {
+            ch[threadIdx.x] = (float)c64[threadIdx.x];
+            cl[threadIdx.x] = (float)(c64[threadIdx.x] - (double)ch[threadIdx.x]);
+        }
         __syncthreads();
     }
-    const double c0 = red[0][0] / n, c1 = red[1][0] / n, c2 = red[2][0] / n;
-    __syncthreads();
-    double r2 = 0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        double d0 = t[i] - c0, d1 = t[n + i] - c1, d2 = t[2 * n + i] - c2;
-        r2 += d0 * d0 + d1 * d1 + d2 * d2;
-    }
-    red[3][threadIdx.x] = r2;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[3][threadIdx.x] += red[3][threadIdx.x + o];
+    {
+        float rh[1] = {0.f}, rl[1] = {0.f};
+#pragma unroll 4
+        for (int i = threadIdx.x; i < n; i += PREP_THREADS)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                // d + e = t - c, and its square
+                float d = t[(size_t)a * n + i], e = 0.f;
+                acc2(d, e, -ch[a]);
+                e = __fsub_rn(e, cl[a]);
+                const float p = __fmul_rn(d, d);
+                acc2(rh[0], rl[0], p);
+                rl[0] = __fadd_rn(rl[0], __fmaf_rn(d, d, -p) + 2.f * d * e);
+            }
+        const double sum = prep_block_sum<1>(rh, rl, red);
+        if (threadIdx.x == 0) r64 = sum;
+        __syncthreads();
+        if (!isfinite(r64)) {
+            double v = 0.0;
+            for (int i = threadIdx.x; i < n; i += PREP_THREADS)
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const double d = t[(size_t)a * n + i] - c64[a];
+                    v += d * d;
+                }
+            v = prep_block_sum64(v, &wide);
+            if (threadIdx.x == 0) r64 = v;
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            r64 = sqrt(r64 / n) + 1e-6;
+            is = (float)(1.0 / r64);
+        }
         __syncthreads();
     }
-    const double sc = sqrt(red[3][0] / n) + 1e-6;
-    const float is = (float)(1.0 / sc);
-    if (threadIdx.x == 0) {
-        cs[4 * b + 0] = (float)c0;
-        cs[4 * b + 1] = (float)c1;
-        cs[4 * b + 2] = (float)c2;
-        cs[4 * b + 3] = (float)sc;
+    const double sc = r64;
+    if (threadIdx.x == PREP_THREADS - 1) {
+        const float sf32 = (float)sc;
+        cs[4 * b] = ch[0];
+        cs[4 * b + 1] = ch[1];
+        cs[4 * b + 2] = ch[2];
+        cs[4 * b + 3] = sf32;
+        if (T_label) {
+            double Tc[16], xi[6];
+            for (int k = 0; k < 16; ++k) Tc[k] = T_label[16 * (size_t)b + k];
+            const double q[3] = {ch[0], ch[1], ch[2]};
+            for (int r = 0; r < 3; ++r)
+                Tc[4 * r + 3] += Tc[4 * r] * q[0] + Tc[4 * r + 1] * q[1] + Tc[4 * r + 2] * q[2] - q[r];
+            se3_log(Tc, xi);
+            for (int k = 0; k < 6; ++k) label[6 * (size_t)b + k] = (float)(k < 3 ? xi[k] : xi[k] / sf32);
+        }
     }
-    const float f0 = (float)c0, f1 = (float)c1, f2 = (float)c2;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        pts[(size_t)(2 * b) * n + i] = make_float4((s[i] - f0) * is, (s[n + i] - f1) * is, (s[2 * n + i] - f2) * is,
-                                                   sf[(size_t)b * sf_stride + i]);
-        pts[(size_t)(2 * b + 1) * n + i] = make_float4((t[i] - f0) * is, (t[n + i] - f1) * is,
-                                                       (t[2 * n + i] - f2) * is, tf[(size_t)b * tf_stride + i]);
+#pragma unroll 2
+    for (int i = threadIdx.x; i < n; i += PREP_THREADS) {
+        pts[(size_t)(2 * b) * n + i] =
+            make_float4((s[i] - ch[0]) * is, (s[(size_t)n + i] - ch[1]) * is, (s[2 * (size_t)n + i] - ch[2]) * is,
+                        sf[(size_t)b * sf_stride + i]);
+        pts[(size_t)(2 * b + 1) * n + i] =
+            make_float4((t[i] - ch[0]) * is, (t[(size_t)n + i] - ch[1]) * is, (t[2 * (size_t)n + i] - ch[2]) * is,
+                        tf[(size_t)b * tf_stride + i]);
     }
 }
 
@@ -398,112 +540,184 @@ __global__ void __launch_bounds__(PT_THREADS, 1)
 size_t point_fwd_smem() { return PT_SMEM + 1024; }
 
 // ---------------------------------------------------------------------------
-// Head: one block (256 threads) per pair.  z1 = relu(H1 u + c1), z2 =
-// relu(H2 z1 + c2), out = H3 z2 + c3; pre-activations y1, y2 kept for
-// backward.
+// Head: one block per pair.  z1 = relu(H1 u + c1), z2 = relu(H2 z1 + c2),
+// out = H3 z2 + c3; pre-activations y1, y2 kept for backward.  A row of
+// weights is read by one warp, 16 (8) BF16 values per lane in 16-byte loads,
+// and its sum taken across the lanes (256 pairs: 19 us); one thread per row
+// read 4 bytes from each of 32 different lines at a time (89 us).
 // ---------------------------------------------------------------------------
-__global__ void k_head_fwd(Net net, const unsigned long long *top, float *feat, int *arg, float *y1, float *y2,
-                           float *out) {
-    const int b = blockIdx.x;
-    __shared__ float u[512], z1[256], z2[128];
-    // the maxima of the pair's two clouds and their points
-    for (int i = threadIdx.x; i < 512; i += blockDim.x) {
+constexpr int HEAD_THREADS = 512;
+
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Dot product of 8 BF16 weights with 8 floats.
+__device__ __forceinline__ float dot8(uint4 w, const float *u, float s) {
+    const uint32_t q[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        s += __uint_as_float(q[k] << 16) * u[2 * k];
+        s += __uint_as_float(q[k] & 0xffff0000u) * u[2 * k + 1];
+    }
+    return s;
+}
+
+__global__ void __launch_bounds__(HEAD_THREADS)
+    k_head_fwd(Net net, const unsigned long long *top, float *feat, int *arg, float *y1, float *y2, float *out) {
+    const int b = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    constexpr int NW = HEAD_THREADS / 32;
+    __shared__ __align__(16) float u[512], z1[256], z2[128];
+    {
+        // the maxima of the pair's two clouds and their points
+        const int i = threadIdx.x;
         const unsigned long long key = top[(size_t)b * 512 + i];
         u[i] = pt_dec((unsigned)(key >> 32));
         feat[(size_t)b * 512 + i] = u[i];
-        arg[(size_t)b * 512 + i] = (int)(0xffffffffu - (unsigned)key);
+        arg[(size_t)b * 512 + i] = key ? (int)(0xffffffffu - (unsigned)key) : 0;   // 0: no block got to it
     }
     __syncthreads();
     {
-        const int o = threadIdx.x;   // 256 outputs
-        const __nv_bfloat16 *w = net.w + net.off[H1] + (size_t)o * 512;
-        float s = net.p[net.off[C1] + o];
-        for (int i = 0; i < 512; i += 2) {
-            float2 wf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(w + i));
-            s += wf.x * u[i] + wf.y * u[i + 1];
+        float x[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) x[k] = u[256 * (k >> 3) + 8 * lane + (k & 7)];
+#pragma unroll 4
+        for (int o = w; o < 256; o += NW) {
+            const uint4 *row = reinterpret_cast<const uint4 *>(net.w + net.off[H1] + (size_t)o * 512);
+            const float s = warp_sum(dot8(row[32 + lane], x + 8, dot8(row[lane], x, 0.f)));
+            if (lane == 0) {
+                const float y = s + net.p[net.off[C1] + o];
+                y1[(size_t)b * 256 + o] = y;
+                z1[o] = fmaxf(y, 0.f);
+            }
         }
-        y1[(size_t)b * 256 + o] = s;
-        z1[o] = fmaxf(s, 0.f);
     }
     __syncthreads();
-    if (threadIdx.x < 128) {
-        const int o = threadIdx.x;
-        const __nv_bfloat16 *w = net.w + net.off[H2] + (size_t)o * 256;
-        float s = net.p[net.off[C2] + o];
-        for (int i = 0; i < 256; i += 2) {
-            float2 wf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(w + i));
-            s += wf.x * z1[i] + wf.y * z1[i + 1];
+    {
+        float x[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) x[k] = z1[8 * lane + k];
+#pragma unroll 4
+        for (int o = w; o < 128; o += NW) {
+            const uint4 *row = reinterpret_cast<const uint4 *>(net.w + net.off[H2] + (size_t)o * 256);
+            const float s = warp_sum(dot8(row[lane], x, 0.f));
+            if (lane == 0) {
+                const float y = s + net.p[net.off[C2] + o];
+                y2[(size_t)b * 128 + o] = y;
+                z2[o] = fmaxf(y, 0.f);
+            }
         }
-        y2[(size_t)b * 128 + o] = s;
-        z2[o] = fmaxf(s, 0.f);
     }
     __syncthreads();
-    if (threadIdx.x < 6) {
-        const int o = threadIdx.x;
-        const __nv_bfloat16 *w = net.w + net.off[H3] + (size_t)o * 128;
-        float s = net.p[net.off[C3] + o];
-        for (int i = 0; i < 128; ++i) s += __bfloat162float(w[i]) * z2[i];
-        out[(size_t)b * 6 + o] = s;
+    if (w < 6) {
+        const __nv_bfloat16 *row = net.w + net.off[H3] + (size_t)w * 128;
+        float s = 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s += __bfloat162float(row[lane + 32 * k]) * z2[lane + 32 * k];
+        s = warp_sum(s);
+        if (lane == 0) out[(size_t)b * 6 + w] = s + net.p[net.off[C3] + w];
     }
 }
 
-// Per-pair backward through the head: deltas of every layer, and d feat.
-__global__ void k_head_bwd(Net net, int B, const float *feat, const float *y1, const float *y2, const float *out,
-                           const float *label, float *d_out, float *d_y1, float *d_y2, float *d_feat, float *loss) {
-    const int b = blockIdx.x;
-    __shared__ float dy2[128], dy1[256], sd_out[6];
-    if (threadIdx.x < 6) {
-        float d = out[(size_t)b * 6 + threadIdx.x] - label[(size_t)b * 6 + threadIdx.x];
-        sd_out[threadIdx.x] = 2.0f * d / (float)B;
-        d_out[(size_t)b * 6 + threadIdx.x] = 2.0f * d / (float)B;
+// Per-pair backward through the head: deltas of every layer, and d feat.  A
+// thread sums a column (the loads of a warp are one line), two threads per
+// column of H2, each half of its rows.
+__global__ void __launch_bounds__(HEAD_THREADS)
+    k_head_bwd(Net net, int B, const float *y1, const float *y2, const float *out, const float *label, float *d_out,
+               float *d_y1, float *d_y2, float *d_feat, float *loss) {
+    const int b = blockIdx.x, i = threadIdx.x;
+    __shared__ float dy2[128], dy1[256], part[256], sd_out[6];
+    if (i < 6) {
+        const float d = out[(size_t)b * 6 + i] - label[(size_t)b * 6 + i];
+        sd_out[i] = 2.0f * d / (float)B;
+        d_out[(size_t)b * 6 + i] = 2.0f * d / (float)B;
         atomicAdd(loss, d * d / (float)B);
     }
     __syncthreads();
-    if (threadIdx.x < 128) {
-        const int i = threadIdx.x;
+    if (i < 128) {
         float s = 0.f;
         for (int o = 0; o < 6; ++o) s += __bfloat162float(net.w[net.off[H3] + o * 128 + i]) * sd_out[o];
-        float d = y2[(size_t)b * 128 + i] > 0.f ? s : 0.f;
+        const float d = y2[(size_t)b * 128 + i] > 0.f ? s : 0.f;
         dy2[i] = d;
         d_y2[(size_t)b * 128 + i] = d;
     }
     __syncthreads();
     {
-        const int i = threadIdx.x;   // 256
+        const int c = i & 255, o0 = (i >> 8) * 64;
         float s = 0.f;
-        for (int o = 0; o < 128; ++o) s += __bfloat162float(net.w[net.off[H2] + o * 256 + i]) * dy2[o];
-        float d = y1[(size_t)b * 256 + i] > 0.f ? s : 0.f;
-        dy1[i] = d;
-        d_y1[(size_t)b * 256 + i] = d;
+#pragma unroll 16
+        for (int o = o0; o < o0 + 64; ++o) s += __bfloat162float(net.w[net.off[H2] + o * 256 + c]) * dy2[o];
+        if (i >= 256) part[c] = s;
+        __syncthreads();
+        if (i < 256) {
+            const float d = y1[(size_t)b * 256 + c] > 0.f ? s + part[c] : 0.f;
+            dy1[c] = d;
+            d_y1[(size_t)b * 256 + c] = d;
+        }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < 512; i += blockDim.x) {
-        float s = 0.f;
-        for (int o = 0; o < 256; ++o) s += __bfloat162float(net.w[net.off[H1] + o * 512 + i]) * dy1[o];
-        // d feat of cloud 2b (i < 256) or 2b+1
-        d_feat[(size_t)(2 * b) * 256 + i] = s;
-    }
+    float s = 0.f;
+#pragma unroll 16
+    for (int o = 0; o < 256; ++o) s += __bfloat162float(net.w[net.off[H1] + o * 512 + i]) * dy1[o];
+    // d feat of cloud 2b (i < 256) or 2b+1
+    d_feat[(size_t)b * 512 + i] = s;
 }
 
-// Head weight gradients: one thread per weight, summed over the batch in
-// order (deterministic).  dW[o][i] = sum_b delta[b][o] * x[b][i].
-__global__ void k_outer_sum(int B, int rows, int cols, const float *delta, int dstride, const float *x, int xstride,
-                            int xrelu_from_pre, float *dW, float *db) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < rows * cols) {
-        const int o = idx / cols, i = idx % cols;
-        float s = 0.f;
-        for (int b = 0; b < B; ++b) {
-            float xv = x[(size_t)b * xstride + i];
-            if (xrelu_from_pre) xv = fmaxf(xv, 0.f);
-            s += delta[(size_t)b * dstride + o] * xv;
-        }
-        dW[idx] += s;
+// Head weight gradients, summed over the batch in order (deterministic):
+// dW[o][i] += sum_b delta[b][o] * x[b][i], db[o] += sum_b delta[b][o], for the
+// three layers in one launch.  A block takes 32 x 32 weights; the batch passes
+// through shared memory 32 pairs at a time, so a delta or an input is read
+// once per 32 weights and not once per weight (256 pairs: three launches of
+// one thread per weight took 264 us, this one 21).
+struct HeadLayer {
+    const float *delta, *x;   // B x rows, B x cols
+    float *dW, *db;
+    int rows, cols, relu;     // relu: x holds pre-activations
+};
+
+__global__ void __launch_bounds__(256) k_head_grad(int B, HeadLayer L0, HeadLayer L1, HeadLayer L2) {
+    __shared__ float sd[32][33], sx[32][33];
+    int t = blockIdx.x;
+    HeadLayer L = L0;
+    for (int q = 0; q < 2; ++q) {
+        const int tiles = (L.rows + 31) / 32 * (L.cols / 32);
+        if (t < tiles) break;
+        t -= tiles;
+        L = q == 0 ? L1 : L2;
     }
-    if (db && idx < rows) {
-        float s = 0.f;
-        for (int b = 0; b < B; ++b) s += delta[(size_t)b * dstride + idx];
-        db[idx] += s;
+    const int o0 = t / (L.cols / 32) * 32, i0 = t % (L.cols / 32) * 32;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // input i0 + tx, outputs o0 + ty + 8 j
+    float s[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int b0 = 0; b0 < B; b0 += 32) {
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int b = b0 + ty + 8 * k;
+            sd[ty + 8 * k][tx] = b < B && o0 + tx < L.rows ? L.delta[(size_t)b * L.rows + o0 + tx] : 0.f;
+            float v = b < B ? L.x[(size_t)b * L.cols + i0 + tx] : 0.f;
+            sx[ty + 8 * k][tx] = L.relu ? fmaxf(v, 0.f) : v;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int b = 0; b < 32; ++b) {
+            const float v = sx[b][tx];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float d = sd[b][ty + 8 * j];
+                s[j] += d * v;
+                sb[j] += d;
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int o = o0 + ty + 8 * j;
+        if (o < L.rows) {
+            L.dW[(size_t)o * L.cols + i0 + tx] += s[j];
+            if (i0 == 0 && tx == 0) L.db[o] += sb[j];
+        }
     }
 }
 
@@ -581,7 +795,7 @@ __global__ void __launch_bounds__(BW_THREADS, 2) k_point_bwd(Net net, int n, int
             const float g = d_feat[e];
             gs[tid] = g;
             // a channel without a gradient adds nothing; a cloud of NaN has no argmax
-            const float4 q = g != 0.f ? pts[(size_t)cloud * n + min(arg[e], n - 1)] : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 q = g != 0.f ? pts[(size_t)cloud * n + min(max(arg[e], 0), n - 1)] : make_float4(0.f, 0.f, 0.f, 0.f);
             *reinterpret_cast<float4 *>(pv + 4 * tid) = q;
             if (g != 0.f) atomicAdd(grad + net.off[B3] + ch0 + tid, g);
         }
@@ -718,10 +932,11 @@ __global__ void __launch_bounds__(BW_THREADS, 2) k_point_bwd(Net net, int n, int
 }
 
 // Adam (Kingma & Ba) on the FP32 master weights; refreshes the BF16 copy.
+// A forward pass that ran out of time (status) leaves the parameters alone.
 __global__ void k_adam(int n, float *p, const float *g, float *m, float *v, __nv_bfloat16 *w, float lr, float b1,
-                       float b2, float eps, float bc1, float bc2) {
+                       float b2, float eps, float bc1, float bc2, const unsigned *status) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n || *status) return;
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi;
     const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
@@ -741,7 +956,7 @@ __global__ void k_to_bf16(int n, const float *p, __nv_bfloat16 *w) {
 }  // namespace gcvo
 
 // ---------------------------------------------------------------------------
-// SE(3) helpers for the label / proposal conversion (host, double).
+// SE(3) exponential of a proposed twist (host, double).
 // ---------------------------------------------------------------------------
 namespace {
 
@@ -774,55 +989,6 @@ void se3_exp(const double xi[6], double T[16]) {
     T[15] = 1;
 }
 
-// log of a rigid transform: rotation vector from the skew part of R (with
-// the symmetric part near pi), translation through the inverse V matrix.
-void se3_log(const double T[16], double xi[6]) {
-    const double R[9] = {T[0], T[1], T[2], T[4], T[5], T[6], T[8], T[9], T[10]};
-    double cth = std::min(1.0, std::max(-1.0, (R[0] + R[4] + R[8] - 1.0) / 2.0));
-    double th = std::acos(cth);
-    double w[3];
-    if (th < 1e-6) {
-        w[0] = (R[7] - R[5]) / 2;
-        w[1] = (R[2] - R[6]) / 2;
-        w[2] = (R[3] - R[1]) / 2;
-    } else if (M_PI - th < 1e-4) {
-        // axis from the diagonal of (R + I) / 2 = n n^T
-        double d[3] = {std::sqrt(std::max(0.0, (R[0] + 1) / 2)), std::sqrt(std::max(0.0, (R[4] + 1) / 2)),
-                       std::sqrt(std::max(0.0, (R[8] + 1) / 2))};
-        int k = d[0] >= d[1] && d[0] >= d[2] ? 0 : (d[1] >= d[2] ? 1 : 2);
-        double nrm[3];
-        nrm[k] = d[k];
-        for (int j = 0; j < 3; ++j)
-            if (j != k) nrm[j] = (R[3 * k + j] + R[3 * j + k]) / (4 * d[k]);
-        double s = 1.0 / std::sqrt(nrm[0] * nrm[0] + nrm[1] * nrm[1] + nrm[2] * nrm[2]);
-        for (int j = 0; j < 3; ++j) w[j] = nrm[j] * s * th;
-    } else {
-        double f = th / (2 * std::sin(th));
-        w[0] = (R[7] - R[5]) * f;
-        w[1] = (R[2] - R[6]) * f;
-        w[2] = (R[3] - R[1]) * f;
-    }
-    // V^-1 t = (I - 1/2 W + (1/th^2)(1 - A / (2B)) W^2) t
-    double th2 = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
-    th = std::sqrt(th2);
-    double D;
-    if (th < 1e-4) D = 1.0 / 12 + th2 / 720;
-    else {
-        double A = std::sin(th) / th, B = (1 - std::cos(th)) / th2;
-        D = (1 - A / (2 * B)) / th2;
-    }
-    double W[9] = {0, -w[2], w[1], w[2], 0, -w[0], -w[1], w[0], 0}, W2[9];
-    for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c) W2[3 * r + c] = W[3 * r] * W[c] + W[3 * r + 1] * W[3 + c] + W[3 * r + 2] * W[6 + c];
-    const double t[3] = {T[3], T[7], T[11]};
-    for (int r = 0; r < 3; ++r) {
-        double s = 0;
-        for (int c = 0; c < 3; ++c) s += ((r == c ? 1.0 : 0.0) - 0.5 * W[3 * r + c] + D * W2[3 * r + c]) * t[c];
-        xi[3 + r] = s;
-    }
-    for (int k = 0; k < 3; ++k) xi[k] = w[k];
-}
-
 }  // namespace
 
 using namespace gcvo;
@@ -831,7 +997,7 @@ struct gcvo_proposal {
     int device = 0;
     prop::Layout L;
     DevBuf p, g, m, v, w;                // master, grad, Adam moments, BF16 copy
-    DevBuf pts, cs, top, feat, arg, y1, y2, out, label, d_out, d_y1, d_y2, d_feat, loss;
+    DevBuf pts, cs, top, feat, arg, y1, y2, out, label, pose, d_out, d_y1, d_y2, d_feat, loss;
     int step = 0;
     int cap_pairs = 0, cap_points = 0;
 };
@@ -860,6 +1026,7 @@ gcvo_status ensure_batch(gcvo_ctx *ctx, gcvo_proposal *P, int B, int n) {
     GCVO_TRY(P->y2.ensure((size_t)B * 128 * sizeof(float), s));
     GCVO_TRY(P->out.ensure((size_t)B * 6 * sizeof(float), s));
     GCVO_TRY(P->label.ensure((size_t)B * 6 * sizeof(float), s));
+    GCVO_TRY(P->pose.ensure((size_t)B * 16 * sizeof(double), s));
     GCVO_TRY(P->d_out.ensure((size_t)B * 6 * sizeof(float), s));
     GCVO_TRY(P->d_y1.ensure((size_t)B * 256 * sizeof(float), s));
     GCVO_TRY(P->d_y2.ensure((size_t)B * 128 * sizeof(float), s));
@@ -870,11 +1037,18 @@ gcvo_status ensure_batch(gcvo_ctx *ctx, gcvo_proposal *P, int B, int n) {
 
 // Normalisation and the forward pass of a batch; leaves out, feat, arg, y1,
 // y2 on the device.
+// With T_label (host, B x 16) the labels' twists too.
 gcvo_status forward_batch(gcvo_ctx *ctx, gcvo_proposal *P, int B, int n, const float *sx, const float *sf, int sfs,
-                          const float *tx, const float *tf, int tfs) {
+                          const float *tx, const float *tf, int tfs, const double *T_label) {
     cudaStream_t s = ctx->stream;
     GCVO_TRY(ensure_batch(ctx, P, B, n));
-    prop::k_prep<<<B, 256, 0, s>>>(n, sx, sf, sfs, tx, tf, tfs, P->pts.as<float4>(), P->cs.as<float>());
+    const double *d_label = nullptr;
+    if (T_label) {
+        d_label = P->pose.as<double>();
+        GCVO_CUDA(cudaMemcpyAsync(P->pose.ptr, T_label, (size_t)B * 16 * sizeof(double), cudaMemcpyHostToDevice, s));
+    }
+    prop::k_prep<<<B, prop::PREP_THREADS, 0, s>>>(n, sx, sf, sfs, tx, tf, tfs, P->pts.as<float4>(), P->cs.as<float>(),
+                                                 d_label, P->label.as<float>());
     static const cudaError_t attr = cudaFuncSetAttribute(
         prop::k_point_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)prop::point_fwd_smem());
     GCVO_CUDA(attr);
@@ -886,7 +1060,7 @@ gcvo_status forward_batch(gcvo_ctx *ctx, gcvo_proposal *P, int B, int n, const f
     GCVO_CUDA(cudaMemsetAsync(P->loss.ptr, 0, 256, s));   // the loss, and the status word behind it
     prop::k_point_fwd<<<(unsigned)std::min<int64_t>(n_tiles, std::max(1, ctx->sm_count)), prop::PT_THREADS,
                         prop::point_fwd_smem(), s>>>(net, n, tiles, n_tiles, P->pts.as<float4>(), top, status_of(P));
-    prop::k_head_fwd<<<B, 256, 0, s>>>(net, top, P->feat.as<float>(), P->arg.as<int>(), P->y1.as<float>(),
+    prop::k_head_fwd<<<B, prop::HEAD_THREADS, 0, s>>>(net, top, P->feat.as<float>(), P->arg.as<int>(), P->y1.as<float>(),
                                       P->y2.as<float>(), P->out.as<float>());
     count_launches(3);
     GCVO_CUDA(cudaGetLastError());
@@ -927,7 +1101,7 @@ gcvo_status gcvo_proposal_destroy(gcvo_proposal *P) {
     if (!P) return GCVO_ERR_INVALID_ARG;
     cudaSetDevice(P->device);
     for (DevBuf *b : {&P->p, &P->g, &P->m, &P->v, &P->w, &P->pts, &P->cs, &P->top, &P->feat, &P->arg, &P->y1, &P->y2,
-                      &P->out, &P->label, &P->d_out, &P->d_y1, &P->d_y2, &P->d_feat, &P->loss})
+                      &P->out, &P->label, &P->pose, &P->d_out, &P->d_y1, &P->d_y2, &P->d_feat, &P->loss})
         b->release();
     delete P;
     return GCVO_OK;
@@ -993,7 +1167,7 @@ gcvo_status gcvo_proposal_infer(gcvo_ctx *ctx, gcvo_proposal *P, int B, int n, c
                                 const float *tgt_feat, int tgt_feat_stride, float *twist_out, double *T0_out) {
     if (!ctx || !P || !src_xyz || !src_feat || !tgt_xyz || !tgt_feat || !valid_batch(B, n)) return GCVO_ERR_INVALID_ARG;
     GCVO_CUDA(cudaSetDevice(ctx->device));
-    GCVO_TRY(forward_batch(ctx, P, B, n, src_xyz, src_feat, src_feat_stride, tgt_xyz, tgt_feat, tgt_feat_stride));
+    GCVO_TRY(forward_batch(ctx, P, B, n, src_xyz, src_feat, src_feat_stride, tgt_xyz, tgt_feat, tgt_feat_stride, nullptr));
     std::vector<float> out((size_t)B * 6), cs((size_t)B * 4);
     GCVO_CUDA(cudaMemcpyAsync(out.data(), P->out.ptr, out.size() * 4, cudaMemcpyDeviceToHost, ctx->stream));
     unsigned st = 0;
@@ -1031,47 +1205,21 @@ gcvo_status gcvo_proposal_train_step(gcvo_ctx *ctx, gcvo_proposal *P, int B, int
         return GCVO_ERR_INVALID_ARG;
     GCVO_CUDA(cudaSetDevice(ctx->device));
     cudaStream_t s = ctx->stream;
-    GCVO_TRY(forward_batch(ctx, P, B, n, src_xyz, src_feat, src_feat_stride, tgt_xyz, tgt_feat, tgt_feat_stride));
-    // labels: the twist of S T S^-1 (S the shift by -c), translation / s
-    std::vector<float> cs((size_t)B * 4), lab((size_t)B * 6);
-    unsigned st = 0;
-    GCVO_CUDA(cudaMemcpyAsync(cs.data(), P->cs.ptr, cs.size() * 4, cudaMemcpyDeviceToHost, s));
-    GCVO_CUDA(cudaMemcpyAsync(&st, status_of(P), sizeof(st), cudaMemcpyDeviceToHost, s));
-    GCVO_CUDA(cudaStreamSynchronize(s));
-    if (st & DEV_ERR_TIMEOUT) return GCVO_ERR_TIMEOUT;
-    for (int b = 0; b < B; ++b) {
-        const double *T = T_label + 16 * b;
-        const double c[3] = {cs[4 * b], cs[4 * b + 1], cs[4 * b + 2]};
-        double Tc[16];
-        memcpy(Tc, T, sizeof(Tc));
-        for (int r = 0; r < 3; ++r)
-            Tc[4 * r + 3] = T[4 * r + 3] - c[r] + (T[4 * r] * c[0] + T[4 * r + 1] * c[1] + T[4 * r + 2] * c[2]);
-        double xi[6];
-        se3_log(Tc, xi);
-        for (int k = 0; k < 3; ++k) {
-            lab[6 * b + k] = (float)xi[k];
-            lab[6 * b + 3 + k] = (float)(xi[3 + k] / cs[4 * b + 3]);
-        }
-    }
-    GCVO_CUDA(cudaMemcpyAsync(P->label.ptr, lab.data(), lab.size() * 4, cudaMemcpyHostToDevice, s));
+    GCVO_TRY(forward_batch(ctx, P, B, n, src_xyz, src_feat, src_feat_stride, tgt_xyz, tgt_feat, tgt_feat_stride,
+                           T_label));
     const int np = P->L.n();
     GCVO_CUDA(cudaMemsetAsync(P->g.ptr, 0, np * sizeof(float), s));
     prop::Net net = net_of(P);
-    prop::k_head_bwd<<<B, 256, 0, s>>>(net, B, P->feat.as<float>(), P->y1.as<float>(), P->y2.as<float>(),
-                                      P->out.as<float>(), P->label.as<float>(), P->d_out.as<float>(),
-                                      P->d_y1.as<float>(), P->d_y2.as<float>(), P->d_feat.as<float>(),
-                                      P->loss.as<float>());
+    prop::k_head_bwd<<<B, prop::HEAD_THREADS, 0, s>>>(net, B, P->y1.as<float>(), P->y2.as<float>(), P->out.as<float>(),
+                                                     P->label.as<float>(), P->d_out.as<float>(), P->d_y1.as<float>(),
+                                                     P->d_y2.as<float>(), P->d_feat.as<float>(), P->loss.as<float>());
     float *g = P->g.as<float>();
     const int *off = P->L.off;
     // dH1 = sum_b dy1 u^T (u = the pair's two features), dH2 = dy2 z1^T, dH3 = dout z2^T
-    prop::k_outer_sum<<<(256 * 512 + 255) / 256, 256, 0, s>>>(B, 256, 512, P->d_y1.as<float>(), 256,
-                                                             P->feat.as<float>(), 512, 0, g + off[prop::H1],
-                                                             g + off[prop::C1]);
-    prop::k_outer_sum<<<(128 * 256 + 255) / 256, 256, 0, s>>>(B, 128, 256, P->d_y2.as<float>(), 128,
-                                                             P->y1.as<float>(), 256, 1, g + off[prop::H2],
-                                                             g + off[prop::C2]);
-    prop::k_outer_sum<<<(6 * 128 + 255) / 256, 256, 0, s>>>(B, 6, 128, P->d_out.as<float>(), 6, P->y2.as<float>(),
-                                                           128, 1, g + off[prop::H3], g + off[prop::C3]);
+    const prop::HeadLayer l1{P->d_y1.as<float>(), P->feat.as<float>(), g + off[prop::H1], g + off[prop::C1], 256, 512, 0};
+    const prop::HeadLayer l2{P->d_y2.as<float>(), P->y1.as<float>(), g + off[prop::H2], g + off[prop::C2], 128, 256, 1};
+    const prop::HeadLayer l3{P->d_out.as<float>(), P->y2.as<float>(), g + off[prop::H3], g + off[prop::C3], 6, 128, 1};
+    prop::k_head_grad<<<8 * 16 + 4 * 8 + 4, 256, 0, s>>>(B, l1, l2, l3);
     // two blocks fit on an SM; fewer when there are not that many units
     static const cudaError_t bwd_attr = cudaFuncSetAttribute(
         prop::k_point_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, prop::BW_SMEM_FLOATS * (int)sizeof(float));
@@ -1080,24 +1228,31 @@ gcvo_status gcvo_proposal_train_step(gcvo_ctx *ctx, gcvo_proposal *P, int B, int
     prop::k_point_bwd<<<std::min(units, 2 * std::max(1, ctx->sm_count)), prop::BW_THREADS,
                         prop::BW_SMEM_FLOATS * sizeof(float), s>>>(net, n, units, P->pts.as<float4>(), P->arg.as<int>(),
                                                                    P->d_feat.as<float>(), g);
-    count_launches(5);
+    count_launches(3);
     GCVO_CUDA(cudaGetLastError());
-    if (grad_out) {
-        GCVO_CUDA(cudaMemcpyAsync(grad_out, g, np * sizeof(float), cudaMemcpyDeviceToHost, s));
-    }
     if (lr > 0.f) {
         P->step += 1;
         const float b1 = 0.9f, b2 = 0.999f;
         const float bc1 = 1.f - std::pow(b1, (float)P->step), bc2 = 1.f - std::pow(b2, (float)P->step);
         prop::k_adam<<<(np + 255) / 256, 256, 0, s>>>(np, P->p.as<float>(), g, P->m.as<float>(), P->v.as<float>(),
-                                                     P->w.as<__nv_bfloat16>(), lr, b1, b2, 1e-8f, bc1, bc2);
+                                                     P->w.as<__nv_bfloat16>(), lr, b1, b2, 1e-8f, bc1, bc2, status_of(P));
         count_launches(1);
         GCVO_CUDA(cudaGetLastError());
     }
-    float L = 0.f;
-    GCVO_CUDA(cudaMemcpyAsync(&L, P->loss.ptr, sizeof(float), cudaMemcpyDeviceToHost, s));
+    float L[2] = {0.f, 0.f};   // the loss, the status word
+    GCVO_CUDA(cudaMemcpyAsync(L, P->loss.ptr, sizeof(L), cudaMemcpyDeviceToHost, s));
     GCVO_CUDA(cudaStreamSynchronize(s));
-    if (loss_out) *loss_out = L;
+    unsigned st;
+    memcpy(&st, &L[1], sizeof(st));
+    if (st) {
+        if (lr > 0.f) P->step -= 1;
+        return GCVO_ERR_TIMEOUT;
+    }
+    if (grad_out) {
+        GCVO_CUDA(cudaMemcpyAsync(grad_out, g, np * sizeof(float), cudaMemcpyDeviceToHost, s));
+        GCVO_CUDA(cudaStreamSynchronize(s));
+    }
+    if (loss_out) *loss_out = L[0];
     return GCVO_OK;
 }
 
