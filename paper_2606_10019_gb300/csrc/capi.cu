@@ -87,6 +87,8 @@ struct Prepared {
     int64_t n_points = 0;
     int feat_dim = 1;
     bool iso = false;
+    bool one = false;           // prepared by prepare_one: state, items and the source at the initial pose
+    int sched = 0;              // the schedule its work items are packed for (0: not the chosen one yet)
     std::vector<ProbDev> probs;
 };
 
@@ -101,18 +103,146 @@ struct Prepared {
 // the tails are worth their 7 instructions per pair; a small scene (2 m,
 // sigma_min 1.4 cm: 1e-4) is accurate in FP32.  Dense mode (no cutoff) and
 // degenerate covariances always take the tails.
-bool pair_needs_lo(const GridDev &g, const gcvo_kernel_params &kp, double rho2, float lmin_src) {
-    if (kp.cutoff <= 0 || !std::isfinite(rho2)) return true;
+double grid_half_diagonal(const GridDev &g) {
     double half = 0.0;
     for (int a = 0; a < 3; ++a) {
         const double e = 0.5 * (double)g.dims[a] * (double)g.h;
         half += e * e;
     }
-    const double R = std::sqrt(half) + std::sqrt(rho2);
+    return std::sqrt(half);
+}
+
+bool pair_needs_lo(const GridDev &g, const gcvo_kernel_params &kp, double rho2, float lmin_src) {
+    if (kp.cutoff <= 0 || !std::isfinite(rho2)) return true;
+    const double R = grid_half_diagonal(g) + std::sqrt(rho2);
     const double s2 = kp.kernel_mode == 1 ? kp.iso_ell * kp.iso_ell
                                           : (double)g.lam_min + (double)std::max(0.0f, lmin_src);
     if (!(s2 > 0.0)) return true;
     return 4.0 * kp.cutoff * R * std::ldexp(1.0, -24) / std::sqrt(s2) > 3e-4;
+}
+
+// The autotuner's key of a problem set's shape: the kernel mode, the feature
+// count and the log2 buckets of the problem count and of the mean source size.
+long long shape_key(const Prepared &P) {
+    int lb_n = 0, lb_p = 0;
+    while ((2LL << lb_n) <= P.n_points / std::max(1, P.n_problems)) ++lb_n;
+    while ((2 << lb_p) <= P.n_problems) ++lb_p;
+    return ((long long)P.iso << 40) | ((long long)P.feat_dim << 32) | ((long long)lb_p << 8) | lb_n;
+}
+
+// The schedule for this shape: a forced one, the tuned one, or 0 when it has
+// to be tuned first.
+int known_schedule(const gcvo_ctx *ctx, const Prepared &P) {
+    if (ctx->forced_sub) return ctx->forced_sub < 256 ? ctx->forced_sub | 2 << 8 : ctx->forced_sub;
+    const long long key = shape_key(P);
+    for (const auto &kv : ctx->tuned)
+        if (kv.first == key) return kv.second;
+    return 0;
+}
+
+// Buffers of the pair and finalize passes.
+gcvo_status pass_buffers(gcvo_ctx *ctx, const Prepared &P) {
+    cudaStream_t s = ctx->stream;
+    GCVO_TRY(ctx->partial.ensure((size_t)std::max(P.n_items, 1) * (64 * sizeof(float) + 4 * sizeof(long long)) +
+                                     fin_chunk_bytes(P.n_items, P.n_problems) + 4096,
+                                 s));
+    GCVO_TRY(ctx->probs.ensure(P.n_problems * sizeof(ProbDev), s));
+    GCVO_TRY(ctx->grids.ensure(P.n_problems * sizeof(GridDev), s));
+    GCVO_TRY(ctx->evalout.ensure(P.n_problems * sizeof(EvalOut) + 256, s));
+    return GCVO_OK;
+}
+
+// A single problem of at most SRC_ONE_MAX points: one launch does all of
+// prepare's work, the work items and the initial transform (srcone.cu), with
+// nothing read back; a non-finite input shows in the status word.
+gcvo_status prepare_one(gcvo_ctx *ctx, const gcvo_problem &q, Prepared &P) {
+    cudaStream_t s = ctx->stream;
+    const gcvo_grid *G = q.target;
+    const gcvo_kernel_params &kp = G->kp;
+    const size_t N = (size_t)q.n_src;
+    P.n_points = q.n_src;
+    P.n_items = (int)q.n_src;
+    P.one = true;
+    const float *in[3] = {q.src_xyz, P.iso ? nullptr : q.src_cov, q.src_feat};
+    const size_t count[3] = {3 * N, 6 * N, (size_t)P.feat_dim * N};
+    size_t need = 0;
+    bool host[3];
+    for (int k = 0; k < 3; ++k) {
+        host[k] = in[k] && !is_device_ptr(in[k]);
+        if (host[k]) need += (count[k] + 63) & ~size_t(63);
+    }
+    if (need) GCVO_TRY(ctx->stage_xyz.ensure(need * sizeof(float), s));
+    size_t off = 0;
+    for (int k = 0; k < 3; ++k)
+        if (host[k]) {
+            float *d = ctx->stage_xyz.as<float>() + off;
+            GCVO_CUDA(cudaMemcpyAsync(d, in[k], count[k] * sizeof(float), cudaMemcpyHostToDevice, s));
+            in[k] = d;
+            off += (count[k] + 63) & ~size_t(63);
+        }
+    GCVO_TRY(ctx->small.ensure(4096, s));
+    GCVO_TRY(ctx->sort_keys.ensure(N * sizeof(unsigned long long), s));
+    for (DevBuf *b : {&ctx->src_pos, &ctx->src_ca, &ctx->src_cb, &ctx->t_pos, &ctx->t_ca, &ctx->t_cb, &ctx->t_lo})
+        GCVO_TRY(b->ensure(N * sizeof(float4), s));
+    if (P.feat_dim > 3)
+        for (DevBuf *b : {&ctx->src_fx, &ctx->t_fx}) GCVO_TRY(b->ensure(N * sizeof(float4), s));
+    GCVO_TRY(ctx->items.ensure(N * sizeof(int4), s));
+    GCVO_TRY(ctx->item_prob.ensure(N * sizeof(int), s));
+    GCVO_TRY(ctx->pack_tmp.ensure(5 * ((N + 63) / 64 * 64) * sizeof(int), s));
+    GCVO_TRY(ctx->status_word.ensure(256, s));
+    GCVO_TRY(pass_buffers(ctx, P));
+    char *sp = ctx->small.as<char>();
+    P.d_nitems = reinterpret_cast<int *>(sp);
+    P.sched = known_schedule(ctx, P);
+    SrcOneArgs a{};
+    a.xyz = in[0];
+    a.cov = in[1];
+    a.feat = in[2];
+    a.n = (int)q.n_src;
+    a.feat_dim = P.feat_dim;
+    a.iso = P.iso;
+    a.inv_hf = 2.0f / G->store.d.h;   // as in prepare
+    a.grid = G->store.d;
+    for (int r = 0; r < 3; ++r) {
+        for (int c = 0; c < 3; ++c) a.T[3 * r + c] = q.T0[4 * r + c];
+        a.T[9 + r] = q.T0[4 * r + 3];
+    }
+    a.cutoff = kp.cutoff;
+    a.sigma2 = kp.sigma2;
+    a.iso_ell = kp.iso_ell;
+    a.half_diag = grid_half_diagonal(G->store.d);
+    a.sub = P.sched ? P.sched & 0xff : 8;
+    a.level = P.sched ? P.sched >> 8 : 2;
+    a.words = ctx->status_word.as<unsigned>();
+    a.prob = ctx->probs.as<ProbDev>();
+    a.grid_out = ctx->grids.as<GridDev>();
+    a.spos = ctx->src_pos.as<float4>();
+    a.sca = ctx->src_ca.as<float4>();
+    a.scb = ctx->src_cb.as<float4>();
+    a.sfx = P.feat_dim > 3 ? ctx->src_fx.as<float4>() : nullptr;
+    a.tpos = ctx->t_pos.as<float4>();
+    a.tca = ctx->t_ca.as<float4>();
+    a.tcb = ctx->t_cb.as<float4>();
+    a.tlo = ctx->t_lo.as<float4>();
+    a.tfx = P.feat_dim > 3 ? ctx->t_fx.as<float4>() : nullptr;
+    a.keys = P.sched ? nullptr : ctx->sort_keys.as<unsigned long long>();
+    a.tmp = ctx->pack_tmp.as<int>();
+    a.items = ctx->items.as<int>();
+    a.item_prob = ctx->item_prob.as<int>();
+    a.n_items = P.d_nitems;
+    GCVO_TRY(launch_src_one(a, s));
+    if (!P.sched) {
+        // the autotuner packs the items for its candidates (pack_items)
+        GCVO_TRY(ctx->scan_tmp.ensure(scan_scratch_bytes(q.n_src) + 1024, s));
+        int *d_pcnt = reinterpret_cast<int *>(sp + 256);
+        int64_t *d_poff = reinterpret_cast<int64_t *>(sp + 512);
+        const int hn = (int)q.n_src;
+        GCVO_CUDA(cudaMemcpyAsync(d_pcnt, &hn, sizeof(int), cudaMemcpyHostToDevice, s));
+        GCVO_CUDA(cudaMemsetAsync(d_poff, 0, sizeof(int64_t), s));
+        P.d_poff = d_poff;
+        P.d_npts = d_pcnt;
+    }
+    return GCVO_OK;
 }
 
 gcvo_status prepare(gcvo_ctx *ctx, int np, const gcvo_problem *pr, Prepared &P) {
@@ -131,6 +261,7 @@ gcvo_status prepare(gcvo_ctx *ctx, int np, const gcvo_problem *pr, Prepared &P) 
     P.n_problems = np;
     P.iso = kp0.kernel_mode == 1;
     P.feat_dim = kp0.feat_dim;
+    if (np == 1 && pr[0].n_src <= SRC_ONE_MAX) return prepare_one(ctx, pr[0], P);
     // stage host inputs
     size_t need = 0;
     int64_t N = 0;
@@ -296,12 +427,7 @@ gcvo_status prepare(gcvo_ctx *ctx, int np, const gcvo_problem *pr, Prepared &P) 
         d.iso_inv = kp.kernel_mode == 1 ? (float)(1.0 / (kp.iso_ell * kp.iso_ell)) : 0.f;
     }
     // per-iteration buffers
-    GCVO_TRY(ctx->partial.ensure((size_t)std::max(P.n_items, 1) * (64 * sizeof(float) + 4 * sizeof(long long)) +
-                                     fin_chunk_bytes(P.n_items, P.n_problems) + 4096,
-                                 s));
-    GCVO_TRY(ctx->probs.ensure(np * sizeof(ProbDev), s));
-    GCVO_TRY(ctx->grids.ensure(np * sizeof(GridDev), s));
-    GCVO_TRY(ctx->evalout.ensure(np * sizeof(EvalOut) + 256, s));
+    GCVO_TRY(pass_buffers(ctx, P));
     std::vector<GridDev> gd(np);
     for (int p = 0; p < np; ++p) gd[p] = pr[p].target->store.d;
     GCVO_CUDA(cudaMemcpyAsync(ctx->probs.ptr, P.probs.data(), np * sizeof(ProbDev), cudaMemcpyHostToDevice, s));
@@ -338,25 +464,17 @@ gcvo_status pack(gcvo_ctx *ctx, const Prepared &P, int sched) {
     return pack_items(P.n_problems, ctx->sort_keys.as<unsigned long long>(), P.n_points, sched & 0xff, sched >> 8,
                       P.d_poff, P.d_npts, ctx->pack_tmp.as<int>(), ctx->items.as<int>(), ctx->item_prob.as<int>(),
                       P.d_nitems, ctx->probs.as<ProbDev>(),
-                      reinterpret_cast<int *>(ctx->status_word.as<char>() + 64) + 2,   // chunk count
+                      ctx->status_word.as<int>() + SRC_WORD_CHUNKS,
                       ctx->scan_tmp.ptr, ctx->stream);
 }
 
 // The autotuner: the schedule for this shape of problem set -- a forced
 // one, the cached choice for the same shape, or the fastest of one timed
-// evaluation pass with each candidate (the second of two, CUDA events).  The
-// shape is the kernel mode, the feature count and the log2 buckets of the
-// problem count and of the mean source size.
+// evaluation pass with each candidate (the second of two, CUDA events).
 gcvo_status choose_schedule(gcvo_ctx *ctx, const Prepared &P, IterBufs &b) {
-    int sched = ctx->forced_sub ? (ctx->forced_sub < 256 ? ctx->forced_sub | 2 << 8 : ctx->forced_sub) : 0;
-    int packed = 0;
-    if (!sched) {
-        int lb_n = 0, lb_p = 0;
-        while ((2LL << lb_n) <= P.n_points / std::max(1, P.n_problems)) ++lb_n;
-        while ((2 << lb_p) <= P.n_problems) ++lb_p;
-        const long long key = ((long long)P.iso << 40) | ((long long)P.feat_dim << 32) | ((long long)lb_p << 8) | lb_n;
-        for (auto &kv : ctx->tuned)
-            if (kv.first == key) sched = kv.second;
+    int sched = P.one && P.sched ? P.sched : known_schedule(ctx, P);
+    int packed = P.one ? P.sched : 0;
+    {
         if (!sched) {
             constexpr int NC = 9;
             const int cands[NC] = {4 | 2 << 8,  8 | 2 << 8,  16 | 2 << 8, 32 | 2 << 8, 8 | 3 << 8,
@@ -392,7 +510,7 @@ gcvo_status choose_schedule(gcvo_ctx *ctx, const Prepared &P, IterBufs &b) {
             }
             for (auto &e : ev) cudaEventDestroy(e);
             if (st != GCVO_OK) return st;
-            ctx->tuned.emplace_back(key, sched);
+            ctx->tuned.emplace_back(shape_key(P), sched);
             GCVO_CUDA(cudaMemsetAsync(b.work, 0, sizeof(int), ctx->stream));
         }
     }
@@ -418,8 +536,8 @@ gcvo_status iter_bufs(gcvo_ctx *ctx, const Prepared &P, IterBufs &b, gcvo_iter_l
     double *chunk = reinterpret_cast<double *>(part + al(ng * 64 * sizeof(float)) + al(ng * 4 * sizeof(long long)));
     long long *chunk_cnt = reinterpret_cast<long long *>(reinterpret_cast<char *>(chunk) +
                                                          al(n_chunk_rows * 64 * sizeof(double)));
-    int *work = reinterpret_cast<int *>(ctx->status_word.as<char>() + 64);
-    int *n_active = work + 1;
+    int *words = ctx->status_word.as<int>();
+    int *work = words + SRC_WORD_WORK, *n_active = words + SRC_WORD_ACTIVE;
     if (exact) GCVO_TRY(ctx->partial2.ensure(ng * 64 * sizeof(float), ctx->stream));
     // the tails of p: every pair pass forms r in double-float
     GCVO_TRY(ctx->t_lo.ensure((size_t)std::max<int64_t>(P.n_points, 1) * sizeof(float4), ctx->stream));
@@ -427,7 +545,7 @@ gcvo_status iter_bufs(gcvo_ctx *ctx, const Prepared &P, IterBufs &b, gcvo_iter_l
     t.spos = ctx->src_pos.as<float4>();
     t.sca = ctx->src_ca.as<float4>();
     t.scb = ctx->src_cb.as<float4>();
-    t.pprob = ctx->pprob.as<int>();
+    t.pprob = P.one ? nullptr : ctx->pprob.as<int>();
     t.probs = ctx->probs.as<ProbDev>();
     t.tpos = ctx->t_pos.as<float4>();
     t.tca = ctx->t_ca.as<float4>();
@@ -462,7 +580,7 @@ gcvo_status iter_bufs(gcvo_ctx *ctx, const Prepared &P, IterBufs &b, gcvo_iter_l
     f.counts = pc;
     f.chunk = chunk;
     f.chunk_cnt = chunk_cnt;
-    f.n_chunks = work + 2;   // written by pack_items
+    f.n_chunks = words + SRC_WORD_CHUNKS;   // written with the work items
     f.reduce_blocks = (int)std::min<int64_t>((int64_t)n_chunk_rows, (int64_t)std::max(1, ctx->sm_count) * 8);
     f.work = work;
     f.evalout = ctx->evalout.as<EvalOut>();
@@ -473,21 +591,27 @@ gcvo_status iter_bufs(gcvo_ctx *ctx, const Prepared &P, IterBufs &b, gcvo_iter_l
     f.eps_tol = 0;
     f.mu0 = 0;
     b.work = work;
-    // transform constants and the transformed source at the initial pose
-    f.mode = FIN_POSE;
-    GCVO_CUDA(launch_finalize(f, ctx->stream));
-    GCVO_CUDA(launch_transform(t, ctx->stream));
+    if (!P.one) {
+        // transform constants and the transformed source at the initial pose
+        f.mode = FIN_POSE;
+        GCVO_CUDA(launch_finalize(f, ctx->stream));
+        GCVO_CUDA(launch_transform(t, ctx->stream));
+    }
     return choose_schedule(ctx, P, b);
+}
+
+gcvo_status status_of_word(unsigned w) {
+    if (w & DEV_ERR_TIMEOUT) return GCVO_ERR_TIMEOUT;
+    if (w & DEV_ERR_CAPACITY) return GCVO_ERR_CAPACITY;
+    if (w & DEV_ERR_NONFINITE) return GCVO_ERR_NONFINITE;
+    return GCVO_OK;
 }
 
 gcvo_status check_status_word(gcvo_ctx *ctx) {
     unsigned w = 0;
     GCVO_CUDA(cudaMemcpyAsync(&w, ctx->status_word.ptr, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream));
     GCVO_CUDA(cudaStreamSynchronize(ctx->stream));
-    if (w & DEV_ERR_TIMEOUT) return GCVO_ERR_TIMEOUT;
-    if (w & DEV_ERR_CAPACITY) return GCVO_ERR_CAPACITY;
-    if (w & DEV_ERR_NONFINITE) return GCVO_ERR_NONFINITE;
-    return GCVO_OK;
+    return status_of_word(w);
 }
 
 // With profiling on, a timed launch is bracketed by two events from the
@@ -650,7 +774,7 @@ gcvo_status run_register(gcvo_ctx *ctx, int np, const gcvo_problem *pr, const gc
     b.fa.eps_tol = sp->eps_tol;
     b.fa.mu0 = sp->mu0;
     int *n_active = b.fa.n_active;
-    GCVO_CUDA(cudaMemcpyAsync(n_active, &np, sizeof(int), cudaMemcpyHostToDevice, s));
+    if (!P.one) GCVO_CUDA(cudaMemcpyAsync(n_active, &np, sizeof(int), cudaMemcpyHostToDevice, s));
     void *hp;
     GCVO_TRY(host_pinned(ctx, 64, &hp));
     int *h_active = static_cast<int *>(hp);
@@ -1001,14 +1125,20 @@ static gcvo_status eval_once(gcvo_ctx *ctx, const gcvo_grid *target, const float
     GCVO_TRY(prepare(ctx, 1, &pr, P));
     IterBufs b{};
     GCVO_TRY(iter_bufs(ctx, P, b, nullptr, 1, mode == PAIR_EXACT));
-    int one = 1;
-    GCVO_CUDA(cudaMemcpyAsync(b.fa.n_active, &one, sizeof(int), cudaMemcpyHostToDevice, ctx->stream));
     GCVO_TRY(launch_pair_pass(ctx, P, b, mode, ctx->stream));
     b.fa.mode = fin;
     GCVO_CUDA(launch_finalize(b.fa, ctx->stream));
-    EvalOut e{};
-    GCVO_CUDA(cudaMemcpyAsync(&e, ctx->evalout.ptr, sizeof(EvalOut), cudaMemcpyDeviceToHost, ctx->stream));
-    GCVO_TRY(check_status_word(ctx));
+    void *hp;
+    GCVO_TRY(host_pinned(ctx, sizeof(EvalOut) + sizeof(unsigned), &hp));
+    GCVO_CUDA(cudaMemcpyAsync(hp, ctx->evalout.ptr, sizeof(EvalOut), cudaMemcpyDeviceToHost, ctx->stream));
+    GCVO_CUDA(cudaMemcpyAsync(static_cast<char *>(hp) + sizeof(EvalOut), ctx->status_word.ptr, sizeof(unsigned),
+                              cudaMemcpyDeviceToHost, ctx->stream));
+    GCVO_CUDA(cudaStreamSynchronize(ctx->stream));
+    EvalOut e;
+    unsigned word;
+    memcpy(&e, hp, sizeof(e));
+    memcpy(&word, static_cast<char *>(hp) + sizeof(EvalOut), sizeof(word));
+    GCVO_TRY(status_of_word(word));
     GCVO_TRY(collect_profile(ctx));
     *f = e.f;
     memcpy(g, e.g, 6 * sizeof(double));
@@ -1018,7 +1148,7 @@ static gcvo_status eval_once(gcvo_ctx *ctx, const gcvo_grid *target, const float
         stats->n_pairs = e.n_pairs;
         stats->n_kept = e.n_kept;
         stats->n_candidates = e.n_cand;
-        stats->rho = std::sqrt((double)P.probs[0].rho2);
+        stats->rho = std::sqrt((double)e.rho2);
     }
     bool finite = std::isfinite(e.f);
     for (int k = 0; k < 6; ++k) finite = finite && std::isfinite(e.g[k]);
@@ -1266,7 +1396,7 @@ gcvo_status gcvo_set_workspace(gcvo_ctx *ctx, void *dev_ptr, size_t bytes, int64
     if (at.type != cudaMemoryTypeDevice || at.device != ctx->device) return GCVO_ERR_INVALID_ARG;
     // the host read-back buffer, sized once for the problem limit
     void *hp;
-    GCVO_TRY(host_pinned(ctx, (size_t)(2 * max_problems + 64) * sizeof(int), &hp));
+    GCVO_TRY(host_pinned(ctx, std::max((size_t)(2 * max_problems + 64) * sizeof(int), sizeof(EvalOut) + 64), &hp));
     const std::vector<size_t> sz = ws_sizes(max_points, max_problems, max_log_rows);
     char *p = static_cast<char *>(dev_ptr);
     for (size_t k = 0; k < bufs.size(); ++k) {

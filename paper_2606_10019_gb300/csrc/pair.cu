@@ -19,6 +19,7 @@
 #include "common.cuh"
 #include "pair.cuh"
 #include "ptx.cuh"
+#include "srcdev.cuh"
 
 namespace gcvo {
 namespace {
@@ -233,28 +234,6 @@ struct FinShared {
     int last;
 };
 
-// The split constants of the transform at the pose T (shared memory): R as
-// float head and tail, and c = R^T t + o (o the grid origin, in memory)
-// likewise.
-__device__ void refresh_pose(const double *T, const double *o, ProbDev *P, int lane) {
-    if (lane >= 12) return;
-    double v;
-    if (lane < 9) {
-        v = T[lane];
-    } else {
-        const int k = lane - 9;
-        v = T[k] * T[9] + T[3 + k] * T[10] + T[6 + k] * T[11] + o[k];
-    }
-    const float h = (float)v, l = (float)(v - (double)h);
-    if (lane < 9) {
-        P->Rh[lane] = h;
-        P->Rl[lane] = l;
-    } else {
-        P->ch[lane - 9] = h;
-        P->cl[lane - 9] = l;
-    }
-}
-
 __device__ __forceinline__ void set_inactive(ProbDev *P, int st, int *n_active) {
     P->status = st;
     atomicSub(n_active, 1);
@@ -294,7 +273,7 @@ __device__ void apply_step(const FinalizeArgs &a, ProbDev *P, FinShared &S, cons
         P->T[lane] = tn;
     }
     __syncwarp();
-    refresh_pose(S.T, o, P, lane);
+    split_pose(S.T, o, P, lane);
     double l1 = 0.0;
 #pragma unroll
     for (int k = 0; k < 6; ++k) l1 += fabs(S.xi[k]);
@@ -400,6 +379,7 @@ __device__ void fin_step(const FinalizeArgs &a, int prob, ProbDev *P, FinShared 
             e->n_pairs = S.ctot[0];
             e->n_kept = S.ctot[1];
             e->n_cand = S.ctot[2];
+            e->rho2 = P->rho2;
         }
         return;
     }
@@ -547,26 +527,12 @@ __global__ void __launch_bounds__(FIN_THREADS) k_finalize(FinalizeArgs a) {
 __global__ void __launch_bounds__(32) k_fin_pose(FinalizeArgs a) {
     const int prob = blockIdx.x;
     const GridDev *G = a.grids + prob;
-    refresh_pose(a.probs[prob].T, G->origin, a.probs + prob, threadIdx.x);
+    split_pose(a.probs[prob].T, G->origin, a.probs + prob, threadIdx.x);
 }
 
 // ---------------------------------------------------------------------------
 // Source grouping.
 // ---------------------------------------------------------------------------
-__device__ inline unsigned spread3(unsigned v) {
-    v &= 0x3ffu;
-    v = (v | (v << 16)) & 0x030000ffu;
-    v = (v | (v << 8)) & 0x0300f00fu;
-    v = (v | (v << 4)) & 0x030c30c3u;
-    v = (v | (v << 2)) & 0x09249249u;
-    return v;
-}
-
-__device__ inline int enc_f(float f) {
-    int i = __float_as_int(f);
-    return i >= 0 ? i : i ^ 0x7fffffff;
-}
-
 __global__ void k_src_keys(SrcArgs a) {
     const int p = blockIdx.y;
     const SrcDesc d = a.desc[p];
@@ -578,13 +544,7 @@ __global__ void k_src_keys(SrcArgs a) {
         c[k] = d.xyz[k * d.n + i];
         r[k] = d.xyz[k * d.n];
     }
-    unsigned m = 0;
-    for (int k = 0; k < 3; ++k) {
-        int q = (int)floorf((c[k] - r[k]) * d.inv_hf) + 512;
-        q = min(max(q, 0), 1023);
-        m |= spread3((unsigned)q) << k;
-    }
-    a.keys[gi] = ((unsigned long long)p << 30) | m;
+    a.keys[gi] = ((unsigned long long)p << 30) | src_code(c, r, d.inv_hf);
     a.vals[gi] = (int)gi;
     a.prob_of[gi] = p;
     a.local[gi] = (int)i;
@@ -597,8 +557,8 @@ __global__ void k_src_keys(SrcArgs a) {
             bad |= !isfinite(s[k]);
         }
         float l = sym3_max_eig(s[0], s[1], s[2], s[3], s[4], s[5]);
-        atomicMax(a.lam_enc + p, enc_f(l));
-        atomicMin(a.lam_min_enc + p, enc_f(sym3_min_eig(s[0], s[1], s[2], s[3], s[4], s[5])));
+        atomicMax(a.lam_enc + p, src_enc(l));
+        atomicMin(a.lam_min_enc + p, src_enc(sym3_min_eig(s[0], s[1], s[2], s[3], s[4], s[5])));
     }
     if (bad) atomicOr(a.status_word, DEV_ERR_NONFINITE);
 }
@@ -628,77 +588,23 @@ __global__ void k_src_pack(SrcArgs a, const unsigned long long *keys, int64_t n)
     a.pprob[i] = (int)(keys[i] >> 30);
 }
 
-// ---------------------------------------------------------------------------
-// The transform of Algorithm 1 (T^-1 z) for every point of an active
-// problem.  p = R^T z - c is formed in double-float arithmetic from the
-// float head / tail splits of R and c: each head product R_h z is split
-// exactly into a float and its rounding error with one FMA (the
-// error-free product of Ogita, Rump and Oishi, "Accurate sum and dot
-// product", SIAM J. Sci. Comput. 2005), the products are added with Knuth's
-// TwoSum and the rounding errors, the tail products and c's tail are
-// summed in a float alongside (their Sum2 / Dot2 scheme), and a final
-// FastTwoSum gives p = p_hi + p_lo with an error near 2^-48 |R| |z|.
-// Sigma' = R^T Sigma R is formed in float from the head of R.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-
+// The transform of Algorithm 1 (T^-1 z, srcdev.cuh) for every point of an
+// active problem.
 __global__ void k_transform(TransformArgs a) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += stride) {
         const ProbDev *P = a.probs + (a.pprob ? a.pprob[i] : 0);
         if (P->status != 0) continue;   // converged or failed: left as it was
-        const float4 z = a.spos[i];
-        const float4 zb = a.scb[i];
-        const float zz[3] = {z.x, z.y, z.z};
-        float hi[3], lo[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            float s = 0.f, err = 0.f;
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                const float rh = P->Rh[3 * j + k];
-                const float pr = __fmul_rn(rh, zz[j]);
-                const float pe = __fmaf_rn(rh, zz[j], -pr);
-                float e;
-                two_sum(s, pr, s, e);
-                err = __fadd_rn(err, __fadd_rn(__fadd_rn(e, pe), __fmul_rn(P->Rl[3 * j + k], zz[j])));
-            }
-            float e;
-            two_sum(s, -P->ch[k], s, e);
-            err = __fadd_rn(err, __fsub_rn(e, P->cl[k]));
-            hi[k] = __fadd_rn(s, err);
-            lo[k] = __fsub_rn(err, __fsub_rn(hi[k], s));
-        }
-        const float sg = P->sigma2;
-        a.tpos[i] = make_float4(hi[0], hi[1], hi[2], sg * z.w);
-        if (a.tlo) a.tlo[i] = make_float4(lo[0], lo[1], lo[2], 0.f);
-        float q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if (!a.iso) {
-            const float4 za = a.sca[i];
-            const float sm[9] = {za.x, za.y, za.z, za.y, za.w, zb.x, za.z, zb.x, zb.y};
-            float Rf[9], T1[9];
-#pragma unroll
-            for (int k = 0; k < 9; ++k) Rf[k] = P->Rh[k];
-#pragma unroll
-            for (int r = 0; r < 3; ++r)
-#pragma unroll
-                for (int c = 0; c < 3; ++c)
-                    T1[3 * r + c] = sm[3 * r] * Rf[c] + sm[3 * r + 1] * Rf[3 + c] + sm[3 * r + 2] * Rf[6 + c];
-            q[0] = Rf[0] * T1[0] + Rf[3] * T1[3] + Rf[6] * T1[6];
-            q[1] = Rf[0] * T1[1] + Rf[3] * T1[4] + Rf[6] * T1[7];
-            q[2] = Rf[0] * T1[2] + Rf[3] * T1[5] + Rf[6] * T1[8];
-            q[3] = Rf[1] * T1[1] + Rf[4] * T1[4] + Rf[7] * T1[7];
-            q[4] = Rf[1] * T1[2] + Rf[4] * T1[5] + Rf[7] * T1[8];
-            q[5] = Rf[2] * T1[2] + Rf[5] * T1[5] + Rf[8] * T1[8];
-        }
-        a.tca[i] = make_float4(q[0], q[1], q[2], q[3]);
-        a.tcb[i] = make_float4(q[4], q[5], sg * zb.z, sg * zb.w);
+        const float4 za = a.iso ? make_float4(0.f, 0.f, 0.f, 0.f) : a.sca[i];
+        float4 tp, tl, ta, tb;
+        transform_point(P, a.spos[i], za, a.scb[i], a.iso != 0, tp, tl, ta, tb);
+        a.tpos[i] = tp;
+        if (a.tlo) a.tlo[i] = tl;
+        a.tca[i] = ta;
+        a.tcb[i] = tb;
         if (a.tfx) {
             const float4 f = a.sfx[i];
+            const float sg = P->sigma2;
             a.tfx[i] = make_float4(sg * f.x, sg * f.y, sg * f.z, sg * f.w);
         }
     }

@@ -55,6 +55,7 @@ struct ProbDev {
 struct EvalOut {
     double f, g[6], M[36], H[36];
     long long n_pairs, n_kept, n_cand;
+    float rho2;
 };
 
 // Source points in the target grid's frame at the current pose, written by
@@ -145,7 +146,32 @@ struct TransformArgs {
     int iso;
 };
 
-size_t pair_smem_bytes(int mode);
+// Words (ints) behind the context's status word: the work counter, the active
+// problems and the finalize's chunks.
+constexpr int SRC_WORD_WORK = 16, SRC_WORD_ACTIVE = 17, SRC_WORD_CHUNKS = 18;
+
+// Everything k_src_one takes and writes for a single problem (srcone.cu).
+constexpr int64_t SRC_ONE_MAX = 65536;
+struct SrcOneArgs {
+    const float *xyz, *cov, *feat;   // SoA source, device
+    int n, feat_dim, iso;
+    float inv_hf;
+    GridDev grid;
+    double T[12];                    // initial pose
+    double cutoff, sigma2, iso_ell;
+    double half_diag;                // half the diagonal of the grid's box
+    int sub, level;                  // schedule of the work items
+    unsigned *words;                 // 64 words: status, SRC_WORD_*
+    ProbDev *prob;
+    GridDev *grid_out;
+    float4 *spos, *sca, *scb, *sfx;  // packed records (sfx, tfx: null up to 3 feature channels)
+    float4 *tpos, *tca, *tcb, *tlo, *tfx;
+    unsigned long long *keys;        // sorted codes (may be null)
+    int *tmp;                        // n ints
+    int *items, *item_prob, *n_items;
+};
+gcvo_status launch_src_one(const SrcOneArgs &a, cudaStream_t s);
+
 // sub: points per sub-tile (4, 8, 16, 32).
 int pair_sub_for(int mode, int sub);
 int pair_blocks_per_sm(int mode, bool iso, int fd, int sub);
