@@ -22,7 +22,7 @@
 // sizes (11 of 32 active) through a hash table rebuilt for three voxel sizes,
 // with a read-back between, and 64-bit Jacobi sweeps on a GPU with 2 FP64
 // results per SM and cycle.  Covariances of a 20,000-point LiDAR frame: 1824
-// -> 228 us; of 32 clouds of 1,000 to 40,000 points: 3135 -> 1107 us.
+// -> 164 us; of 32 clouds of 1,000 to 40,000 points: 3135 -> 978 us.
 #include <algorithm>
 #include <cstring>
 
@@ -308,35 +308,40 @@ __global__ void __launch_bounds__(KNN_WARPS * 32)
     int vox[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) vox[a] = knn_voxel(u[a], g.bits);
-    // the smallest cell of the point with knn more points to one side of it
+    // the smallest cell of the point with two thirds of knn more points to
+    // one side of it: on surfaces the block around it then holds 95 to 130
+    // points, and 3 to 8 points in 100 need a larger one (knn points to one
+    // side: 130 to 155 and 1 to 3; half of knn: 90 to 115 and 10 to 20)
     int L = max(g.bits, 1);
     {
         const unsigned long long k0 = code[me];
+        const int away = (2 * knn + 2) / 3;
 #pragma unroll
         for (int s = -1; s <= 1; s += 2) {
-            const int o = me + s * knn;
+            const int o = me + s * away;
             if (o >= 0 && o < n) L = min(L, (66 - __clzll((long long)(k0 ^ code[o]))) / 3);
         }
         L = max(L, 1);
     }
     KnnEntry best{~0ull, 0};
     for (;; ++L) {
-        // lanes 0..7: first places of the 2 x 2 x 2 cells; lanes 8..15: their ends
+        // lanes 0..7: first places of the 2 x 2 x 2 cells, the point's own
+        // first (it holds the nearest points, and the list soon turns the
+        // others' away); lanes 8..15: their ends
         const int cells = L >= g.bits ? 1 : 1 << (g.bits - L);
-        int i0[3];
+        int cell[3];
         float reach = INFINITY;
+        bool inside = lane < 16;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            i0[a] = ((vox[a] >> (L - 1)) - 1) >> 1;
-            if (i0[a] > 0) reach = fminf(reach, u[a] - (float)(i0[a] << L));
-            if (i0[a] + 2 < cells) reach = fminf(reach, (float)((i0[a] + 2) << L) - u[a]);
+            const int i0 = ((vox[a] >> (L - 1)) - 1) >> 1, own = (vox[a] >> L) - i0;
+            if (i0 > 0) reach = fminf(reach, u[a] - (float)(i0 << L));
+            if (i0 + 2 < cells) reach = fminf(reach, (float)((i0 + 2) << L) - u[a]);
+            cell[a] = i0 + ((lane >> a & 1) ^ own);
+            inside = inside && cell[a] >= 0 && cell[a] < cells;
         }
         int end = 0;
-        if (lane < 16) {
-            const int cx = i0[0] + (lane & 1), cy = i0[1] + (lane >> 1 & 1), cz = i0[2] + (lane >> 2 & 1);
-            if (cx >= 0 && cy >= 0 && cz >= 0 && cx < cells && cy < cells && cz < cells)
-                end = lower_bound(code, n, (morton(cx, cy, cz) + (lane >> 3)) << (3 * L));
-        }
+        if (inside) end = lower_bound(code, n, (morton(cell[0], cell[1], cell[2]) + (lane >> 3)) << (3 * L));
         const int last = __shfl_down_sync(FULL, end, 8);
         const int len = lane < 8 ? last - end : 0;
         // inclusive sums of the runs' lengths in lanes 0..7
