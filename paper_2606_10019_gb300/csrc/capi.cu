@@ -754,6 +754,8 @@ gcvo_status capture_chunk(gcvo_ctx *ctx, const Prepared &P, IterBufs &b, int ord
     return GCVO_OK;
 }
 
+constexpr int LOOP_ITERS = 512;
+
 gcvo_status run_register(gcvo_ctx *ctx, int np, const gcvo_problem *pr, const gcvo_solver_params *sp,
                          double *T_out, gcvo_iter_log *logs, int *n_iter, int *status) {
     if (!sp || !T_out || sp->order < 1 || sp->order > 3 || sp->k_max < 1 || sp->k_max > GCVO_MAX_KMAX ||
@@ -778,21 +780,44 @@ gcvo_status run_register(gcvo_ctx *ctx, int np, const gcvo_problem *pr, const gc
     void *hp;
     GCVO_TRY(host_pinned(ctx, 64, &hp));
     int *h_active = static_cast<int *>(hp);
-    // U iterations per host check, replayed from one CUDA graph.  Iterations
-    // past a problem's convergence or k_max leave it untouched (the finalize
-    // skips inactive problems, the pair kernel their items).
-    const int U = std::min(8, sp->k_max);
-    ChunkGraph cg;
-    GCVO_TRY(capture_chunk(ctx, P, b, sp->order, U, cg));
-    int it = 0;
-    while (it < sp->k_max) {
-        GCVO_CUDA(cudaGraphLaunch(cg.exec, s));
-        count_launches(cg.kernels);
-        it += U;
-        GCVO_CUDA(cudaMemcpyAsync(h_active, n_active, sizeof(int), cudaMemcpyDeviceToHost, s));
-        GCVO_CUDA(cudaStreamSynchronize(s));
-        GCVO_TRY(collect_profile(ctx, true));
-        if (*h_active <= 0) break;
+    if (sp->order == 2 && !ctx->profiling) {
+        // the whole loop in one cooperative kernel (loop.cu), LOOP_ITERS
+        // iterations at most before the host looks again
+        LoopArgs la{};
+        la.pair = b.pa;
+        la.fin = b.fa;
+        la.fin.mode = FIN_GN;
+        la.tr = b.ta;
+        la.barrier = ctx->status_word.as<unsigned>() + SRC_WORD_BARRIER;
+        // one warp per work item, of which there are up to about twice as
+        // many as full ones; more blocks only lengthen the barriers
+        const int blocks = (int)std::min<int64_t>(1 << 20, (2 * P.n_points / b.sub + PAIR_WARPS - 1) / PAIR_WARPS);
+        for (int it = 0; it < sp->k_max; it += LOOP_ITERS) {
+            la.max_iters = std::min(LOOP_ITERS, sp->k_max - it);
+            if (it > 0) GCVO_CUDA(cudaMemsetAsync(la.barrier, 0, sizeof(unsigned), s));
+            GCVO_CUDA(launch_loop(la, P.iso, P.feat_dim, b.sub, blocks, std::max(1, ctx->sm_count), s));
+            if (it + LOOP_ITERS >= sp->k_max) break;
+            GCVO_CUDA(cudaMemcpyAsync(h_active, n_active, sizeof(int), cudaMemcpyDeviceToHost, s));
+            GCVO_CUDA(cudaStreamSynchronize(s));
+            if (*h_active <= 0) break;
+        }
+    } else {
+        // U iterations per host check, replayed from one CUDA graph.
+        // Iterations past a problem's convergence or k_max leave it untouched
+        // (the finalize skips inactive problems, the pair kernel their items).
+        const int U = std::min(8, sp->k_max);
+        ChunkGraph cg;
+        GCVO_TRY(capture_chunk(ctx, P, b, sp->order, U, cg));
+        int it = 0;
+        while (it < sp->k_max) {
+            GCVO_CUDA(cudaGraphLaunch(cg.exec, s));
+            count_launches(cg.kernels);
+            it += U;
+            GCVO_CUDA(cudaMemcpyAsync(h_active, n_active, sizeof(int), cudaMemcpyDeviceToHost, s));
+            GCVO_CUDA(cudaStreamSynchronize(s));
+            GCVO_TRY(collect_profile(ctx, true));
+            if (*h_active <= 0) break;
+        }
     }
     ctx->ev_used = 0;
     GCVO_TRY(check_status_word(ctx));

@@ -39,16 +39,17 @@ constexpr size_t NA_IPROB = NA_ITEMS + al256(NA_MAX_ITEMS * 4);
 constexpr size_t NA_PART = NA_IPROB + al256(NA_MAX_ITEMS * 4);
 constexpr size_t NA_COUNTS = NA_PART + al256((size_t)NA_MAX_ITEMS * 64 * 4);
 constexpr size_t NA_CHUNK_ROWS = NA_MAX_ITEMS / FIN_CHUNK + 2;
-constexpr size_t NA_CHUNK = NA_COUNTS + al256((size_t)NA_MAX_ITEMS * 4 * 8);
+// the finalize's chunk rows lie over the tails, which only the pair pass before it reads
+constexpr size_t NA_CHUNK = NA_TLO;
 constexpr size_t NA_CHUNKCNT = NA_CHUNK + al256(NA_CHUNK_ROWS * 64 * 8);
-constexpr size_t NA_PROB = NA_CHUNKCNT + al256(NA_CHUNK_ROWS * 4 * 8);
+static_assert(NA_CHUNKCNT + al256(NA_CHUNK_ROWS * 4 * 8) <= NA_ITEMS, "the chunk rows fit over the tails");
+constexpr size_t NA_PROB = NA_COUNTS + al256((size_t)NA_MAX_ITEMS * 4 * 8);
 constexpr size_t NA_GRID = NA_PROB + al256(sizeof(ProbDev));
 constexpr size_t NA_EVAL = NA_GRID + al256(sizeof(GridDev));
 constexpr size_t NA_WORDS = NA_EVAL + al256(sizeof(EvalOut));   // work, n_items, lam, status, n_active, n_chunks
 constexpr size_t NA_BYTES = NA_WORDS + 256;
 // 4 MiB of source records and position tails, 2 MiB of partials, 256 KiB of
-// counters, 64 KiB of work items and 18 KiB of finalize chunk sums: the
-// 6.3 MiB the header documents
+// counters and 64 KiB of work items: the 6.3 MiB the header documents
 static_assert(NA_BYTES >= size_t(6300) * 1048576 / 1000 && NA_BYTES <= size_t(6350) * 1048576 / 1000,
               "the documented size of the static scratch (6.3 MiB)");
 

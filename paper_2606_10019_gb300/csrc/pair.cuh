@@ -83,9 +83,9 @@ struct PairArgs {
 // items of one problem) into one FP64 row; the block that finishes a
 // problem's last chunk adds its rows in order and takes the FP64 step.  The
 // chunk rows depend only on the problem's own items, so a problem's result
-// does not depend on the rest of the batch.  128 items are 16 per warp, two
-// rounds of loads; 20,000 source points still make 20 to 40 chunks.
-constexpr int FIN_CHUNK = 128;
+// does not depend on the rest of the batch.  64 items are 16 per warp, one
+// round of loads; 20,000 source points make 40 to 80 chunks.
+constexpr int FIN_CHUNK = 64;
 
 // Bytes of the chunk rows for at most n_items work items over np problems.
 inline size_t fin_chunk_bytes(int64_t n_items, int np) {
@@ -147,8 +147,8 @@ struct TransformArgs {
 };
 
 // Words (ints) behind the context's status word: the work counter, the active
-// problems and the finalize's chunks.
-constexpr int SRC_WORD_WORK = 16, SRC_WORD_ACTIVE = 17, SRC_WORD_CHUNKS = 18;
+// problems, the finalize's chunks and the register loop's barrier.
+constexpr int SRC_WORD_WORK = 16, SRC_WORD_ACTIVE = 17, SRC_WORD_CHUNKS = 18, SRC_WORD_BARRIER = 19;
 
 // Everything k_src_one takes and writes for a single problem (srcone.cu).
 constexpr int64_t SRC_ONE_MAX = 65536;
@@ -176,6 +176,16 @@ gcvo_status launch_src_one(const SrcOneArgs &a, cudaStream_t s);
 int pair_sub_for(int mode, int sub);
 int pair_blocks_per_sm(int mode, bool iso, int fd, int sub);
 cudaError_t launch_pair(const PairArgs &a, int mode, bool iso, int fd, int sub, int grid, cudaStream_t s);
+// The register loop of G-CVO-2 (loop.cu): up to max_iters iterations, or until
+// no problem is active, in one cooperative launch of at most `blocks` blocks.
+struct LoopArgs {
+    PairArgs pair;
+    FinalizeArgs fin;
+    TransformArgs tr;
+    unsigned *barrier;   // zero before the launch
+    int max_iters;
+};
+cudaError_t launch_loop(const LoopArgs &a, bool iso, int fd, int sub, int blocks, int sm_count, cudaStream_t s);
 cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t s);
 cudaError_t launch_src_keys(const SrcArgs &a, int n_problems, int64_t max_n, cudaStream_t s);
 cudaError_t launch_src_pack(const SrcArgs &a, const unsigned long long *keys, int64_t n, cudaStream_t s);

@@ -124,4 +124,25 @@ __device__ __forceinline__ void transform_point(const Prob *P, float4 z, float4 
     tcb = make_float4(q[4], q[5], sg * zb.z, sg * zb.w);
 }
 
+// The transform for every point of the active problems.
+__device__ __forceinline__ void transform_points(const TransformArgs &a, int block, int blocks) {
+    const int64_t stride = (int64_t)blocks * blockDim.x;
+    for (int64_t i = (int64_t)block * blockDim.x + threadIdx.x; i < a.n; i += stride) {
+        const ProbDev *P = a.probs + (a.pprob ? a.pprob[i] : 0);
+        if (P->status != 0) continue;   // converged or failed: left as it was
+        const float4 za = a.iso ? make_float4(0.f, 0.f, 0.f, 0.f) : a.sca[i];
+        float4 tp, tl, ta, tb;
+        transform_point(P, a.spos[i], za, a.scb[i], a.iso != 0, tp, tl, ta, tb);
+        a.tpos[i] = tp;
+        if (a.tlo) a.tlo[i] = tl;
+        a.tca[i] = ta;
+        a.tcb[i] = tb;
+        if (a.tfx) {
+            const float4 f = a.sfx[i];
+            const float sg = P->sigma2;
+            a.tfx[i] = make_float4(sg * f.x, sg * f.y, sg * f.z, sg * f.w);
+        }
+    }
+}
+
 }  // namespace gcvo
