@@ -756,6 +756,20 @@ gcvo_status capture_chunk(gcvo_ctx *ctx, const Prepared &P, IterBufs &b, int ord
 
 constexpr int LOOP_ITERS = 512;
 
+// Whether the register loop's kernel may take these problems.  Its barriers
+// wait for the slowest block's pair pass, at most LOOP_SPINS polls of about 0.7
+// us (loop.cu), so the pass has to be short against that even when every pair
+// is evaluated: 2^39 pairs take 2 s (2.8e11 pairs/s on dense clouds; 5 s with 7
+// feature channels).  Larger sets, whose passes dwarf the launches, replay the
+// graphs, where nothing waits; 64 pairs of 40,000-point clouds are 2^37.
+constexpr double LOOP_MAX_PAIRS = 549755813888.0;
+
+bool loop_fits(int np, const gcvo_problem *pr) {
+    double pairs = 0.0;
+    for (int p = 0; p < np; ++p) pairs += (double)pr[p].n_src * (double)pr[p].target->store.d.n;
+    return pairs <= LOOP_MAX_PAIRS;
+}
+
 gcvo_status run_register(gcvo_ctx *ctx, int np, const gcvo_problem *pr, const gcvo_solver_params *sp,
                          double *T_out, gcvo_iter_log *logs, int *n_iter, int *status) {
     if (!sp || !T_out || sp->order < 1 || sp->order > 3 || sp->k_max < 1 || sp->k_max > GCVO_MAX_KMAX ||
@@ -780,7 +794,7 @@ gcvo_status run_register(gcvo_ctx *ctx, int np, const gcvo_problem *pr, const gc
     void *hp;
     GCVO_TRY(host_pinned(ctx, 64, &hp));
     int *h_active = static_cast<int *>(hp);
-    if (sp->order == 2 && !ctx->profiling) {
+    if (sp->order == 2 && !ctx->profiling && loop_fits(np, pr)) {
         // the whole loop in one cooperative kernel (loop.cu), LOOP_ITERS
         // iterations at most before the host looks again
         LoopArgs la{};

@@ -79,3 +79,19 @@ def test_batch_and_long_loop(env):
                 assert a[2][:-1].max() == k_max
     finally:
         G.gcvo_pair_schedule(ctx, 0)
+
+
+def test_large_sets_replay_the_graphs(env):
+    """More than 2^39 pairs in all (copies of one problem): kernels of their own, and the same poses."""
+    G, ctx, dev = env
+    prob = _problem(G, ctx, dev, 60000, 3)
+    copies = int(2.0 ** 39 // (60000 * 54000)) + 1
+    sp = G.solver_params(k_max=3, eps_tol=1e-12)
+    try:
+        G.gcvo_pair_schedule(ctx, 8)
+        one = G.gcvo_register(ctx, *prob, sp)
+        many = G.gcvo_register_batched(ctx, [prob] * copies, sp)
+    finally:
+        G.gcvo_pair_schedule(ctx, 0)
+    assert all(np.array_equal(T, one[0]) for T in many[0])
+    assert set(many[2]) == {one[2]} and set(many[3]) == {one[3]}
