@@ -439,16 +439,83 @@ __global__ void __launch_bounds__(KNN_WARPS * 32)
     if (lane < 6) c.cov[(int64_t)lane * n + __float_as_int(q.w)] = s * (1.0f / (float)(knn - 1));
 }
 
+// Whether every off-diagonal entry of A' has E_pq^2 <= 2e-9 top |d_p - d_q|, top
+// the largest clamped eigenvalue.
+__device__ __forceinline__ bool eig_converged(const double d[3], double e01, double e02, double e12, double top) {
+    const float i = 1.0f / (float)top;
+    const float a = (float)e01 * i, b = (float)e02 * i, c = (float)e12 * i;
+    return a * a <= 2e-9f * fabsf((float)(d[0] - d[1]) * i) && b * b <= 2e-9f * fabsf((float)(d[0] - d[2]) * i) &&
+           c * c <= 2e-9f * fabsf((float)(d[1] - d[2]) * i);
+}
+
+// Turns V until A' = V^T A V passes eig_converged, by sweeps of Jacobi's method
+// in FP64; d and e: the diagonal of A' and its entries 01, 02, 12.  An angle is
+// as good as FP32 makes it, which leaves 1e-7 of an entry, but its cosine and
+// sine belong together to FP64 rounding (Newton steps), and V is made
+// orthonormal again before every A'.
+__device__ __noinline__ void eig_refine(const float *s, double lo, double hi, double (*V)[3], double *d, double *e) {
+    const double A[3][3] = {{s[0], s[1], s[2]}, {s[1], s[3], s[4]}, {s[2], s[4], s[5]}};
+    for (int sweep = 0;; ++sweep) {
+        double G[3][3], B[3][3], a[3][3];
+        for (int p = 0; p < 3; ++p)
+            for (int q = 0; q < 3; ++q)
+                G[p][q] = (p == q ? 1.5 : 0.0) - 0.5 * (V[0][p] * V[0][q] + V[1][p] * V[1][q] + V[2][p] * V[2][q]);
+        for (int r = 0; r < 3; ++r)
+            for (int q = 0; q < 3; ++q) B[r][q] = V[r][0] * G[0][q] + V[r][1] * G[1][q] + V[r][2] * G[2][q];
+        for (int r = 0; r < 3; ++r)
+            for (int q = 0; q < 3; ++q) {
+                V[r][q] = B[r][q];
+                G[r][q] = A[r][0] * B[0][q] + A[r][1] * B[1][q] + A[r][2] * B[2][q];
+            }
+        for (int p = 0; p < 3; ++p)
+            for (int q = p; q < 3; ++q) a[p][q] = a[q][p] = B[0][p] * G[0][q] + B[1][p] * G[1][q] + B[2][p] * G[2][q];
+        double top = lo;
+        for (int p = 0; p < 3; ++p) {
+            d[p] = a[p][p];
+            top = fmax(top, fmin(d[p], hi));
+        }
+        e[0] = a[0][1];
+        e[1] = a[0][2];
+        e[2] = a[1][2];
+        if (sweep == 8 || (sweep > 0 && eig_converged(d, e[0], e[1], e[2], top))) return;
+        for (int k = 0; k < 3; ++k) {
+            const int p = k == 2 ? 1 : 0, q = k == 0 ? 1 : 2, r = 3 - p - q;
+            const float den = 2.0f * (float)a[p][q];
+            if (den == 0.f) continue;
+            const float tau = (float)(a[q][q] - a[p][p]) / den;
+            const double t = copysignf(1.0f, tau) / (fabsf(tau) + sqrtf(1.0f + tau * tau)), u = 1.0 + t * t;
+            double c = rsqrtf((float)u);
+            c = c * (1.5 - 0.5 * u * c * c);
+            c = c * (1.5 - 0.5 * u * c * c);
+            const double sn = t * c, app = a[p][p], aqq = a[q][q], apq = a[p][q], arp = a[r][p], arq = a[r][q];
+            a[p][p] = c * c * app - 2.0 * c * sn * apq + sn * sn * aqq;
+            a[q][q] = sn * sn * app + 2.0 * c * sn * apq + c * c * aqq;
+            a[p][q] = a[q][p] = c * sn * (app - aqq) + (c * c - sn * sn) * apq;
+            a[r][p] = a[p][r] = c * arp - sn * arq;
+            a[r][q] = a[q][r] = sn * arp + c * arq;
+            for (int m = 0; m < 3; ++m) {
+                const double vp = V[m][p], vq = V[m][q];
+                V[m][p] = c * vp - sn * vq;
+                V[m][q] = sn * vp + c * vq;
+            }
+        }
+    }
+}
+
 // Clamps the eigenvalues of every covariance to [eig_max / eig_ratio,
 // eig_max].  FP64 sweeps of Jacobi's method would be most of the time
 // (about 1500 FP64 operations per point, at 2 per SM and cycle), so the
 // eigenvectors come from FP32 sweeps and FP64 only corrects them: with V the
-// FP32 vectors made orthonormal to 1e-14 by one Newton step, A' = V^T A V is
-// diagonal up to E of about 1e-7 of the largest eigenvalue, and to first
+// FP32 vectors made orthonormal to about 1e-13 by one Newton step, A' = V^T A V
+// is diagonal up to E of about 1e-7 of the largest eigenvalue, and to first
 // order in E (the Daleckii-Krein formula) the clamped matrix f(A') has f of
 // the diagonal and E_pq (f(d_p) - f(d_q)) / (d_p - d_q) beside it: about 150
-// FP64 operations.  The clamp is linear between its bounds, where that is
-// exact; what remains is of order E^2, below the float result's rounding.
+// FP64 operations.  The terms left out are E_pr E_rq times a second divided
+// difference of f, which is at most the inverse of the largest gap among its
+// three eigenvalues.  eig_converged keeps them below 4e-9 of the result's
+// largest eigenvalue, a fifteenth of a float's rounding.  Points that miss it
+// (elongated neighbourhoods: with the largest eigenvalue 1e4 times eig_max the
+// formula alone was off by 4e-5) go through eig_refine; surfaces do not.
 __global__ void __launch_bounds__(128) k_knn_eig(const KnnCloud *cl, const int *cloud, int64_t N, const unsigned *status) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= N || (*status & DEV_ERR_NONFINITE)) return;
@@ -507,26 +574,47 @@ __global__ void __launch_bounds__(128) k_knn_eig(const KnnCloud *cl, const int *
     const double A[3][3] = {{s[0], s[1], s[2]}, {s[1], s[3], s[4]}, {s[2], s[4], s[5]}};
     double F[3][3];   // f(A')
     {
-        double AV[3][3], d[3], f[3];
+        double AV[3][3], d[3], e[3], f[3];
 #pragma unroll
         for (int r = 0; r < 3; ++r)
 #pragma unroll
             for (int q = 0; q < 3; ++q) AV[r][q] = A[r][0] * V[0][q] + A[r][1] * V[1][q] + A[r][2] * V[2][q];
         const double lo = c.eig_max / c.eig_ratio;
+        double top = lo, largest = 0.0;
 #pragma unroll
         for (int p = 0; p < 3; ++p) {
             d[p] = V[0][p] * AV[0][p] + V[1][p] * AV[1][p] + V[2][p] * AV[2][p];
-            f[p] = fmin(fmax(d[p], lo), c.eig_max);
-            F[p][p] = f[p];
+            top = fmax(top, fmin(d[p], c.eig_max));
+            largest = fmax(largest, d[p]);
         }
 #pragma unroll
         for (int p = 0; p < 3; ++p)
 #pragma unroll
+            for (int q = p + 1; q < 3; ++q)
+                e[p + q - 1] = V[0][p] * AV[0][q] + V[1][p] * AV[1][q] + V[2][p] * AV[2][q];
+        // V's own 1e-13 of the largest eigenvalue counts beyond 1e4 times the clamp
+        if (!eig_converged(d, e[0], e[1], e[2], top) || (float)largest > 1e4f * (float)top) {
+            double Vr[3][3], dr[3], er[3];
+#pragma unroll
+            for (int r = 0; r < 9; ++r) Vr[r / 3][r % 3] = V[r / 3][r % 3];
+            eig_refine(s, lo, c.eig_max, Vr, dr, er);
+#pragma unroll
+            for (int r = 0; r < 9; ++r) V[r / 3][r % 3] = Vr[r / 3][r % 3];
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+                d[p] = dr[p];
+                e[p] = er[p];
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < 3; ++p) F[p][p] = f[p] = fmin(fmax(d[p], lo), c.eig_max);
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
             for (int q = p + 1; q < 3; ++q) {
-                const double E = V[0][p] * AV[0][q] + V[1][p] * AV[1][q] + V[2][p] * AV[2][q];
                 const float gap = (float)(d[p] - d[q]);
                 const float slope = gap != 0.f ? (float)(f[p] - f[q]) / gap : (d[p] == f[p] ? 1.f : 0.f);
-                F[p][q] = F[q][p] = E * (double)slope;
+                F[p][q] = F[q][p] = e[p + q - 1] * (double)slope;
             }
     }
     double VF[3][3];
