@@ -467,13 +467,22 @@ __device__ __forceinline__ bool tile_pass(const PairArgs &a, StageT<MODE, FD> *s
         // a target whose farthest corner of the box is nearer than this is
         // within rho of every point: r is formed from the same heads, and the
         // tails move it by less than 2^-22 of the largest coordinate
-        float rin2 = -1.f;
+        float rin2 = -1.f, lam_box = lam_sub;
         if (two_lists) {
             float mag = rho;
 #pragma unroll
             for (int k = 0; k < 3; ++k) mag = fmaxf(mag, fmaxf(-bmin[k], bmax[k]) + rho);
             const float ri = rho * 0.9999f - (dfr ? 1e-6f * mag : 0.f);
             rin2 = ri > 0.f ? ri * ri : -1.f;
+            if (dfr) {
+                // the per-pair limits are tested on heads too: a distance up to
+                // rho that the tails shorten by e has a square up to 2 rho e +
+                // e^2 larger there
+                const float e = 2.4e-7f * mag, s1 = e * (2.f * rho + e) / c2;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) dmax[k] += s1;
+                lam_box += 3.f * s1;
+            }
         }
         int lo[3], hi[3];
         bool empty = !(bmin[0] <= bmax[0]);
@@ -589,7 +598,7 @@ __device__ __forceinline__ bool tile_pass(const PairArgs &a, StageT<MODE, FD> *s
                             const float lam_j = sqrt_approx(ca.x * ca.x + ca.w * ca.w + cbv.y * cbv.y +
                                                             2.f * (ca.y * ca.y + ca.z * ca.z + cbv.x * cbv.x));
                             const float c2m = c2 * 1.01f, sl = c2 * 1e-5f * lam_j + 1e-12f;
-                            near = db2 <= c2 * (lam_sub + lam_j) * 1.001f + 1e-12f &&
+                            near = db2 <= c2 * (lam_box + lam_j) * 1.001f + 1e-12f &&
                                    dx * dx <= c2m * (dmax[0] + ca.x) + sl && dyy * dyy <= c2m * (dmax[1] + ca.w) + sl &&
                                    dz * dz <= c2m * (dmax[2] + cbv.y) + sl;
                         }
