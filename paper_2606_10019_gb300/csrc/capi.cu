@@ -468,6 +468,20 @@ gcvo_status pack(gcvo_ctx *ctx, const Prepared &P, int sched) {
                       ctx->scan_tmp.ptr, ctx->stream);
 }
 
+gcvo_status status_of_word(unsigned w) {
+    if (w & DEV_ERR_TIMEOUT) return GCVO_ERR_TIMEOUT;
+    if (w & DEV_ERR_CAPACITY) return GCVO_ERR_CAPACITY;
+    if (w & DEV_ERR_NONFINITE) return GCVO_ERR_NONFINITE;
+    return GCVO_OK;
+}
+
+gcvo_status check_status_word(gcvo_ctx *ctx) {
+    unsigned w = 0;
+    GCVO_CUDA(cudaMemcpyAsync(&w, ctx->status_word.ptr, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream));
+    GCVO_CUDA(cudaStreamSynchronize(ctx->stream));
+    return status_of_word(w);
+}
+
 // The autotuner: the schedule for this shape of problem set -- a forced
 // one, the cached choice for the same shape, or the fastest of one timed
 // evaluation pass with each candidate (the second of two, CUDA events).
@@ -476,6 +490,9 @@ gcvo_status choose_schedule(gcvo_ctx *ctx, const Prepared &P, IterBufs &b) {
     int packed = P.one ? P.sched : 0;
     {
         if (!sched) {
+            // a single problem has had nothing read back: with a non-finite input
+            // its passes do no work, and must not decide the schedule of later calls
+            if (P.one) GCVO_TRY(check_status_word(ctx));
             constexpr int NC = 9;
             const int cands[NC] = {4 | 2 << 8,  8 | 2 << 8,  16 | 2 << 8, 32 | 2 << 8, 8 | 3 << 8,
                                    16 | 3 << 8, 32 | 3 << 8, 4 | 1 << 8,  8 | 1 << 8};
@@ -598,20 +615,6 @@ gcvo_status iter_bufs(gcvo_ctx *ctx, const Prepared &P, IterBufs &b, gcvo_iter_l
         GCVO_CUDA(launch_transform(t, ctx->stream));
     }
     return choose_schedule(ctx, P, b);
-}
-
-gcvo_status status_of_word(unsigned w) {
-    if (w & DEV_ERR_TIMEOUT) return GCVO_ERR_TIMEOUT;
-    if (w & DEV_ERR_CAPACITY) return GCVO_ERR_CAPACITY;
-    if (w & DEV_ERR_NONFINITE) return GCVO_ERR_NONFINITE;
-    return GCVO_OK;
-}
-
-gcvo_status check_status_word(gcvo_ctx *ctx) {
-    unsigned w = 0;
-    GCVO_CUDA(cudaMemcpyAsync(&w, ctx->status_word.ptr, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream));
-    GCVO_CUDA(cudaStreamSynchronize(ctx->stream));
-    return status_of_word(w);
 }
 
 // With profiling on, a timed launch is bracketed by two events from the
