@@ -28,6 +28,7 @@
 
 #include "common.cuh"
 #include "csort.cuh"
+#include "perdevice.cuh"
 
 namespace gcvo {
 namespace {
@@ -643,8 +644,8 @@ cudaError_t knn_sort_attr() {
 template <int ITEMS>
 gcvo_status launch_knn_sort(const KnnCloud *cl, const int *ids, int n_clouds, int blocks, KnnGrid *grids,
                             unsigned long long *code, float4 *pos, int *cloud, unsigned *status, cudaStream_t s) {
-    static const cudaError_t attr = knn_sort_attr<ITEMS>();
-    GCVO_CUDA(attr);
+    static PerDevice<cudaError_t> attr;
+    GCVO_CUDA(attr.get(knn_sort_attr<ITEMS>));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(blocks * n_clouds));
     cfg.blockDim = dim3(csort::THREADS);

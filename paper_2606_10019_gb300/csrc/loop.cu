@@ -22,6 +22,7 @@
 #include "common.cuh"
 #include "fin.cuh"
 #include "pair.cuh"
+#include "perdevice.cuh"
 #include "srcdev.cuh"
 #include "tile.cuh"
 
@@ -82,14 +83,15 @@ __global__ void __launch_bounds__(PAIR_WARPS * 32, 5) k_loop(LoopArgs a) {
 template <bool ISO, int FD, int SUB>
 cudaError_t launch_t(const LoopArgs &a, int blocks, int sm_count, cudaStream_t s) {
     constexpr size_t smem = tile_smem_bytes<PAIR_EVAL, FD>();
-    static int per_sm = 0;
-    static const cudaError_t setup = [] {
+    static PerDevice<std::pair<cudaError_t, int>> setup;
+    const auto [err, per_sm] = setup.get([] {
+        int n = 0;
         cudaError_t e = cudaFuncSetAttribute(k_loop<ISO, FD, SUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_loop<ISO, FD, SUB>, PAIR_WARPS * 32, smem);
-        return e;
-    }();
-    if (setup != cudaSuccess) return setup;
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_loop<ISO, FD, SUB>, PAIR_WARPS * 32, smem);
+        return std::make_pair(e, n);
+    });
+    if (err != cudaSuccess) return err;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)std::max(1, std::min(blocks, std::max(1, per_sm) * sm_count)));
     cfg.blockDim = dim3(PAIR_WARPS * 32);

@@ -7,6 +7,7 @@
 
 #include "common.cuh"
 #include "csort.cuh"
+#include "perdevice.cuh"
 
 namespace gcvo {
 
@@ -292,8 +293,8 @@ cudaError_t cluster_sort_attr() {
 
 template <int ITEMS>
 gcvo_status cluster_sort_t(unsigned long long *keys, int *vals, int n, int bits, int blocks, cudaStream_t s) {
-    static const cudaError_t attr = cluster_sort_attr<ITEMS>();
-    GCVO_CUDA(attr);
+    static PerDevice<cudaError_t> attr;
+    GCVO_CUDA(attr.get(cluster_sort_attr<ITEMS>));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(csort::THREADS);

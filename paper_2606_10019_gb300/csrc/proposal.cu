@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "perdevice.cuh"
 #include "ptx.cuh"
 
 namespace gcvo {
@@ -1049,9 +1050,10 @@ gcvo_status forward_batch(gcvo_ctx *ctx, gcvo_proposal *P, int B, int n, const f
     }
     prop::k_prep<<<B, prop::PREP_THREADS, 0, s>>>(n, sx, sf, sfs, tx, tf, tfs, P->pts.as<float4>(), P->cs.as<float>(),
                                                  d_label, P->label.as<float>());
-    static const cudaError_t attr = cudaFuncSetAttribute(
-        prop::k_point_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)prop::point_fwd_smem());
-    GCVO_CUDA(attr);
+    static PerDevice<cudaError_t> attr;
+    GCVO_CUDA(attr.get([] {
+        return cudaFuncSetAttribute(prop::k_point_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)prop::point_fwd_smem());
+    }));
     prop::Net net = net_of(P);
     auto *top = P->top.as<unsigned long long>();
     const int tiles = (n + prop::PT_TILE - 1) / prop::PT_TILE;
@@ -1221,9 +1223,11 @@ gcvo_status gcvo_proposal_train_step(gcvo_ctx *ctx, gcvo_proposal *P, int B, int
     const prop::HeadLayer l3{P->d_out.as<float>(), P->y2.as<float>(), g + off[prop::H3], g + off[prop::C3], 6, 128, 1};
     prop::k_head_grad<<<8 * 16 + 4 * 8 + 4, 256, 0, s>>>(B, l1, l2, l3);
     // two blocks fit on an SM; fewer when there are not that many units
-    static const cudaError_t bwd_attr = cudaFuncSetAttribute(
-        prop::k_point_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, prop::BW_SMEM_FLOATS * (int)sizeof(float));
-    GCVO_CUDA(bwd_attr);
+    static PerDevice<cudaError_t> bwd_attr;
+    GCVO_CUDA(bwd_attr.get([] {
+        return cudaFuncSetAttribute(prop::k_point_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    prop::BW_SMEM_FLOATS * (int)sizeof(float));
+    }));
     const int units = 2 * B * (256 / prop::BW_CH);
     prop::k_point_bwd<<<std::min(units, 2 * std::max(1, ctx->sm_count)), prop::BW_THREADS,
                         prop::BW_SMEM_FLOATS * sizeof(float), s>>>(net, n, units, P->pts.as<float4>(), P->arg.as<int>(),

@@ -18,6 +18,7 @@
 #include "common.cuh"
 #include "csort.cuh"
 #include "pair.cuh"
+#include "perdevice.cuh"
 #include "srcdev.cuh"
 
 namespace gcvo {
@@ -294,8 +295,8 @@ cudaError_t src_one_attr() {
 
 template <int ITEMS>
 gcvo_status launch_t(const SrcOneArgs &a, int blocks, cudaStream_t s) {
-    static const cudaError_t attr = src_one_attr<ITEMS>();
-    GCVO_CUDA(attr);
+    static PerDevice<cudaError_t> attr;
+    GCVO_CUDA(attr.get(src_one_attr<ITEMS>));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(csort::THREADS);

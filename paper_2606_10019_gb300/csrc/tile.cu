@@ -2,6 +2,7 @@
 // packing of the work items that its warps take.
 #include "common.cuh"
 #include "pair.cuh"
+#include "perdevice.cuh"
 #include "tile.cuh"
 
 namespace gcvo {
@@ -90,12 +91,14 @@ __global__ void __launch_bounds__(CHUNK_THREADS) k_chunk_ranges(int np, ProbDev 
 // ---------------------------------------------------------------------------
 // Host launchers.
 // ---------------------------------------------------------------------------
-// The opt-in above the 48 KB default, made once per kernel instance.
+// The opt-in above the 48 KB default, made once per kernel instance and device.
 template <int MODE, bool ISO, int FD, int SUB>
 static cudaError_t tile_smem_optin() {
-    static const cudaError_t once = cudaFuncSetAttribute(
-        k_tile<MODE, ISO, FD, SUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_smem_bytes<MODE, FD>());
-    return once;
+    static PerDevice<cudaError_t> once;
+    return once.get([] {
+        return cudaFuncSetAttribute(k_tile<MODE, ISO, FD, SUB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)tile_smem_bytes<MODE, FD>());
+    });
 }
 
 template <int MODE, bool ISO, int FD, int SUB>

@@ -1,0 +1,86 @@
+"""What the library's host code asks of the CUDA runtime, against a stand-in for
+it that runs no kernel (fake_cudart.cpp): the library's objects are linked with
+the stand-in and called in a process of their own."""
+import glob
+import json
+import os
+import subprocess
+import sys
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+CHILD = r"""
+import ctypes, json, sys
+import numpy as np
+import torch
+sys.path.insert(0, sys.argv[1])
+from paper_2606_10019_gb300 import gcvo as G
+G.LIB_PATH = sys.argv[2]
+L = G.lib()
+L.fake_log.restype = ctypes.c_char_p
+
+
+def log():
+    out = [l.split() for l in L.fake_log().decode().splitlines()]
+    L.fake_clear()
+    return [(int(d), name, int(grid), int(cluster)) for d, name, grid, cluster in out]
+
+
+def cloud(n):
+    return np.random.default_rng(n).normal(size=(3, n)).astype(np.float32)
+
+
+def problem(ctx, n_src, n_tgt, feat=1, **kw):
+    kp = G.kernel_params(eig_max=0.01, feat_dim=feat, cell_size=1.0, **kw)
+    cov = lambda n: np.tile(np.float32([1, 0, 0, 1, 0, 1])[:, None], n)
+    f = lambda n: np.ones((feat, n), np.float32)
+    return G.gcvo_build_grid(ctx, cloud(n_tgt), cov(n_tgt), f(n_tgt), kp), cloud(n_src), cov(n_src), f(n_src), np.eye(4)
+
+
+"""
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    from paper_2606_10019_gb300 import build as B
+    lib = B.build()
+    out = str(tmp_path_factory.mktemp("fake") / "libgcvo_fake.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(B._nvcc()))), "include")
+    objs = glob.glob(os.path.join(os.path.dirname(lib), "*.o"))
+    r = subprocess.run(["g++", "-shared", "-fPIC", "-O1", "-Wl,-Bsymbolic", "-I", cuda, "-o", out, os.path.join(HERE, "fake_cudart.cpp")] + objs,
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-3000:]
+
+    def run(code):
+        r = subprocess.run([sys.executable, "-c", CHILD + code, ROOT, out], capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stderr[-3000:]
+        return json.loads(r.stdout.splitlines()[-1])
+
+    return run
+
+
+def test_every_device_is_set_up(fake):
+    """Kernels with more shared memory or larger clusters than the default on the second device used in a process."""
+    out = fake(r"""
+res = []
+for d in (0, 1):
+    ctx = G.gcvo_create(d)
+    for n in (1500, 5000, 9000, 20000, 40000, 70000):
+        G.gcvo_estimate_covariances(ctx, cloud(n), G.kernel_params(eig_max=0.01), np.zeros((6, n), np.float32))
+    for feat in (1, 7):
+        for n in (1500, 20000):
+            p = problem(ctx, n, 1600, feat)
+            G.gcvo_eval(ctx, *p)
+            G.gcvo_eval_exact(ctx, *p)
+            for order in (1, 2, 3):
+                G.gcvo_register(ctx, *p, G.solver_params(order=order, k_max=3))
+    P = G.Proposal(ctx)
+    z, f = torch.zeros((2, 3, 300)), torch.zeros((2, 300))     # (the stand-in's device memory is host memory)
+    P.train_step(z, f, z, f, np.tile(np.eye(4), (2, 1, 1)), 1e-3)
+    res.append([x[1:] for x in log() if x[0] == d])
+print(json.dumps(res))
+""")
+    assert out[0] == out[1] and len(out[0]) > 100
