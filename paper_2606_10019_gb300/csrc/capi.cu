@@ -261,7 +261,7 @@ gcvo_status prepare(gcvo_ctx *ctx, int np, const gcvo_problem *pr, Prepared &P) 
     P.n_problems = np;
     P.iso = kp0.kernel_mode == 1;
     P.feat_dim = kp0.feat_dim;
-    if (np == 1 && pr[0].n_src <= SRC_ONE_MAX) return prepare_one(ctx, pr[0], P);
+    if (np == 1 && pr[0].n_src <= SRC_ONE_MAX && src_one_fits(pr[0].n_src)) return prepare_one(ctx, pr[0], P);
     // stage host inputs
     size_t need = 0;
     int64_t N = 0;

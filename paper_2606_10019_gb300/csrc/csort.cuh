@@ -20,6 +20,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "perdevice.cuh"
 
 namespace gcvo {
 namespace csort {
@@ -181,6 +182,41 @@ __device__ int sort(Smem<ITEMS> &S, int n, int bits) {
         cluster_barrier(nblk);
     }
     return cur;
+}
+
+// Opens a kernel with an Smem<ITEMS> to all clusters on the current device and
+// returns the sizes of which it can hold at least one (bit b: 2^b blocks).  A
+// partition with few SMs to a GPC may not place 8 or 16 blocks of 1024 threads;
+// the callers then take the grid-wide sort, and a single problem the batched
+// preparation.
+template <int ITEMS, class Kernel>
+unsigned cluster_sizes(Kernel kernel) {
+    unsigned sizes = 0;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem<ITEMS>)) == cudaSuccess &&
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+        for (int b = 0; 1 << b <= MAX_BLOCKS; ++b) {
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3(1u << b);
+            cfg.blockDim = dim3(THREADS);
+            cfg.dynamicSmemBytes = sizeof(Smem<ITEMS>);
+            cudaLaunchAttribute at{};
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = 1u << b;
+            at.val.clusterDim.y = at.val.clusterDim.z = 1;
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0) sizes |= 1u << b;
+        }
+    cudaGetLastError();   // a size that does not fit is no error
+    return sizes;
+}
+
+// The launch of a cluster of `blocks` blocks among those sizes.
+inline bool placed(unsigned sizes, int blocks) {
+    int b = 0;
+    while (1 << b < blocks) ++b;
+    return (sizes >> b & 1u) != 0;
 }
 
 // Keys per thread and blocks of a cluster for n keys (0 items: too many).

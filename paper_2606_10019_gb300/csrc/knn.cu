@@ -28,7 +28,6 @@
 
 #include "common.cuh"
 #include "csort.cuh"
-#include "perdevice.cuh"
 
 namespace gcvo {
 namespace {
@@ -212,7 +211,8 @@ __global__ void __launch_bounds__(csort::THREADS)
     }
 }
 
-// The steps of k_knn_sort for a cloud that no cluster holds: its box, its
+// The steps of k_knn_sort for a cloud that no cluster holds (or none that the
+// device can place): its box, its
 // codes, and after the grid-wide sort its points.
 __global__ void __launch_bounds__(256) k_knn_box(const KnnCloud *cl, int id, int *box) {
     __shared__ int red[8][KNN_BOX];
@@ -634,18 +634,23 @@ __global__ void __launch_bounds__(128) k_knn_eig(const KnnCloud *cl, const int *
 size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
 
 template <int ITEMS>
-cudaError_t knn_sort_attr() {
-    const cudaError_t e = cudaFuncSetAttribute(k_knn_sort<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)sizeof(csort::Smem<ITEMS>));
-    return e != cudaSuccess ? e
-                            : cudaFuncSetAttribute(k_knn_sort<ITEMS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+bool knn_sort_fits(int blocks) {
+    static PerDevice<unsigned> sizes;
+    return csort::placed(sizes.get([] { return csort::cluster_sizes<ITEMS>(k_knn_sort<ITEMS>); }), blocks);
+}
+
+bool knn_sort_fits(int items, int blocks) {
+    switch (items) {
+        case 1: return knn_sort_fits<1>(blocks);
+        case 2: return knn_sort_fits<2>(blocks);
+        case 4: return knn_sort_fits<4>(blocks);
+        default: return false;   // too many points
+    }
 }
 
 template <int ITEMS>
 gcvo_status launch_knn_sort(const KnnCloud *cl, const int *ids, int n_clouds, int blocks, KnnGrid *grids,
                             unsigned long long *code, float4 *pos, int *cloud, unsigned *status, cudaStream_t s) {
-    static PerDevice<cudaError_t> attr;
-    GCVO_CUDA(attr.get(knn_sort_attr<ITEMS>));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(blocks * n_clouds));
     cfg.blockDim = dim3(csort::THREADS);
@@ -697,7 +702,7 @@ gcvo_status knn_covariances(gcvo_ctx *ctx, int n_clouds, const KnnJob *jobs) {
         N += j.n;
         int items, blocks;
         csort::shape(j.n, items, blocks);
-        if (!items) {
+        if (!knn_sort_fits(items, blocks)) {
             large.push_back(c);
             n_large = std::max(n_large, j.n);
             continue;

@@ -170,6 +170,8 @@ struct SrcOneArgs {
     int *tmp;                        // n ints
     int *items, *item_prob, *n_items;
 };
+// Whether the current device can place the cluster for n points.
+bool src_one_fits(int64_t n);
 gcvo_status launch_src_one(const SrcOneArgs &a, cudaStream_t s);
 
 // sub: points per sub-tile (4, 8, 16, 32).

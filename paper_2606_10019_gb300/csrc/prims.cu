@@ -7,7 +7,6 @@
 
 #include "common.cuh"
 #include "csort.cuh"
-#include "perdevice.cuh"
 
 namespace gcvo {
 
@@ -179,7 +178,7 @@ gcvo_status scan_inclusive_max(int *data, int64_t n, void *scratch, cudaStream_t
 // then a scatter in which each warp walks its tile in order, ranking equal
 // digits with ballots so that the order of equal keys is kept.  Up to
 // csort::MAX_N keys of at most csort::MAX_KEY_BITS bits the whole sort runs in
-// one cluster instead (csort.cuh), in one launch.
+// one cluster instead (csort.cuh), in one launch, where the device can place it.
 // ---------------------------------------------------------------------------
 namespace {
 
@@ -283,18 +282,13 @@ __global__ void __launch_bounds__(csort::THREADS) k_cluster_sort(unsigned long l
 }
 
 template <int ITEMS>
-cudaError_t cluster_sort_attr() {
-    const cudaError_t e = cudaFuncSetAttribute(k_cluster_sort<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)sizeof(csort::Smem<ITEMS>));
-    return e != cudaSuccess ? e
-                            : cudaFuncSetAttribute(k_cluster_sort<ITEMS>,
-                                                   cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+bool cluster_sort_fits(int blocks) {
+    static PerDevice<unsigned> sizes;
+    return csort::placed(sizes.get([] { return csort::cluster_sizes<ITEMS>(k_cluster_sort<ITEMS>); }), blocks);
 }
 
 template <int ITEMS>
 gcvo_status cluster_sort_t(unsigned long long *keys, int *vals, int n, int bits, int blocks, cudaStream_t s) {
-    static PerDevice<cudaError_t> attr;
-    GCVO_CUDA(attr.get(cluster_sort_attr<ITEMS>));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(csort::THREADS);
@@ -309,6 +303,15 @@ gcvo_status cluster_sort_t(unsigned long long *keys, int *vals, int n, int bits,
     GCVO_CUDA(cudaLaunchKernelEx(&cfg, k_cluster_sort<ITEMS>, keys, vals, n, bits));
     count_launches(1);
     return GCVO_OK;
+}
+
+bool cluster_sort_fits(int items, int blocks) {
+    switch (items) {
+        case 1: return cluster_sort_fits<1>(blocks);
+        case 2: return cluster_sort_fits<2>(blocks);
+        case 4: return cluster_sort_fits<4>(blocks);
+        default: return false;   // too many keys
+    }
 }
 
 gcvo_status cluster_sort(unsigned long long *keys, int *vals, int n, int bits, int items, int blocks, cudaStream_t s) {
@@ -333,7 +336,7 @@ gcvo_status radix_sort_pairs(unsigned long long *keys, int *vals, int64_t n, int
     if (n <= 1 || bits <= 0) return GCVO_OK;
     int items, blocks;
     csort::shape(n, items, blocks);
-    if (items && bits <= csort::MAX_KEY_BITS) return cluster_sort(keys, vals, (int)n, bits, items, blocks, s);
+    if (bits <= csort::MAX_KEY_BITS && cluster_sort_fits(items, blocks)) return cluster_sort(keys, vals, (int)n, bits, items, blocks, s);
     if (scratch_bytes < radix_sort_scratch_bytes(n)) return GCVO_ERR_WORKSPACE;
     int n_tiles = (int)((n + RS_TILE - 1) / RS_TILE);
     auto al = [](size_t b) { return (b + 255) & ~size_t(255); };

@@ -18,7 +18,6 @@
 #include "common.cuh"
 #include "csort.cuh"
 #include "pair.cuh"
-#include "perdevice.cuh"
 #include "srcdev.cuh"
 
 namespace gcvo {
@@ -286,17 +285,13 @@ __global__ void __launch_bounds__(csort::THREADS) k_src_one(const SrcOneArgs a) 
 }
 
 template <int ITEMS>
-cudaError_t src_one_attr() {
-    const cudaError_t e = cudaFuncSetAttribute(k_src_one<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)sizeof(csort::Smem<ITEMS>));
-    return e != cudaSuccess ? e
-                            : cudaFuncSetAttribute(k_src_one<ITEMS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+bool fits_t(int blocks) {
+    static PerDevice<unsigned> sizes;
+    return csort::placed(sizes.get([] { return csort::cluster_sizes<ITEMS>(k_src_one<ITEMS>); }), blocks);
 }
 
 template <int ITEMS>
 gcvo_status launch_t(const SrcOneArgs &a, int blocks, cudaStream_t s) {
-    static PerDevice<cudaError_t> attr;
-    GCVO_CUDA(attr.get(src_one_attr<ITEMS>));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(csort::THREADS);
@@ -314,6 +309,17 @@ gcvo_status launch_t(const SrcOneArgs &a, int blocks, cudaStream_t s) {
 }
 
 }  // namespace
+
+bool src_one_fits(int64_t n) {
+    int items, blocks;
+    csort::shape(n, items, blocks);
+    switch (items) {
+        case 1: return fits_t<1>(blocks);
+        case 2: return fits_t<2>(blocks);
+        case 4: return fits_t<4>(blocks);
+        default: return false;
+    }
+}
 
 gcvo_status launch_src_one(const SrcOneArgs &a, cudaStream_t s) {
     int items, blocks;

@@ -84,3 +84,24 @@ for d in (0, 1):
 print(json.dumps(res))
 """)
     assert out[0] == out[1] and len(out[0]) > 100
+
+
+@pytest.mark.parametrize("most", [1, 2, 8, 16])
+def test_clusters_that_cannot_be_placed(fake, most):
+    """On a device that places no cluster of more than `most` blocks every size still runs, through clusters of at
+    most that size or the grid-wide kernels; with 16 nothing up to 65,536 points leaves the clusters."""
+    out = fake(f"most = {most}" + r"""
+L.fake_limits(most, 1 << 30)
+ctx = G.gcvo_create(0)
+for n in (1500, 4000, 9000, 20000, 65536):
+    G.gcvo_estimate_covariances(ctx, cloud(n), G.kernel_params(eig_max=0.01), np.zeros((6, n), np.float32))
+    p = problem(ctx, n, 1600)
+    G.gcvo_eval(ctx, *p)
+    G.gcvo_register(ctx, *p, G.solver_params(k_max=3))
+    if n <= 20000:
+        G.gcvo_register_batched(ctx, [p, p], G.solver_params(k_max=3))
+print(json.dumps(log()))
+""")
+    assert max(x[3] for x in out) == {1: 1, 2: 1, 8: 8, 16: 16}[most]     # 4,000 keys take 4 blocks, 8,000 8, 9,000 16
+    assert any("rs_hist" in x[1] for x in out) == any("k_knn_box" in x[1] for x in out) == (most < 16)
+    assert any("k_src_keys" in x[1] for x in out) and any("k_src_one" in x[1] for x in out)
