@@ -440,13 +440,23 @@ __global__ void __launch_bounds__(KNN_WARPS * 32)
     if (lane < 6) c.cov[(int64_t)lane * n + __float_as_int(q.w)] = s * (1.0f / (float)(knn - 1));
 }
 
-// Whether every off-diagonal entry of A' has E_pq^2 <= 2e-9 top |d_p - d_q|, top
-// the largest clamped eigenvalue.
-__device__ __forceinline__ bool eig_converged(const double d[3], double e01, double e02, double e12, double top) {
-    const float i = 1.0f / (float)top;
-    const float a = (float)e01 * i, b = (float)e02 * i, c = (float)e12 * i;
-    return a * a <= 2e-9f * fabsf((float)(d[0] - d[1]) * i) && b * b <= 2e-9f * fabsf((float)(d[0] - d[2]) * i) &&
-           c * c <= 2e-9f * fabsf((float)(d[1] - d[2]) * i);
+// Whether the entries of A' beside the diagonal d (e: 01, 02, 12) are small
+// enough for the first-order clamp to [lo, hi]: E_pq^2 <= 2e-9 top |d_p - d_q|
+// (the gaps less the rounding of d in FP32), top the largest clamped eigenvalue.
+// Whatever the gap, an entry below 3e-9 top moves the result by no more, and
+// between two eigenvalues on the same piece of the clamp (which meet on regular
+// grids of points) the formula is exact but for the third: 1e-6 top will do.
+// wide: the largest of d over top.
+__device__ __forceinline__ bool eig_converged(const double (&d)[3], const double (&e)[3], float lo, float hi, float &wide) {
+    const float x = (float)d[0], y = (float)d[1], z = (float)d[2], most = fmaxf(fmaxf(x, y), z);
+    const float i = 1.0f / fmaxf(fminf(most, hi), lo), off = 2e-7f * most;
+    wide = most * i;
+    auto good = [&](float u, float v, double entry) {
+        const float w = (float)entry * i;
+        const bool same = (u <= lo) == (v <= lo) && (u >= hi) == (v >= hi);
+        return w * w <= fmaxf(2e-9f * i * (fabsf(u - v) - off), same ? 1e-12f : 1e-17f);
+    };
+    return good(x, y, e[0]) && good(x, z, e[1]) && good(y, z, e[2]);
 }
 
 // Turns V until A' = V^T A V passes eig_converged, by sweeps of Jacobi's method
@@ -454,7 +464,7 @@ __device__ __forceinline__ bool eig_converged(const double d[3], double e01, dou
 // as good as FP32 makes it, which leaves 1e-7 of an entry, but its cosine and
 // sine belong together to FP64 rounding (Newton steps), and V is made
 // orthonormal again before every A'.
-__device__ __noinline__ void eig_refine(const float *s, double lo, double hi, double (*V)[3], double *d, double *e) {
+__device__ __noinline__ void eig_refine(const float *s, float lo, float hi, double (&V)[3][3], double (&d)[3], double (&e)[3]) {
     const double A[3][3] = {{s[0], s[1], s[2]}, {s[1], s[3], s[4]}, {s[2], s[4], s[5]}};
     for (int sweep = 0;; ++sweep) {
         double G[3][3], B[3][3], a[3][3];
@@ -470,15 +480,12 @@ __device__ __noinline__ void eig_refine(const float *s, double lo, double hi, do
             }
         for (int p = 0; p < 3; ++p)
             for (int q = p; q < 3; ++q) a[p][q] = a[q][p] = B[0][p] * G[0][q] + B[1][p] * G[1][q] + B[2][p] * G[2][q];
-        double top = lo;
-        for (int p = 0; p < 3; ++p) {
-            d[p] = a[p][p];
-            top = fmax(top, fmin(d[p], hi));
-        }
+        for (int p = 0; p < 3; ++p) d[p] = a[p][p];
         e[0] = a[0][1];
         e[1] = a[0][2];
         e[2] = a[1][2];
-        if (sweep == 8 || (sweep > 0 && eig_converged(d, e[0], e[1], e[2], top))) return;
+        float wide;
+        if (sweep == 8 || (sweep > 0 && eig_converged(d, e, lo, hi, wide))) return;
         for (int k = 0; k < 3; ++k) {
             const int p = k == 2 ? 1 : 0, q = k == 0 ? 1 : 2, r = 3 - p - q;
             const float den = 2.0f * (float)a[p][q];
@@ -581,24 +588,20 @@ __global__ void __launch_bounds__(128) k_knn_eig(const KnnCloud *cl, const int *
 #pragma unroll
             for (int q = 0; q < 3; ++q) AV[r][q] = A[r][0] * V[0][q] + A[r][1] * V[1][q] + A[r][2] * V[2][q];
         const double lo = c.eig_max / c.eig_ratio;
-        double top = lo, largest = 0.0;
 #pragma unroll
-        for (int p = 0; p < 3; ++p) {
-            d[p] = V[0][p] * AV[0][p] + V[1][p] * AV[1][p] + V[2][p] * AV[2][p];
-            top = fmax(top, fmin(d[p], c.eig_max));
-            largest = fmax(largest, d[p]);
-        }
+        for (int p = 0; p < 3; ++p) d[p] = V[0][p] * AV[0][p] + V[1][p] * AV[1][p] + V[2][p] * AV[2][p];
 #pragma unroll
         for (int p = 0; p < 3; ++p)
 #pragma unroll
             for (int q = p + 1; q < 3; ++q)
                 e[p + q - 1] = V[0][p] * AV[0][q] + V[1][p] * AV[1][q] + V[2][p] * AV[2][q];
         // V's own 1e-13 of the largest eigenvalue counts beyond 1e4 times the clamp
-        if (!eig_converged(d, e[0], e[1], e[2], top) || (float)largest > 1e4f * (float)top) {
+        float wide;
+        if (!eig_converged(d, e, (float)lo, (float)c.eig_max, wide) || wide > 1e4f) {
             double Vr[3][3], dr[3], er[3];
 #pragma unroll
             for (int r = 0; r < 9; ++r) Vr[r / 3][r % 3] = V[r / 3][r % 3];
-            eig_refine(s, lo, c.eig_max, Vr, dr, er);
+            eig_refine(s, (float)lo, (float)c.eig_max, Vr, dr, er);
 #pragma unroll
             for (int r = 0; r < 9; ++r) V[r / 3][r % 3] = Vr[r / 3][r % 3];
 #pragma unroll
