@@ -797,7 +797,8 @@ gcvo_status run_register(gcvo_ctx *ctx, int np, const gcvo_problem *pr, const gc
     void *hp;
     GCVO_TRY(host_pinned(ctx, 64, &hp));
     int *h_active = static_cast<int *>(hp);
-    if (sp->order == 2 && !ctx->profiling && loop_fits(np, pr)) {
+    bool looped = sp->order == 2 && !ctx->profiling && loop_fits(np, pr);
+    if (looped) {
         // the whole loop in one cooperative kernel (loop.cu), LOOP_ITERS
         // iterations at most before the host looks again
         LoopArgs la{};
@@ -812,13 +813,21 @@ gcvo_status run_register(gcvo_ctx *ctx, int np, const gcvo_problem *pr, const gc
         for (int it = 0; it < sp->k_max; it += LOOP_ITERS) {
             la.max_iters = std::min(LOOP_ITERS, sp->k_max - it);
             if (it > 0) GCVO_CUDA(cudaMemsetAsync(la.barrier, 0, sizeof(unsigned), s));
-            GCVO_CUDA(launch_loop(la, P.iso, P.feat_dim, b.sub, blocks, std::max(1, ctx->sm_count), s));
+            const cudaError_t e = launch_loop(la, P.iso, P.feat_dim, b.sub, blocks, std::max(1, ctx->sm_count), s);
+            if (it == 0 && e == cudaErrorCooperativeLaunchTooLarge) {
+                // the process has fewer SMs than the device: the graphs need none at once
+                cudaGetLastError();
+                looped = false;
+                break;
+            }
+            GCVO_CUDA(e);
             if (it + LOOP_ITERS >= sp->k_max) break;
             GCVO_CUDA(cudaMemcpyAsync(h_active, n_active, sizeof(int), cudaMemcpyDeviceToHost, s));
             GCVO_CUDA(cudaStreamSynchronize(s));
             if (*h_active <= 0) break;
         }
-    } else {
+    }
+    if (!looped) {
         // U iterations per host check, replayed from one CUDA graph.
         // Iterations past a problem's convergence or k_max leave it untouched
         // (the finalize skips inactive problems, the pair kernel their items).

@@ -103,7 +103,7 @@ cudaError_t launch_t(const LoopArgs &a, int blocks, int sm_count, cudaStream_t s
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, k_loop<ISO, FD, SUB>, a);
-    count_launches(1);
+    if (e == cudaSuccess) count_launches(1);
     return e;
 }
 

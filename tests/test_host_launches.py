@@ -105,3 +105,21 @@ print(json.dumps(log()))
     assert max(x[3] for x in out) == {1: 1, 2: 1, 8: 8, 16: 16}[most]     # 4,000 keys take 4 blocks, 8,000 8, 9,000 16
     assert any("rs_hist" in x[1] for x in out) == any("k_knn_box" in x[1] for x in out) == (most < 16)
     assert any("k_src_keys" in x[1] for x in out) and any("k_src_one" in x[1] for x in out)
+
+
+def test_cooperative_grid_that_does_not_fit(fake):
+    """A register loop whose grid cannot be resident at once replays the graphs."""
+    out = fake(r"""
+res = []
+for coop in (1 << 30, 100):
+    L.fake_limits(16, coop)
+    ctx = G.gcvo_create(0)
+    p = problem(ctx, 20000, 1600)
+    log()
+    G.gcvo_register(ctx, *p, G.solver_params(k_max=30))
+    res.append(log())
+print(json.dumps(res))
+""")
+    loop, graph = (["k_loop" in x[1] for x in r] for r in out)
+    assert sum(loop) == 1 and not any(graph)
+    assert not any(x[1] == "graph" for x in out[0]) and any(x[1] == "graph" for x in out[1])
