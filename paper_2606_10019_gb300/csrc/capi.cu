@@ -759,18 +759,29 @@ gcvo_status capture_chunk(gcvo_ctx *ctx, const Prepared &P, IterBufs &b, int ord
 
 constexpr int LOOP_ITERS = 512;
 
-// Whether the register loop's kernel may take these problems.  Its barriers
-// wait for the slowest block's pair pass, at most LOOP_SPINS polls of about 0.7
-// us (loop.cu), so the pass has to be short against that even when every pair
-// is evaluated: 2^39 pairs take 2 s (2.8e11 pairs/s on dense clouds; 5 s with 7
-// feature channels).  Larger sets, whose passes dwarf the launches, replay the
-// graphs, where nothing waits; 64 pairs of 40,000-point clouds are 2^37.
-constexpr double LOOP_MAX_PAIRS = 549755813888.0;
+// Whether the register loop's kernel may take these problems.  A barrier of
+// it waits for the slowest warp's pair pass, at most LOOP_SPINS polls of about
+// 0.7 us (12 s; loop.cu), so the pass has to be short against that even when
+// every pair is evaluated.  Two terms bound it.  The GPU takes 2.8e11 pairs/s
+// on dense clouds (a warp 9e7 beside its SM's others), a 2.5th of that with
+// more than 3 feature channels:
+//   - all pairs: 2^39 are 2 s;
+//   - the last grab of a warp, PAIR_GRAB items of up to `sub` points each
+//     against every target, which no other warp shares: 2^29 pairs are 6 s (a
+//     target of 8 million points in sub-tiles of 32, of 33 million in 8).
+// Larger sets, whose passes dwarf the launches, replay the graphs, where nothing
+// waits; 64 pairs of 40,000-point clouds are 2^37.
+constexpr double LOOP_MAX_PAIRS = 549755813888.0, LOOP_MAX_GRAB = 536870912.0;
 
-bool loop_fits(int np, const gcvo_problem *pr) {
-    double pairs = 0.0;
-    for (int p = 0; p < np; ++p) pairs += (double)pr[p].n_src * (double)pr[p].target->store.d.n;
-    return pairs <= LOOP_MAX_PAIRS;
+bool loop_fits(int np, const gcvo_problem *pr, int feat_dim, int sub) {
+    const double cost = feat_dim > 3 ? 2.5 : 1.0;
+    double pairs = 0.0, most = 0.0;
+    for (int p = 0; p < np; ++p) {
+        const double n_tgt = (double)pr[p].target->store.d.n;
+        pairs += (double)pr[p].n_src * n_tgt;
+        most = std::max(most, std::min((double)PAIR_GRAB * sub, (double)pr[p].n_src) * n_tgt);
+    }
+    return cost * pairs <= LOOP_MAX_PAIRS && cost * most <= LOOP_MAX_GRAB;
 }
 
 gcvo_status run_register(gcvo_ctx *ctx, int np, const gcvo_problem *pr, const gcvo_solver_params *sp,
@@ -797,7 +808,7 @@ gcvo_status run_register(gcvo_ctx *ctx, int np, const gcvo_problem *pr, const gc
     void *hp;
     GCVO_TRY(host_pinned(ctx, 64, &hp));
     int *h_active = static_cast<int *>(hp);
-    bool looped = sp->order == 2 && !ctx->profiling && loop_fits(np, pr);
+    bool looped = sp->order == 2 && !ctx->profiling && loop_fits(np, pr, P.feat_dim, b.sub);
     if (looped) {
         // the whole loop in one cooperative kernel (loop.cu), LOOP_ITERS
         // iterations at most before the host looks again

@@ -123,3 +123,17 @@ print(json.dumps(res))
     loop, graph = (["k_loop" in x[1] for x in r] for r in out)
     assert sum(loop) == 1 and not any(graph)
     assert not any(x[1] == "graph" for x in out[0]) and any(x[1] == "graph" for x in out[1])
+
+
+@pytest.mark.parametrize("n_src,n_tgt,feat,sub,loop", [(64, 3300000, 7, 32, True), (64, 3400000, 7, 32, False),
+                                                       (20, 3400000, 7, 32, True), (3000, 3400000, 7, 8, True)])
+def test_work_items_too_long_for_a_barrier(fake, n_src, n_tgt, feat, sub, loop):
+    """The pairs of one warp's last work items bound the register loop's kernel as well as those of the whole set."""
+    out = fake(f"n_src, n_tgt, feat, sub = {n_src}, {n_tgt}, {feat}, {sub}" + r"""
+ctx = G.gcvo_create(0)
+G.gcvo_pair_schedule(ctx, sub)
+G.gcvo_register(ctx, *problem(ctx, n_src, n_tgt, feat), G.solver_params(k_max=3))
+print(json.dumps(log()))
+""")
+    assert any("k_loop" in x[1] for x in out) == loop
+    assert any(x[1] == "graph" for x in out) != loop
