@@ -25,7 +25,10 @@
  *    valid until the call returns.
  *  - All work runs on the stream given to gcvo_create, in stream order.
  *    Calls that return host results (eval, register) synchronise that stream
- *    before returning.  A context is used by one host thread at a time.
+ *    before returning.  A context is used by one host thread at a time.  A
+ *    G-CVO-2 registration runs as launches of one kernel that takes every SM for
+ *    some iterations, about 4 ms (or one iteration that is longer); kernels of
+ *    other streams start between them.
  *  - Every call returns a gcvo_status.  On any status other than GCVO_OK the
  *    outputs are left untouched, except where a call documents otherwise.
  *    Device-side failures (a bounded wait that ran out, a capacity limit, a

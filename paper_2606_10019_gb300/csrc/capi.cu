@@ -757,7 +757,18 @@ gcvo_status capture_chunk(gcvo_ctx *ctx, const Prepared &P, IterBufs &b, int ord
     return GCVO_OK;
 }
 
-constexpr int LOOP_ITERS = 512;
+// Iterations of one launch of the register loop's kernel.  It keeps every SM
+// until it ends, and the kernels of other streams with it, so a launch takes
+// about 4 ms: an iteration is about 30 us of barriers and finalize, 0.4 ns per
+// source point (64 pairs, 0.9 million points: 360 us) and, without a cutoff,
+// its pairs at 2.8e11 a second.
+int loop_iters(int64_t n_points, double dense_pairs) {
+    const double us = 30.0 + 4e-4 * (double)n_points + dense_pairs / 2.8e5;
+    return (int)std::max(1.0, std::min(128.0, 4000.0 / us));
+}
+
+// Iterations at least between two looks of the host at the active problems.
+constexpr int LOOP_LOOK = 8;
 
 // Whether the register loop's kernel may take these problems.  A barrier of
 // it waits for the slowest warp's pair pass, at most LOOP_SPINS polls of about
@@ -810,8 +821,12 @@ gcvo_status run_register(gcvo_ctx *ctx, int np, const gcvo_problem *pr, const gc
     int *h_active = static_cast<int *>(hp);
     bool looped = sp->order == 2 && !ctx->profiling && loop_fits(np, pr, P.feat_dim, b.sub);
     if (looped) {
-        // the whole loop in one cooperative kernel (loop.cu), LOOP_ITERS
-        // iterations at most before the host looks again
+        // whole iterations in one cooperative kernel (loop.cu), which returns at
+        // once when no problem is active
+        double dense = 0.0;
+        for (int p = 0; p < np; ++p)
+            if (pr[p].target->kp.cutoff == 0) dense += (double)pr[p].n_src * (double)pr[p].target->store.d.n;
+        const int iters = loop_iters(P.n_points, dense);
         LoopArgs la{};
         la.pair = b.pa;
         la.fin = b.fa;
@@ -821,8 +836,14 @@ gcvo_status run_register(gcvo_ctx *ctx, int np, const gcvo_problem *pr, const gc
         // one warp per work item, of which there are up to about twice as
         // many as full ones; more blocks only lengthen the barriers
         const int blocks = (int)std::min<int64_t>(1 << 20, (2 * P.n_points / b.sub + PAIR_WARPS - 1) / PAIR_WARPS);
-        for (int it = 0; it < sp->k_max; it += LOOP_ITERS) {
-            la.max_iters = std::min(LOOP_ITERS, sp->k_max - it);
+        for (int it = 0, look = LOOP_LOOK; it < sp->k_max; it += iters) {
+            if (it >= look) {
+                GCVO_CUDA(cudaMemcpyAsync(h_active, n_active, sizeof(int), cudaMemcpyDeviceToHost, s));
+                GCVO_CUDA(cudaStreamSynchronize(s));
+                if (*h_active <= 0) break;
+                look = it + LOOP_LOOK;
+            }
+            la.max_iters = std::min(iters, sp->k_max - it);
             if (it > 0) GCVO_CUDA(cudaMemsetAsync(la.barrier, 0, sizeof(unsigned), s));
             const cudaError_t e = launch_loop(la, P.iso, P.feat_dim, b.sub, blocks, std::max(1, ctx->sm_count), s);
             if (it == 0 && e == cudaErrorCooperativeLaunchTooLarge) {
@@ -832,10 +853,6 @@ gcvo_status run_register(gcvo_ctx *ctx, int np, const gcvo_problem *pr, const gc
                 break;
             }
             GCVO_CUDA(e);
-            if (it + LOOP_ITERS >= sp->k_max) break;
-            GCVO_CUDA(cudaMemcpyAsync(h_active, n_active, sizeof(int), cudaMemcpyDeviceToHost, s));
-            GCVO_CUDA(cudaStreamSynchronize(s));
-            if (*h_active <= 0) break;
         }
     }
     if (!looped) {

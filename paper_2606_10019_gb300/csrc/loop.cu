@@ -16,7 +16,8 @@
 // other orders, and a context that times its kernels, keep the graphs.
 //
 // The blocks of a cooperative launch are all resident, so the barrier's spin
-// ends; it is bounded all the same.
+// ends; it is bounded all the same.  They hold every SM, and the kernels of other
+// streams wait, so a launch takes some iterations only (loop_iters, capi.cu).
 #include <algorithm>
 
 #include "common.cuh"
@@ -67,6 +68,8 @@ __global__ void __launch_bounds__(PAIR_WARPS * 32, 5) k_loop(LoopArgs a) {
     tile_init(stage);
     unsigned parity = 0, round = 0;
     bool ok = true;
+    // (it changes only behind a barrier that every block has to reach)
+    if (*(volatile int *)a.fin.n_active <= 0) return;
     for (int it = 0; it < a.max_iters; ++it) {
         ok = tile_pass<PAIR_EVAL, ISO, FD, SUB>(a.pair, stage, parity);
         if (!__syncthreads_and(ok)) break;

@@ -137,3 +137,17 @@ print(json.dumps(log()))
 """)
     assert any("k_loop" in x[1] for x in out) == loop
     assert any(x[1] == "graph" for x in out) != loop
+
+
+@pytest.mark.parametrize("n_src,pairs,k_max,cutoff,least,most", [(1000, 2, 100, 3.0, 1, 1), (1000, 2, 300, 3.0, 2, 10),
+                                                                 (200000, 5, 90, 3.0, 9, 30), (9000, 6, 40, 0.0, 10, 40)])
+def test_register_loop_gives_the_gpu_back(fake, n_src, pairs, k_max, cutoff, least, most):
+    """The loop's kernel holds every SM, so a launch of it is some milliseconds of iterations, fewer on large sets."""
+    out = fake(f"n_src, pairs, k_max, cutoff = {n_src}, {pairs}, {k_max}, {cutoff}" + r"""
+ctx = G.gcvo_create(0)
+G.gcvo_pair_schedule(ctx, 8)
+p = problem(ctx, n_src, 9000, cutoff=cutoff)
+G.gcvo_register_batched(ctx, [p] * pairs, G.solver_params(k_max=k_max))
+print(json.dumps(log()))
+""")
+    assert least <= sum("k_loop" in x[1] for x in out) <= most
