@@ -326,6 +326,14 @@ __device__ __forceinline__ void pt_stage(unsigned char *dst, const __nv_bfloat16
     }
 }
 
+// One output of layer 1 before its relu, for the point p = (x, y, z, l).  The
+// forward pass (two outputs at a time, pt_layer1) and the backward pass sum in
+// this order, so that they see the same activations: the last bits decide a
+// BF16 rounding, and whether a relu near zero is open.
+__device__ __forceinline__ float layer1_sum(float4 w, float bias, float4 p) {
+    return __fadd_rn(__fmaf_rn(w.w, p.w, __fmaf_rn(w.z, p.z, __fmaf_rn(w.x, p.x, __fmul_rn(w.y, p.y)))), bias);
+}
+
 // Layer 1 of one point into row r of a tile.
 __device__ __forceinline__ void pt_layer1(const float *w1, float4 p, unsigned char *h1, int r) {
     const uint64_t x = f2_pack(p.x, p.x), y = f2_pack(p.y, p.y), z = f2_pack(p.z, p.z), l = f2_pack(p.w, p.w);
@@ -807,11 +815,7 @@ __global__ void __launch_bounds__(BW_THREADS, 2) k_point_bwd(Net net, int n, int
             for (int k = 0; k < 16; ++k) {
                 const int o = (tid & 3) + 4 * k;
                 const float4 w = *reinterpret_cast<const float4 *>(w1 + 4 * o);
-                float s = b1[o];
-                s += w.x * q.x;
-                s += w.y * q.y;
-                s += w.z * q.z;
-                s += w.w * q.w;
+                const float s = layer1_sum(w, b1[o], q);
                 h1[(tid >> 2) * BW_LD1 + o] = __bfloat162float(__float2bfloat16_rn(fmaxf(s, 0.f)));
             }
         }
