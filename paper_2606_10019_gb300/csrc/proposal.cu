@@ -288,7 +288,7 @@ constexpr int PT_BAR = PT_B2 + 128 * 4;
 constexpr int PT_SMEM = PT_BAR + 256;
 
 struct PtBars {
-    uint64_t h1_full[2], d2_full[2], h2_full[2], h2_free[2], d3_full[2], d3_free[2];
+    uint64_t h1_full[2], d2_full[2], h2_full[2], h2_free[2], d3_full[2], d3_free[2], drained;
     uint32_t tmem;
 };
 static_assert(sizeof(PtBars) <= 256, "the barriers fit");
@@ -384,6 +384,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1)
             mbar_init(&B.h2_free[k], 1);
             mbar_init(&B.d3_full[k], 1);
         }
+        mbar_init(&B.drained, 1);
     }
     fence_proxy_async_smem();
     tc5_fence_before();
@@ -473,6 +474,9 @@ __global__ void __launch_bounds__(PT_THREADS, 1)
                 }
                 if (ok) tc5_commit(&B.h2_free[b]);
             }
+            // a wait may have run out with products in flight: they end before the tensor memory goes
+            tc5_commit(&B.drained);
+            ok = mbar_wait(&B.drained, 0) && ok;
         }
         ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
     } else {
