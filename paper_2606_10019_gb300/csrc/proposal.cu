@@ -190,13 +190,14 @@ __global__ void __launch_bounds__(PREP_THREADS)
         for (int i = threadIdx.x; i < n; i += PREP_THREADS)
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                // d + e = t - c, and its square
+                // d + e = t - c, and its square (far from the origin e, with the centroid's tail in it, is
+                // not small: 4 mm at 100 km)
                 float d = t[(size_t)a * n + i], e = 0.f;
                 acc2(d, e, -ch[a]);
                 e = __fsub_rn(e, cl[a]);
                 const float p = __fmul_rn(d, d);
                 acc2(rh[0], rl[0], p);
-                rl[0] = __fadd_rn(rl[0], __fmaf_rn(d, d, -p) + 2.f * d * e);
+                rl[0] = __fadd_rn(rl[0], __fmaf_rn(d, d, -p) + e * (2.f * d + e));
             }
         const double sum = prep_block_sum<1>(rh, rl, red);
         if (threadIdx.x == 0) r64 = sum;
