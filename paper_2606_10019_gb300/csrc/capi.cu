@@ -759,11 +759,12 @@ gcvo_status capture_chunk(gcvo_ctx *ctx, const Prepared &P, IterBufs &b, int ord
 
 // Iterations of one launch of the register loop's kernel.  It keeps every SM
 // until it ends, and the kernels of other streams with it, so a launch takes
-// about 4 ms: an iteration is about 30 us of barriers and finalize, 0.4 ns per
-// source point (64 pairs, 0.9 million points: 360 us) and, without a cutoff,
-// its pairs at 2.8e11 a second.
+// about 4 ms: an iteration is about 30 us of barriers and finalize, up to a
+// nanosecond per source point (16 pairs of dense scenes and LiDAR frames, 150,000
+// points: 230 us; 64, 600,000 points: 430 us) and, without a cutoff, its pairs
+// at 2.8e11 a second.
 int loop_iters(int64_t n_points, double dense_pairs) {
-    const double us = 30.0 + 4e-4 * (double)n_points + dense_pairs / 2.8e5;
+    const double us = 30.0 + 1e-3 * (double)n_points + dense_pairs / 2.8e5;
     return (int)std::max(1.0, std::min(128.0, 4000.0 / us));
 }
 

@@ -126,7 +126,8 @@ print(json.dumps(res))
 
 
 @pytest.mark.parametrize("n_src,n_tgt,feat,sub,loop", [(64, 3300000, 7, 32, True), (64, 3400000, 7, 32, False),
-                                                       (20, 3400000, 7, 32, True), (3000, 3400000, 7, 8, True)])
+                                                       (20, 3400000, 7, 32, True), (3000, 3400000, 7, 8, True),
+                                                       (200000, 1200000, 7, 8, False)])
 def test_work_items_too_long_for_a_barrier(fake, n_src, n_tgt, feat, sub, loop):
     """The pairs of one warp's last work items bound the register loop's kernel as well as those of the whole set."""
     out = fake(f"n_src, n_tgt, feat, sub = {n_src}, {n_tgt}, {feat}, {sub}" + r"""
