@@ -412,7 +412,12 @@ static __device__ __noinline__ void fin_chunks(const FinalizeArgs &a, FinShared 
     const int nch = *a.n_chunks;
     // the pair pass is done with its work counter: ready for the next one
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.work = 0;
-    for (int c = blockIdx.x; c < nch; c += gridDim.x) {
+    // with many chunks a block takes `run` consecutive ones and counts those of a
+    // problem together: the count is a fence and an atomic's round trip (256
+    // problems, 1.6 million points: 160 -> 97 us in sub-tiles of 8, 131 -> 72 in 16)
+    const int lg = nch > 4 * (int)gridDim.x ? 2 : 0, run = 1 << lg;
+    int counted = 0;   // chunks of this block that their problem's count lacks yet
+    for (int i = 0, c; (c = (((i >> lg) * (int)gridDim.x + (int)blockIdx.x) << lg) + (i & (run - 1))) < nch; ++i) {
         int lo = 0, hi = a.n_problems - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -475,12 +480,18 @@ static __device__ __noinline__ void fin_chunks(const FinalizeArgs &a, FinShared 
             if (c1 - c0 > 1) a.chunk_cnt[(size_t)c * 4 + threadIdx.x] = cs;
         }
         if (c1 - c0 > 1) {
-            __threadfence();   // the row before the count of finished chunks
+            ++counted;
+            if (((i + 1) & (run - 1)) != 0 && c + 1 < c1) {
+                __syncthreads();   // the shared sums are read
+                continue;
+            }
+            __threadfence();   // the rows before the count of finished chunks
             __syncthreads();
             if (threadIdx.x == 0) {
-                S.last = atomicAdd(&P->done, 1) == c1 - c0 - 1;
+                S.last = atomicAdd(&P->done, counted) == c1 - c0 - counted;
                 if (S.last) P->done = 0;
             }
+            counted = 0;
             __syncthreads();
             if (!S.last) continue;
             __threadfence();   // the other chunks' rows after the count
