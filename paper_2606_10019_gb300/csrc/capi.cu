@@ -7,6 +7,7 @@
 
 #include "common.cuh"
 #include "pair.cuh"
+#include "perdevice.cuh"
 
 using namespace gcvo;
 
@@ -423,6 +424,7 @@ gcvo_status prepare(gcvo_ctx *ctx, int np, const gcvo_problem *pr, Prepared &P) 
         d.rho2 = (float)rho2;
         d.c2 = (float)c2;
         d.lo = pair_needs_lo(G->store.d, kp, rho2, lmin_src) ? 1 : 0;
+        d.tails = tail_slack(grid_half_diagonal(G->store.d), rho2, c2);
         d.sigma2 = (float)kp.sigma2;
         d.iso_inv = kp.kernel_mode == 1 ? (float)(1.0 / (kp.iso_ell * kp.iso_ell)) : 0.f;
     }
@@ -1010,7 +1012,7 @@ gcvo_status gcvo_create(gcvo_ctx **ctx, int device, void *cuda_stream) {
         cudaGetLastError();
         return GCVO_ERR_INVALID_ARG;
     }
-    GCVO_CUDA(cudaSetDevice(device));
+    GCVO_CUDA(use_device(device));
     gcvo_ctx *c = new (std::nothrow) gcvo_ctx();
     if (!c) return GCVO_ERR_WORKSPACE;
     c->device = device;
@@ -1050,7 +1052,7 @@ gcvo_status gcvo_destroy(gcvo_ctx *ctx) {
 
 gcvo_status gcvo_profile_enable(gcvo_ctx *ctx, int enable) {
     if (!ctx) return GCVO_ERR_INVALID_ARG;
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     GCVO_CUDA(cudaStreamSynchronize(ctx->stream));
     ctx->profiling = enable ? 1 : 0;
     ctx->ev_used = 0;
@@ -1077,7 +1079,7 @@ gcvo_status gcvo_pair_schedule(gcvo_ctx *ctx, int set, int *last_used) {
 
 gcvo_status gcvo_profile_read(gcvo_ctx *ctx, gcvo_profile *out) {
     if (!ctx || !out) return GCVO_ERR_INVALID_ARG;
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     GCVO_CUDA(cudaStreamSynchronize(ctx->stream));
     GCVO_TRY(collect_profile(ctx));
     out->n_launches = launches_so_far() - ctx->launch_base;
@@ -1099,7 +1101,7 @@ gcvo_status gcvo_estimate_covariances(gcvo_ctx *ctx, const float *xyz, int64_t n
         return GCVO_ERR_INVALID_ARG;
     if (params->eig_max > 0 && !(params->eig_ratio >= 1.0)) return GCVO_ERR_INVALID_ARG;
     if (!(params->cutoff >= 0)) return GCVO_ERR_INVALID_ARG;
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     size_t need = staged_floats(xyz, 3 * (size_t)n);
     bool host_out = !is_device_ptr(cov_out);
     if (need) GCVO_TRY(ctx->stage_xyz.ensure(need * sizeof(float), ctx->stream));
@@ -1125,7 +1127,7 @@ static gcvo_status build_into(gcvo_ctx *ctx, const float *xyz, const float *cov,
     if (!ctx || !xyz || !feat || !valid_kernel_params(params)) return GCVO_ERR_INVALID_ARG;
     if (params->kernel_mode == 0 && !cov) return GCVO_ERR_INVALID_ARG;
     if (n < 1 || n > (1 << 28)) return GCVO_ERR_INVALID_ARG;
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     cudaStream_t s = ctx->stream;
     size_t need = staged_floats(xyz, 3 * (size_t)n) + staged_floats(feat, (size_t)params->feat_dim * n) +
                   (params->kernel_mode == 0 ? staged_floats(cov, 6 * (size_t)n) : 0);
@@ -1193,7 +1195,7 @@ gcvo_status gcvo_grid_info(const gcvo_grid *grid, int64_t *n_points, int64_t *n_
 static gcvo_status eval_once(gcvo_ctx *ctx, const gcvo_grid *target, const float *src_xyz, const float *src_cov,
                              const float *src_feat, int64_t n_src, const double T[16], int mode, int fin,
                              double *f, double g[6], double H[36], double *M_out, gcvo_eval_stats *stats) {
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     gcvo_problem pr{};
     pr.target = target;
     pr.src_xyz = src_xyz;
@@ -1257,7 +1259,7 @@ gcvo_status gcvo_register(gcvo_ctx *ctx, const gcvo_grid *target, const float *s
                           const float *src_feat, int64_t n_src, const double T0[16],
                           const gcvo_solver_params *params, double T_out[16], gcvo_iter_log *log, int *n_iter) {
     if (!ctx || !target || !src_xyz || !src_feat || !T0 || !T_out) return GCVO_ERR_INVALID_ARG;
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     gcvo_problem pr{};
     pr.target = target;
     pr.src_xyz = src_xyz;
@@ -1277,7 +1279,7 @@ gcvo_status gcvo_register_batched(gcvo_ctx *ctx, int n_problems, const gcvo_prob
                                   const gcvo_solver_params *params, double *T_out, gcvo_iter_log *logs,
                                   int *n_iter, int *status) {
     if (!ctx || !problems || !T_out || n_problems < 1) return GCVO_ERR_INVALID_ARG;
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     return run_register(ctx, n_problems, problems, params, T_out, logs, n_iter, status);
 }
 
@@ -1296,7 +1298,7 @@ gcvo_status gcvo_estimate_covariances_batched(gcvo_ctx *ctx, int n_clouds, const
         if (n[k] < params->knn || n[k] > (1 << 28)) return GCVO_ERR_INVALID_ARG;
         jobs[k] = KnnJob{xyz[k], cov_out[k], n[k], params};
     }
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     return knn_covariances(ctx, n_clouds, jobs.data());
 }
 
@@ -1313,7 +1315,7 @@ gcvo_status gcvo_build_grids_batched(gcvo_ctx *ctx, int n_clouds, const float *c
     if (!valid_kernel_params(params)) return GCVO_ERR_INVALID_ARG;
     for (int k = 0; k < n_clouds; ++k)
         if (n[k] < 1 || n[k] > (1 << 28)) return GCVO_ERR_INVALID_ARG;
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     // new grids for the empty slots; on failure they are released again
     std::vector<TgJob> jobs(n_clouds);
     std::vector<char> created(n_clouds, 0);
@@ -1357,7 +1359,7 @@ gcvo_status gcvo_register_clouds(gcvo_ctx *ctx, int n_pairs, const gcvo_cloud_pa
             return GCVO_ERR_INVALID_ARG;
         if (kp[k]->knn < 2 || kp[k]->knn > GCVO_MAX_KNN) return GCVO_ERR_INVALID_ARG;
     }
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     cudaStream_t s = ctx->stream;
     const int fd = params->feat_dim;
     // cloud c = 2k (target of pair k) or 2k + 1 (its source)
@@ -1454,7 +1456,7 @@ gcvo_status gcvo_workspace_size(const gcvo_ctx *ctx, int64_t max_points, int max
 gcvo_status gcvo_set_workspace(gcvo_ctx *ctx, void *dev_ptr, size_t bytes, int64_t max_points, int max_problems,
                                int64_t max_log_rows) {
     if (!ctx) return GCVO_ERR_INVALID_ARG;
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     GCVO_CUDA(cudaStreamSynchronize(ctx->stream));
     std::vector<DevBuf *> bufs = ws_bufs(ctx);
     if (!dev_ptr) {

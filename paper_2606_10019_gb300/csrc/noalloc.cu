@@ -18,6 +18,7 @@
 
 #include "common.cuh"
 #include "pair.cuh"
+#include "perdevice.cuh"
 
 namespace gcvo {
 namespace {
@@ -129,6 +130,9 @@ __global__ void k_na_setup(NaSetup a, unsigned char *base) {
     if (a.cutoff == 0) rho2 = c2 = INFINITY;   // dense: every pair
     P->rho2 = (float)rho2;
     P->c2 = (float)c2;
+    double half = 0.0;
+    for (int k = 0; k < 3; ++k) half += 0.25 * (double)G->dims[k] * G->dims[k] * G->h * G->h;
+    P->tails = tail_slack(sqrt(half), rho2, c2);
     P->sigma2 = (float)a.sigma2;
     P->iso_inv = a.kernel_mode == 1 ? (float)(1.0 / (a.iso_ell * a.iso_ell)) : 0.f;
     words[1] = a.n_items;
@@ -167,7 +171,7 @@ extern "C" gcvo_status gcvo_eval_static(const gcvo_grid *target, const float *sr
         if (at.type != cudaMemoryTypeDevice && at.type != cudaMemoryTypeManaged) return GCVO_ERR_INVALID_ARG;
         if (at.type == cudaMemoryTypeDevice && at.device != dev) return GCVO_ERR_INVALID_ARG;
     }
-    GCVO_CUDA(cudaSetDevice(dev));
+    GCVO_CUDA(use_device(dev));
     unsigned char *base;
     {
         std::lock_guard<std::mutex> lk(g_na_mutex);

@@ -46,6 +46,7 @@ struct ProbDev {
     int c0, c1;        // range of finalize chunks (FIN_CHUNK work items each)
     int done;          // chunks of the running finalize that are summed (0 between launches)
     int lo;            // 1: the pair passes form r from double-float positions
+    float tails;       // slack of the per-pair limits for the position tails (tail_slack)
     float rho2;        // Euclidean pre-test radius squared
     float c2;          // cutoff squared
     float sigma2;
@@ -57,6 +58,16 @@ struct EvalOut {
     long long n_pairs, n_kept, n_cand;
     float rho2;
 };
+
+// What the pair pass adds to a covariance in its per-pair limits, which it
+// tests on position heads: the tails shorten a distance of up to rho by up to e =
+// 2.4e-7 R (2^-24 of either position, and the difference's rounding; R: half the
+// diagonal of the target's box and rho), its square by 2 rho e + e^2.
+__host__ __device__ inline float tail_slack(double half_diag, double rho2, double c2) {
+    if (!(rho2 < 1e30)) return 0.f;   // no cutoff: no limits
+    const double rho = sqrt(rho2), e = 2.4e-7 * (half_diag + rho);
+    return (float)(e * (2.0 * rho + e) / c2 * 1.001);
+}
 
 // Source points in the target grid's frame at the current pose, written by
 // k_transform once per iteration (sorted order, one record per point):

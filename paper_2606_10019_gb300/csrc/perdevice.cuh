@@ -5,28 +5,43 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <mutex>
-#include <utility>
-#include <vector>
 
 namespace gcvo {
 
+// The device of this thread's call: every entry point that launches names it
+// with use_device, so that a launch need not ask the runtime for it.
+inline int &call_device() {
+    static thread_local int device = 0;
+    return device;
+}
+inline cudaError_t use_device(int device) {
+    call_device() = device;
+    return cudaSetDevice(device);
+}
+
 template <class T>
 class PerDevice {
+    static constexpr int MOST = 64;
     std::mutex m_;
-    std::vector<std::pair<int, T>> known_;   // few devices
+    std::atomic<bool> known_[MOST] = {};
+    T value_[MOST];
 
 public:
-    // The value of the current device, made by make() on its first use there.
+    // The value of the call's device, made by make() on its first use there.
     template <class Make>
     T get(Make make) {
-        int d = 0;
-        cudaGetDevice(&d);
-        std::lock_guard<std::mutex> lk(m_);
-        for (const auto &kv : known_)
-            if (kv.first == d) return kv.second;
-        known_.emplace_back(d, make());
-        return known_.back().second;
+        const int d = call_device();
+        if (d < 0 || d >= MOST) return make();
+        if (!known_[d].load(std::memory_order_acquire)) {
+            std::lock_guard<std::mutex> lk(m_);
+            if (!known_[d].load(std::memory_order_relaxed)) {
+                value_[d] = make();
+                known_[d].store(true, std::memory_order_release);
+            }
+        }
+        return value_[d];
     }
 };
 

@@ -1086,7 +1086,7 @@ extern "C" {
 
 gcvo_status gcvo_proposal_create(gcvo_ctx *ctx, gcvo_proposal **out) {
     if (!ctx || !out) return GCVO_ERR_INVALID_ARG;
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     gcvo_proposal *P = new (std::nothrow) gcvo_proposal();
     if (!P) return GCVO_ERR_WORKSPACE;
     P->device = ctx->device;
@@ -1122,7 +1122,7 @@ int64_t gcvo_proposal_n_params(void) { return prop::Layout().n(); }
 
 gcvo_status gcvo_proposal_set_params(gcvo_ctx *ctx, gcvo_proposal *P, const float *params) {
     if (!ctx || !P || !params) return GCVO_ERR_INVALID_ARG;
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     const int n = P->L.n();
     cudaStream_t s = ctx->stream;
     GCVO_CUDA(cudaMemcpyAsync(P->p.ptr, params, n * sizeof(float), cudaMemcpyDefault, s));
@@ -1138,7 +1138,7 @@ gcvo_status gcvo_proposal_set_params(gcvo_ctx *ctx, gcvo_proposal *P, const floa
 
 gcvo_status gcvo_proposal_get_params(gcvo_ctx *ctx, const gcvo_proposal *P, float *params_out) {
     if (!ctx || !P || !params_out) return GCVO_ERR_INVALID_ARG;
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     GCVO_CUDA(cudaMemcpyAsync(params_out, P->p.ptr, P->L.n() * sizeof(float), cudaMemcpyDefault, ctx->stream));
     GCVO_CUDA(cudaStreamSynchronize(ctx->stream));
     return GCVO_OK;
@@ -1146,7 +1146,7 @@ gcvo_status gcvo_proposal_get_params(gcvo_ctx *ctx, const gcvo_proposal *P, floa
 
 gcvo_status gcvo_proposal_get_state(gcvo_ctx *ctx, const gcvo_proposal *P, float *state_out, int64_t *step_out) {
     if (!ctx || !P || !state_out || !step_out) return GCVO_ERR_INVALID_ARG;
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     const size_t n = (size_t)P->L.n();
     const DevBuf *parts[3] = {&P->p, &P->m, &P->v};
     for (int k = 0; k < 3; ++k)
@@ -1159,7 +1159,7 @@ gcvo_status gcvo_proposal_get_state(gcvo_ctx *ctx, const gcvo_proposal *P, float
 
 gcvo_status gcvo_proposal_set_state(gcvo_ctx *ctx, gcvo_proposal *P, const float *state, int64_t step) {
     if (!ctx || !P || !state || step < 0 || step > (int64_t)1 << 30) return GCVO_ERR_INVALID_ARG;
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     const size_t n = (size_t)P->L.n();
     cudaStream_t s = ctx->stream;
     DevBuf *parts[3] = {&P->p, &P->m, &P->v};
@@ -1177,7 +1177,7 @@ gcvo_status gcvo_proposal_infer(gcvo_ctx *ctx, gcvo_proposal *P, int B, int n, c
                                 const float *src_feat, int src_feat_stride, const float *tgt_xyz,
                                 const float *tgt_feat, int tgt_feat_stride, float *twist_out, double *T0_out) {
     if (!ctx || !P || !src_xyz || !src_feat || !tgt_xyz || !tgt_feat || !valid_batch(B, n)) return GCVO_ERR_INVALID_ARG;
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     GCVO_TRY(forward_batch(ctx, P, B, n, src_xyz, src_feat, src_feat_stride, tgt_xyz, tgt_feat, tgt_feat_stride, nullptr));
     std::vector<float> out((size_t)B * 6), cs((size_t)B * 4);
     GCVO_CUDA(cudaMemcpyAsync(out.data(), P->out.ptr, out.size() * 4, cudaMemcpyDeviceToHost, ctx->stream));
@@ -1214,7 +1214,7 @@ gcvo_status gcvo_proposal_train_step(gcvo_ctx *ctx, gcvo_proposal *P, int B, int
     if (!ctx || !P || !src_xyz || !src_feat || !tgt_xyz || !tgt_feat || !T_label || !valid_batch(B, n) ||
         !(lr >= 0.f))
         return GCVO_ERR_INVALID_ARG;
-    GCVO_CUDA(cudaSetDevice(ctx->device));
+    GCVO_CUDA(use_device(ctx->device));
     cudaStream_t s = ctx->stream;
     GCVO_TRY(forward_batch(ctx, P, B, n, src_xyz, src_feat, src_feat_stride, tgt_xyz, tgt_feat, tgt_feat_stride,
                            T_label));

@@ -166,6 +166,7 @@ __global__ void __launch_bounds__(csort::THREADS) k_src_one(const SrcOneArgs a) 
             const double s2 = a.iso ? a.iso_ell * a.iso_ell : (double)a.grid.lam_min + (double)fmaxf(0.0f, lam_low);
             P->lo = a.cutoff <= 0 || !isfinite(r2) || !(s2 > 0.0) ||
                     4.0 * a.cutoff * (a.half_diag + sqrt(r2)) * 5.9604644775390625e-08 / sqrt(s2) > 3e-4;
+            P->tails = tail_slack(a.half_diag, r2, c2);
             a.words[SRC_WORD_ACTIVE] = bad ? 0u : 1u;
             if (bad) a.words[0] = DEV_ERR_NONFINITE;
         }

@@ -446,6 +446,7 @@ __device__ __forceinline__ bool tile_pass(const PairArgs &a, StageT<MODE, FD> *s
                 bmax[k] = ord_dec(__reduce_max_sync(FULL, ord_enc(sval ? pp[k] : -INFINITY)));
             }
         }
+        const float tails = P->tails;   // the limits are tested on position heads
         const float lam_sub = bounded ? ord_dec(__reduce_max_sync(FULL, ord_enc(lam_i))) : 0.f;
         // largest diagonal entries of Sigma'_j, the limits' slack included
         float dmax[3] = {0.f, 0.f, 0.f};
@@ -453,8 +454,9 @@ __device__ __forceinline__ bool tile_pass(const PairArgs &a, StageT<MODE, FD> *s
             const float dd[3] = {qv[0], qv[3], qv[5]};
 #pragma unroll
             for (int k = 0; k < 3; ++k)
-                dmax[k] = ord_dec(__reduce_max_sync(FULL, ord_enc(sval ? dd[k] : 0.f))) + 1e-5f * lam_sub;
+                dmax[k] = ord_dec(__reduce_max_sync(FULL, ord_enc(sval ? dd[k] : 0.f))) + (1e-5f * lam_sub + tails);
         }
+        const float lam_box = lam_sub + 3.f * tails;   // of the norm bound
         const float rho = sqrtf(rho2);
         const float h = G->h, ih = G->inv_h;
         // culling radius: rho plus a margin for the float voxel assignment
@@ -467,22 +469,13 @@ __device__ __forceinline__ bool tile_pass(const PairArgs &a, StageT<MODE, FD> *s
         // a target whose farthest corner of the box is nearer than this is
         // within rho of every point: r is formed from the same heads, and the
         // tails move it by less than 2^-22 of the largest coordinate
-        float rin2 = -1.f, lam_box = lam_sub;
+        float rin2 = -1.f;
         if (two_lists) {
             float mag = rho;
 #pragma unroll
             for (int k = 0; k < 3; ++k) mag = fmaxf(mag, fmaxf(-bmin[k], bmax[k]) + rho);
             const float ri = rho * 0.9999f - (dfr ? 1e-6f * mag : 0.f);
             rin2 = ri > 0.f ? ri * ri : -1.f;
-            if (dfr) {
-                // the per-pair limits are tested on heads too: a distance up to
-                // rho that the tails shorten by e has a square up to 2 rho e +
-                // e^2 larger there
-                const float e = 2.4e-7f * mag, s1 = e * (2.f * rho + e) / c2;
-#pragma unroll
-                for (int k = 0; k < 3; ++k) dmax[k] += s1;
-                lam_box += 3.f * s1;
-            }
         }
         int lo[3], hi[3];
         bool empty = !(bmin[0] <= bmax[0]);
