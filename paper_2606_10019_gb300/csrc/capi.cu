@@ -819,9 +819,17 @@ gcvo_status run_register(gcvo_ctx *ctx, int np, const gcvo_problem *pr, const gc
     b.fa.mu0 = sp->mu0;
     int *n_active = b.fa.n_active;
     if (!P.one) GCVO_CUDA(cudaMemcpyAsync(n_active, &np, sizeof(int), cudaMemcpyHostToDevice, s));
+    // the status word and the words behind it, read together
+    static_assert(SRC_WORD_ACTIVE < 32, "the active problems are among the words read");
     void *hp;
-    GCVO_TRY(host_pinned(ctx, 64, &hp));
-    int *h_active = static_cast<int *>(hp);
+    GCVO_TRY(host_pinned(ctx, 32 * sizeof(int), &hp));
+    int *h_words = static_cast<int *>(hp);
+    auto look_at = [&]() -> gcvo_status {
+        GCVO_CUDA(cudaMemcpyAsync(h_words, ctx->status_word.ptr, 32 * sizeof(int), cudaMemcpyDeviceToHost, s));
+        GCVO_CUDA(cudaStreamSynchronize(s));
+        return GCVO_OK;
+    };
+    bool done = false;   // the last look was after the last launch
     bool looped = sp->order == 2 && !ctx->profiling && loop_fits(np, pr, P.feat_dim, b.sub);
     if (looped) {
         // whole iterations in one cooperative kernel (loop.cu), which returns at
@@ -841,12 +849,13 @@ gcvo_status run_register(gcvo_ctx *ctx, int np, const gcvo_problem *pr, const gc
         const int blocks = (int)std::min<int64_t>(1 << 20, (2 * P.n_points / b.sub + PAIR_WARPS - 1) / PAIR_WARPS);
         for (int it = 0, look = LOOP_LOOK; it < sp->k_max; it += iters) {
             if (it >= look) {
-                GCVO_CUDA(cudaMemcpyAsync(h_active, n_active, sizeof(int), cudaMemcpyDeviceToHost, s));
-                GCVO_CUDA(cudaStreamSynchronize(s));
-                if (*h_active <= 0) break;
+                GCVO_TRY(look_at());
+                done = h_words[SRC_WORD_ACTIVE] <= 0;
+                if (done) break;
                 look = it + LOOP_LOOK;
             }
             la.max_iters = std::min(iters, sp->k_max - it);
+            la.resumed = it > 0;
             if (it > 0) GCVO_CUDA(cudaMemsetAsync(la.barrier, 0, sizeof(unsigned), s));
             const cudaError_t e = launch_loop(la, P.iso, P.feat_dim, b.sub, blocks, std::max(1, ctx->sm_count), s);
             if (it == 0 && e == cudaErrorCooperativeLaunchTooLarge) {
@@ -870,14 +879,15 @@ gcvo_status run_register(gcvo_ctx *ctx, int np, const gcvo_problem *pr, const gc
             GCVO_CUDA(cudaGraphLaunch(cg.exec, s));
             count_launches(cg.kernels);
             it += U;
-            GCVO_CUDA(cudaMemcpyAsync(h_active, n_active, sizeof(int), cudaMemcpyDeviceToHost, s));
-            GCVO_CUDA(cudaStreamSynchronize(s));
+            GCVO_TRY(look_at());
+            done = true;
             GCVO_TRY(collect_profile(ctx, true));
-            if (*h_active <= 0) break;
+            if (h_words[SRC_WORD_ACTIVE] <= 0) break;
         }
     }
     ctx->ev_used = 0;
-    GCVO_TRY(check_status_word(ctx));
+    if (!done) GCVO_TRY(look_at());
+    GCVO_TRY(status_of_word((unsigned)h_words[0]));
     std::vector<ProbDev> out(np);
     GCVO_CUDA(cudaMemcpyAsync(out.data(), ctx->probs.ptr, np * sizeof(ProbDev), cudaMemcpyDeviceToHost, s));
     if (logs)

@@ -70,7 +70,8 @@ __global__ void __launch_bounds__(PAIR_WARPS * 32, 5) k_loop(LoopArgs a) {
     bool ok = true;
     // nothing to do, or a wait of an earlier launch ran out (both change only
     // behind a barrier that every block has to reach, or to give up on)
-    if (*(volatile int *)a.fin.n_active <= 0 || (*(volatile unsigned *)a.pair.status_word & DEV_ERR_TIMEOUT)) return;
+    if (a.resumed && (*(volatile int *)a.fin.n_active <= 0 || (*(volatile unsigned *)a.pair.status_word & DEV_ERR_TIMEOUT)))
+        return;
     for (int it = 0; it < a.max_iters; ++it) {
         ok = tile_pass<PAIR_EVAL, ISO, FD, SUB>(a.pair, stage, parity);
         if (!__syncthreads_and(ok)) break;

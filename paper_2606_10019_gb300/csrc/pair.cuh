@@ -197,6 +197,7 @@ struct LoopArgs {
     TransformArgs tr;
     unsigned *barrier;   // zero before the launch
     int max_iters;
+    int resumed;         // not the first launch: there may be nothing left to do
 };
 cudaError_t launch_loop(const LoopArgs &a, bool iso, int fd, int sub, int blocks, int sm_count, cudaStream_t s);
 cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t s);

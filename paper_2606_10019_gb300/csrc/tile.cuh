@@ -408,6 +408,7 @@ __device__ __forceinline__ bool tile_pass(const PairArgs &a, StageT<MODE, FD> *s
             plz = L4.z;
         }
         const float rho2 = P->rho2, c2 = P->c2, iso_inv = P->iso_inv;
+        const float tails = P->tails;   // the limits below are tested on position heads
         // Two target lists per sub-tile (anisotropic kernel with a cutoff):
         // every pair within rho is counted (the pair-eval unit), but a pair
         // can only pass d^2 <= c^2 if |r|^2 <= c^2 lambda_max(Sigma_ij) <=
@@ -446,7 +447,6 @@ __device__ __forceinline__ bool tile_pass(const PairArgs &a, StageT<MODE, FD> *s
                 bmax[k] = ord_dec(__reduce_max_sync(FULL, ord_enc(sval ? pp[k] : -INFINITY)));
             }
         }
-        const float tails = P->tails;   // the limits are tested on position heads
         const float lam_sub = bounded ? ord_dec(__reduce_max_sync(FULL, ord_enc(lam_i))) : 0.f;
         // largest diagonal entries of Sigma'_j, the limits' slack included
         float dmax[3] = {0.f, 0.f, 0.f};
