@@ -90,7 +90,7 @@ namespace gcvo {
 
 static_assert(PAIR_WCAP <= 65535, "target list entries are 16-bit");
 static_assert(PAIR_SLOTS * 33 * 4 <= PAIR_WCAP * 32, "epilogue transpose fits in a warp's staged pos, ca");
-static_assert(PAIR_WARPS * (PAIR_WCAP * 80 + PAIR_WCAP * 4 + 64) <= 227 * 1024, "the largest block stage fits");
+static_assert(PAIR_WARPS * (PAIR_WCAP * 80 + PAIR_WCAP * 4 + 112) <= 227 * 1024, "the largest block stage fits");
 static_assert(PAIR_SLOTS_EXACT * 33 * 4 <= PAIR_WCAP * 48, "exact epilogue transpose fits in pos, ca, cb");
 
 // Per warp: staged target points (with their coordinate tails when LO and
@@ -105,6 +105,7 @@ struct __align__(16) WarpStage {
     float4 fx[FX ? PAIR_WCAP : 1];   // feature channels 3..6
     unsigned short list[PAIR_WCAP];    // staged targets within rho of the sub-tile box
     unsigned short listB[PAIR_WCAP];   // those of them within the per-pair bound
+    float4 lim[3];                     // the sub-tile's box and limits (see tile_pass)
     uint64_t bar;
 };
 
@@ -477,6 +478,15 @@ __device__ __forceinline__ bool tile_pass(const PairArgs &a, StageT<MODE, FD> *s
             const float ri = rho * 0.9999f - (dfr ? 1e-6f * mag : 0.f);
             rin2 = ri > 0.f ? ri * ri : -1.f;
         }
+        // the box and the limits wait in shared memory for the columns and the
+        // filters: in registers they would be carried through the evaluation
+        // loop, where 16 of them were spilled
+        if (lane == 0) {
+            S.lim[0] = make_float4(bmin[0], bmin[1], bmin[2], rc2);
+            S.lim[1] = make_float4(bmax[0], bmax[1], bmax[2], rin2);
+            S.lim[2] = make_float4(dmax[0], dmax[1], dmax[2], lam_box);
+        }
+        __syncwarp();
         int lo[3], hi[3];
         bool empty = !(bmin[0] <= bmax[0]);
 #pragma unroll
@@ -508,13 +518,14 @@ __device__ __forceinline__ bool tile_pass(const PairArgs &a, StageT<MODE, FD> *s
             if (c < n_cols) {
                 const int cx = lo[0] + c / ncy, cy = lo[1] + c % ncy;
                 const float x0 = G->corner[0] + (float)cx * h, y0 = G->corner[1] + (float)cy * h;
-                const float ddx = fmaxf(0.0f, fmaxf(x0 - bmax[0], bmin[0] - (x0 + h)));
-                const float ddy = fmaxf(0.0f, fmaxf(y0 - bmax[1], bmin[1] - (y0 + h)));
+                const float4 bl = S.lim[0], bh = S.lim[1];
+                const float ddx = fmaxf(0.0f, fmaxf(x0 - bh.x, bl.x - (x0 + h)));
+                const float ddy = fmaxf(0.0f, fmaxf(y0 - bh.y, bl.y - (y0 + h)));
                 const float d2xy = ddx * ddx + ddy * ddy;
-                if (d2xy <= rc2) {
-                    const float ez = sqrtf(rc2 - d2xy);
-                    const int czl = max(lo[2], (int)floorf(fmaxf((bmin[2] - ez - G->corner[2]) * ih, -1.0f)));
-                    const int czh = min(hi[2], (int)floorf(fminf((bmax[2] + ez - G->corner[2]) * ih, (float)dzs)));
+                if (d2xy <= bl.w) {
+                    const float ez = sqrtf(bl.w - d2xy);
+                    const int czl = max(lo[2], (int)floorf(fmaxf((bl.z - ez - G->corner[2]) * ih, -1.0f)));
+                    const int czh = min(hi[2], (int)floorf(fminf((bh.z + ez - G->corner[2]) * ih, (float)dzs)));
                     if (czl <= czh) {
                         const size_t base = ((size_t)cx * dy + cy) * dzs;
                         rs = __ldg(G->vox_first + base + czl);
@@ -571,29 +582,30 @@ __device__ __forceinline__ bool tile_pass(const PairArgs &a, StageT<MODE, FD> *s
                 // whose pairs have to be counted one by one (list), and
                 // those within the per-pair bounds (listB), evaluated.
                 int L = 0, LB = 0, inside = 0;
+                const float4 bl = S.lim[0], bh = S.lim[1], lim = S.lim[2];
                 for (int t0 = 0; t0 < m; t0 += 32) {
                     const int tt = t0 + lane;
                     bool hit = false, near = false, count = false;
                     if (tt < m) {
                         const float4 x = S.pos[tt];
-                        const float ex = bmin[0] - x.x, fx = x.x - bmax[0];
-                        const float ey = bmin[1] - x.y, fy = x.y - bmax[1];
-                        const float ez = bmin[2] - x.z, fz = x.z - bmax[2];
+                        const float ex = bl.x - x.x, fx = x.x - bh.x;
+                        const float ey = bl.y - x.y, fy = x.y - bh.y;
+                        const float ez = bl.z - x.z, fz = x.z - bh.z;
                         const float dx = fmaxf(0.f, fmaxf(ex, fx));
                         const float dyy = fmaxf(0.f, fmaxf(ey, fy));
                         const float dz = fmaxf(0.f, fmaxf(ez, fz));
                         const float db2 = dx * dx + dyy * dyy + dz * dz;
-                        hit = count = db2 <= rc2;
+                        hit = count = db2 <= bl.w;
                         if (two_lists && hit) {
                             const float4 ca = S.ca[tt], cbv = S.cb[tt];
                             const float gx = fminf(ex, fx), gy = fminf(ey, fy), gz = fminf(ez, fz);
-                            count = gx * gx + gy * gy + gz * gz > rin2;
+                            count = gx * gx + gy * gy + gz * gz > bh.w;
                             const float lam_j = sqrt_approx(ca.x * ca.x + ca.w * ca.w + cbv.y * cbv.y +
                                                             2.f * (ca.y * ca.y + ca.z * ca.z + cbv.x * cbv.x));
                             const float c2m = c2 * 1.01f, sl = c2 * 1e-5f * lam_j + 1e-12f;
-                            near = db2 <= c2 * (lam_box + lam_j) * 1.001f + 1e-12f &&
-                                   dx * dx <= c2m * (dmax[0] + ca.x) + sl && dyy * dyy <= c2m * (dmax[1] + ca.w) + sl &&
-                                   dz * dz <= c2m * (dmax[2] + cbv.y) + sl;
+                            near = db2 <= c2 * (lim.w + lam_j) * 1.001f + 1e-12f &&
+                                   dx * dx <= c2m * (lim.x + ca.x) + sl && dyy * dyy <= c2m * (lim.y + ca.w) + sl &&
+                                   dz * dz <= c2m * (lim.z + cbv.y) + sl;
                         }
                     }
                     const unsigned bal = __ballot_sync(FULL, count);
