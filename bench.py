@@ -41,15 +41,15 @@ UNIT = "pair-evals/s"
 FLOP_PER_PAIR = 76          # FP32 flops (FMA = 2) of one pair evaluation
 FLOP_PER_PAIR_EXACT = 232   # the G-CVO-E pass: the 76 above plus y, Sigma'y, u, K and the S_yy, S_B sums
 # DRAM bytes per active point (source + target) of one launch of the pair
-# kernel's evaluation pass: 112.75 MB over 1,201,176 points in one ncu
-# capture of the first iteration of the 64-problem batch (4 points per
+# kernel's evaluation pass: 92.45 MB over 1,201,176 points in one ncu
+# capture of the first iteration of the 64-problem batch (16 points per
 # sub-tile in that capture), from the kernel whose source (PAIR_KERNEL_FILES)
 # hashes to PAIR_KERNEL_SHA.  The pass reads every point of an active
 # problem once and writes one partial row per sub-tile, so its traffic grows
 # with the active points; the traffic is reported only while the source
 # still matches.
-PAIR_DRAM_BYTES_PER_POINT = 112.750848e6 / 1201176
-PAIR_KERNEL_SHA = "7b263fa72408aff8"
+PAIR_DRAM_BYTES_PER_POINT = 92.449792e6 / 1201176
+PAIR_KERNEL_SHA = "6c0a34b445574d1c"
 PAIR_KERNEL_FILES = ("tile.cuh", "tile.cu")
 EIG_MAX = 0.09              # (0.3 m)^2: eigenvalue bound for the 0.3 m voxel scans
 
@@ -356,7 +356,7 @@ def run_gcvo(args, rank, world):
     peak = sm_count * 128 * 2 * clock_ghz / 1e3      # FP32 TFLOP/s at the maximum SM clock
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": traffic,
-                "traffic_basis": "DRAM bytes per active point (93.9 B, ncu capture of the first iteration of the "
+                "traffic_basis": "DRAM bytes per active point (77.0 B, ncu capture of the first iteration of the "
                                  "64-problem batch) x mean active points per launch; null if the kernel source "
                                  "changed since the capture",
                 "active_points_per_launch": active_points / n_launch,
@@ -789,9 +789,10 @@ def learned_proposal_block(G, ctx, dev, frames, T_true_frames, n_train=100_000, 
     ev1.record()
     torch.cuda.synchronize(dev)
     t_train = time.perf_counter() - t2
-    # point MLP 4-64-128-256: forward 2 (4*64 + 64*128 + 128*256) flops a point,
-    # backward about twice that; two clouds of n points per pair
-    flop_step = batch_size * 2 * n * 3 * 2 * (4 * 64 + 64 * 128 + 128 * 256)
+    # point MLP 4-64-128-256: forward 2 (4*64 + 64*128 + 128*256) flops a point, two
+    # clouds of n points per pair; backward about twice that for the largest
+    # point of each of a cloud's 256 channels
+    flop_step = batch_size * 2 * (n + 2 * 256) * 2 * (4 * 64 + 64 * 128 + 128 * 256)
     train_tflops = flop_step * steps / (ev0.elapsed_time(ev1) / 1e3) / 1e12
     del sx, tx, sf, tf
     # held-out evaluation
@@ -864,8 +865,9 @@ def learned_proposal_block(G, ctx, dev, frames, T_true_frames, n_train=100_000, 
                       "point_mlp_tflops_incl_head_and_adam": train_tflops,
                       "bf16_peak_tflops": _measured_bf16_peak()[0], "bf16_peak_basis": _measured_bf16_peak()[1],
                       "frac_of_bf16_peak": train_tflops / _measured_bf16_peak()[0],
-                      "flop_basis": "3 x 2 (4*64 + 64*128 + 128*256) flops per point per step (forward + "
-                                    "backward of the shared MLP), over the CUDA-event time of the whole step"},
+                      "flop_basis": "2 (4*64 + 64*128 + 128*256) flops per point of the forward shared MLP, twice "
+                                    "that per channel's largest point in the backward (256 per cloud), over the "
+                                    "CUDA-event time of the whole step"},
             **arms,
             "proposal_gain_over_batched_identity": arms["batched_with_proposal"]["registrations_per_s"]
             / arms["batched_from_identity"]["registrations_per_s"],

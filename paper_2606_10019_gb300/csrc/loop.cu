@@ -11,9 +11,11 @@
 // Measured: a registration of 22 iterations at 2,000 points 940 -> 685 us (31
 // us an iteration; pair pass 12, its barrier 6, finalize 9 to 12, transform and
 // barrier 3), the tracking of a LiDAR frame 1454 -> 1274 us.  Of this 108 and
-// 47 us are the finalize's step in fewer FP64 instructions (fin.cuh); a batch of
-// 64 pairs, whose phases are long against the launches, 27.4 -> 27.3 ms.  The
-// other orders, and a context that times its kernels, keep the graphs.
+// 47 us are the finalize's step in fewer FP64 instructions (fin.cuh).  On batches
+// of 50,000 to 600,000 points, whose phases are long against the launches, the
+// graphs are 1 to 5 % faster while most problems are active, and this kernel
+// where few run on (128 pairs, one of them to 186 iterations: 94.9 -> 79.7 ms).
+// The other orders, and a context that times its kernels, keep the graphs.
 //
 // The blocks of a cooperative launch are all resident, so the barrier's spin
 // ends; it is bounded all the same.  They hold every SM, and the kernels of other
