@@ -196,8 +196,7 @@ gcvo_status gcvo_set_workspace(gcvo_ctx *ctx, void *dev_ptr, size_t bytes, int64
  * nearest points (the point itself included, ties broken by lower index),
  * then each eigenvalue is clamped to [eig_max/eig_ratio, eig_max].
  * xyz: 3 x n input; cov_out: 6 x n output, device memory, caller-owned.
- * Requires n >= knn.  Synchronises the stream (the search reads back how
- * many points need the coarse second pass, and its status). */
+ * Requires n >= knn.  Synchronises the stream (the status is read back). */
 gcvo_status gcvo_estimate_covariances(gcvo_ctx *ctx, const float *xyz, int64_t n,
                                       const gcvo_kernel_params *params, float *cov_out);
 
@@ -229,10 +228,9 @@ gcvo_status gcvo_grid_destroy(gcvo_grid *grid);
 /* gcvo_estimate_covariances for n_clouds clouds in one call: cloud k has
  * n[k] points at xyz[k] (3 x n[k]) and its covariances go to cov_out[k]
  * (6 x n[k]); all device memory.  All clouds share one set of launches on
- * the context's stream: their points are gathered into one array, every
- * cloud gets its own voxel box and size, and one sort and one hash table
- * (voxel keys offset per cloud) serve the batch, so the cost no longer
- * grows with the number of clouds beyond their points.  The results equal
+ * the context's stream: every cloud is sorted by its own voxels, one
+ * thread-block cluster each, and one search serves the batch, so the cost no
+ * longer grows with the number of clouds beyond their points.  The results equal
  * those of one call per cloud, bit for bit (the neighbour lists do not
  * depend on the voxel grid).  Synchronises the stream; a failure (a
  * non-finite coordinate in any cloud) fails the whole call. */
@@ -294,9 +292,8 @@ gcvo_status gcvo_register(gcvo_ctx *ctx, const gcvo_grid *target, const float *s
                           const gcvo_solver_params *params, double T_out[16], gcvo_iter_log *log, int *n_iter);
 
 /* Algorithm 1 for n_problems independent problems in one set of launches:
- * every iteration evaluates all still-active problems in one pair-kernel
- * launch and updates them in one reduction and one solver launch; a
- * problem that converged
+ * every iteration evaluates all still-active problems in one pair pass and
+ * updates them in one finalize; a problem that converged
  * or failed is masked out.  T_out: n_problems x 16 (host); logs: n_problems
  * x k_max rows (host, may be NULL); n_iter and status: n_problems (host).
  * The call returns GCVO_OK when every problem ran (per-problem outcomes
