@@ -255,7 +255,8 @@ extern "C" gcvo_status gcvo_eval_static(const gcvo_grid *target, const float *sr
     GCVO_CUDA(cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev));
     int per_sm = pair_blocks_per_sm(PAIR_EVAL, iso, fd, NA_SUB);
     int grid = std::max(1, std::min(n_items, std::max(1, per_sm) * sm));
-    GCVO_CUDA(launch_pair(pa, PAIR_EVAL, iso, fd, NA_SUB, grid, s));
+    static_assert(NA_SUB == 8, "the sub-tiles of the pass over points in no order");
+    GCVO_CUDA(launch_pair_unsorted(pa, iso, fd, grid, s));
     fa.mode = FIN_EVAL;
     fa.reduce_blocks = std::min((n_items + FIN_CHUNK - 1) / FIN_CHUNK, std::max(1, sm) * 8);
     fa.work = words;

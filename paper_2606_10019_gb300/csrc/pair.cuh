@@ -189,6 +189,8 @@ gcvo_status launch_src_one(const SrcOneArgs &a, cudaStream_t s);
 int pair_sub_for(int mode, int sub);
 int pair_blocks_per_sm(int mode, bool iso, int fd, int sub);
 cudaError_t launch_pair(const PairArgs &a, int mode, bool iso, int fd, int sub, int grid, cudaStream_t s);
+// The evaluation pass over points in no order, in sub-tiles of 8 (up to 3 feature channels).
+cudaError_t launch_pair_unsorted(const PairArgs &a, bool iso, int fd, int grid, cudaStream_t s);
 // The register loop of G-CVO-2 (loop.cu): up to max_iters iterations, or until
 // no problem is active, in one cooperative launch of at most `blocks` blocks.
 struct LoopArgs {

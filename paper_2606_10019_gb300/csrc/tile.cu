@@ -8,13 +8,13 @@
 namespace gcvo {
 namespace {
 
-template <int MODE, bool ISO, int FD, int SUB>
+template <int MODE, bool ISO, int FD, int SUB, bool WIDE = false>
 __global__ void __launch_bounds__(PAIR_WARPS * 32, MODE == PAIR_EVAL ? 5 : 4) k_tile(PairArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];   // PAIR_WARPS stages
     StageT<MODE, FD> *stage = reinterpret_cast<StageT<MODE, FD> *>(smem_raw);
     tile_init(stage);
     unsigned parity = 0;
-    tile_pass<MODE, ISO, FD, SUB>(a, stage, parity);
+    tile_pass<MODE, ISO, FD, SUB, WIDE>(a, stage, parity);
 }
 
 // Work-item packing over the sorted source points (keys: problem << 30 |
@@ -92,20 +92,20 @@ __global__ void __launch_bounds__(CHUNK_THREADS) k_chunk_ranges(int np, ProbDev 
 // Host launchers.
 // ---------------------------------------------------------------------------
 // The opt-in above the 48 KB default, made once per kernel instance and device.
-template <int MODE, bool ISO, int FD, int SUB>
+template <int MODE, bool ISO, int FD, int SUB, bool WIDE = false>
 static cudaError_t tile_smem_optin() {
     static PerDevice<cudaError_t> once;
     return once.get([] {
-        return cudaFuncSetAttribute(k_tile<MODE, ISO, FD, SUB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        return cudaFuncSetAttribute(k_tile<MODE, ISO, FD, SUB, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)tile_smem_bytes<MODE, FD>());
     });
 }
 
-template <int MODE, bool ISO, int FD, int SUB>
+template <int MODE, bool ISO, int FD, int SUB, bool WIDE = false>
 static cudaError_t launch_tile_t(const PairArgs &a, int grid, cudaStream_t s) {
-    const cudaError_t e = tile_smem_optin<MODE, ISO, FD, SUB>();
+    const cudaError_t e = tile_smem_optin<MODE, ISO, FD, SUB, WIDE>();
     if (e != cudaSuccess) return e;
-    k_tile<MODE, ISO, FD, SUB><<<grid, PAIR_WARPS * 32, tile_smem_bytes<MODE, FD>(), s>>>(a);
+    k_tile<MODE, ISO, FD, SUB, WIDE><<<grid, PAIR_WARPS * 32, tile_smem_bytes<MODE, FD>(), s>>>(a);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -149,6 +149,12 @@ cudaError_t launch_pair(const PairArgs &a, int mode, bool iso, int fd, int sub, 
     PAIR_VARIANTS(L)
 #undef L
     return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_pair_unsorted(const PairArgs &a, bool iso, int fd, int grid, cudaStream_t s) {
+    if (iso) return launch_pair(a, PAIR_EVAL, true, fd, 8, grid, s);   // one list anyway
+    return fd <= 1 ? launch_tile_t<PAIR_EVAL, false, 1, 8, true>(a, grid, s)
+                   : launch_tile_t<PAIR_EVAL, false, 3, 8, true>(a, grid, s);
 }
 
 gcvo_status pack_items(int np, const unsigned long long *keys, int64_t n, int sub, int level,

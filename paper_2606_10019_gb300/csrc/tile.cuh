@@ -315,8 +315,9 @@ __device__ __forceinline__ void ls_terms(float wgt, float kr1, float kr2, float 
 
 // The work items of one pass, by all warps of the grid.  stage: the block's
 // stages, with their barriers set up (tile_init); parity: this warp's, kept
-// from pass to pass.  False when a bounded wait ran out.
-template <int MODE, bool ISO, int FD, int SUB>
+// from pass to pass.  False when a bounded wait ran out.  WIDE: the points come
+// in no order, so that a sub-tile's box may span the scene.
+template <int MODE, bool ISO, int FD, int SUB, bool WIDE = false>
 __device__ __forceinline__ bool tile_pass(const PairArgs &a, StageT<MODE, FD> *stage, unsigned &parity) {
     static_assert(SUB == 4 || SUB == 8 || SUB == 16 || SUB == 32, "sub-tile of 4, 8, 16 or 32 points");
     static_assert(FD == 1 || FD == 3 || FD == 7, "1, up to 3 or up to 7 feature channels");
@@ -586,42 +587,53 @@ __device__ __forceinline__ bool tile_pass(const PairArgs &a, StageT<MODE, FD> *s
                 // One list: all of them, evaluated and counted.  Two: those
                 // whose pairs have to be counted one by one (list), and
                 // those within the per-pair bounds (listB), evaluated.
-                int L = 0, LB = 0, inside = 0;
+                int L, LB, inside;
                 const float4 bl = S.lim[0], bh = S.lim[1], lim = S.lim[2];
-                for (int t0 = 0; t0 < m; t0 += 32) {
-                    const int tt = t0 + lane;
-                    bool hit = false, near = false, count = false;
-                    if (tt < m) {
-                        const float4 x = S.pos[tt];
-                        const float ex = bl.x - x.x, fx = x.x - bh.x;
-                        const float ey = bl.y - x.y, fy = x.y - bh.y;
-                        const float ez = bl.z - x.z, fz = x.z - bh.z;
-                        const float dx = fmaxf(0.f, fmaxf(ex, fx));
-                        const float dyy = fmaxf(0.f, fmaxf(ey, fy));
-                        const float dz = fmaxf(0.f, fmaxf(ez, fz));
-                        const float db2 = dx * dx + dyy * dyy + dz * dz;
-                        hit = count = db2 <= bl.w;
-                        if (two_lists && hit) {
-                            const float4 ca = S.ca[tt], cbv = S.cb[tt];
-                            const float gx = fminf(ex, fx), gy = fminf(ey, fy), gz = fminf(ez, fz);
-                            count = gx * gx + gy * gy + gz * gz > bh.w;
-                            const float lam_j = sqrt_approx(ca.x * ca.x + ca.w * ca.w + cbv.y * cbv.y +
-                                                            2.f * (ca.y * ca.y + ca.z * ca.z + cbv.x * cbv.x));
-                            const float c2m = c2 * 1.01f, sl = c2 * 1e-5f * lam_j + 1e-12f;
-                            near = db2 <= c2 * (lim.w + lam_j) * 1.001f + 1e-12f &&
-                                   dx * dx <= c2m * (lim.x + ca.x) + sl && dyy * dyy <= c2m * (lim.y + ca.w) + sl &&
-                                   dz * dz <= c2m * (lim.z + cbv.y) + sl;
+                bool split = two_lists;
+                for (;;) {
+                    L = LB = inside = 0;
+                    for (int t0 = 0; t0 < m; t0 += 32) {
+                        const int tt = t0 + lane;
+                        bool hit = false, near = false, count = false;
+                        if (tt < m) {
+                            const float4 x = S.pos[tt];
+                            const float ex = bl.x - x.x, fx = x.x - bh.x;
+                            const float ey = bl.y - x.y, fy = x.y - bh.y;
+                            const float ez = bl.z - x.z, fz = x.z - bh.z;
+                            const float dx = fmaxf(0.f, fmaxf(ex, fx));
+                            const float dyy = fmaxf(0.f, fmaxf(ey, fy));
+                            const float dz = fmaxf(0.f, fmaxf(ez, fz));
+                            const float db2 = dx * dx + dyy * dyy + dz * dz;
+                            hit = count = db2 <= bl.w;
+                            if (split && hit) {
+                                const float4 ca = S.ca[tt], cbv = S.cb[tt];
+                                const float gx = fminf(ex, fx), gy = fminf(ey, fy), gz = fminf(ez, fz);
+                                count = gx * gx + gy * gy + gz * gz > bh.w;
+                                const float lam_j = sqrt_approx(ca.x * ca.x + ca.w * ca.w + cbv.y * cbv.y +
+                                                                2.f * (ca.y * ca.y + ca.z * ca.z + cbv.x * cbv.x));
+                                const float c2m = c2 * 1.01f, sl = c2 * 1e-5f * lam_j + 1e-12f;
+                                near = db2 <= c2 * (lim.w + lam_j) * 1.001f + 1e-12f &&
+                                       dx * dx <= c2m * (lim.x + ca.x) + sl && dyy * dyy <= c2m * (lim.y + ca.w) + sl &&
+                                       dz * dz <= c2m * (lim.z + cbv.y) + sl;
+                            }
+                        }
+                        const unsigned bal = __ballot_sync(FULL, count);
+                        if (count) S.list[L + __popc(bal & lt_mask)] = (unsigned short)tt;
+                        L += __popc(bal);
+                        if (split) {
+                            const unsigned balB = __ballot_sync(FULL, near);
+                            if (near) S.listB[LB + __popc(balB & lt_mask)] = (unsigned short)tt;
+                            LB += __popc(balB);
+                            inside += __popc(__ballot_sync(FULL, hit && !count));
                         }
                     }
-                    const unsigned bal = __ballot_sync(FULL, count);
-                    if (count) S.list[L + __popc(bal & lt_mask)] = (unsigned short)tt;
-                    L += __popc(bal);
-                    if (two_lists) {
-                        const unsigned balB = __ballot_sync(FULL, near);
-                        if (near) S.listB[LB + __popc(balB & lt_mask)] = (unsigned short)tt;
-                        LB += __popc(balB);
-                        inside += __popc(__ballot_sync(FULL, hit && !count));
-                    }
+                    // counting apart costs a fifth of an evaluation: where the second
+                    // list saves less, once more as one list (40,000 points in no
+                    // order: 6.3 -> 5.6 ms; sorted ones, whose boxes are small, would
+                    // pay up to 2 % for the question)
+                    if (!WIDE || !split || 5 * (L + inside - LB) >= L) break;
+                    split = false;
+                    __syncwarp();
                 }
                 __syncwarp();
                 if (qi == 0 && sval) {
@@ -629,9 +641,9 @@ __device__ __forceinline__ bool tile_pass(const PairArgs &a, StageT<MODE, FD> *s
                     n_pairs += inside;
                 }
                 // the evaluated list: listB follows list in the stage
-                const int eoff = two_lists ? PAIR_WCAP : 0;
-                const int EL = two_lists ? LB : L;
-                if (two_lists) {
+                const int eoff = split ? PAIR_WCAP : 0;
+                const int EL = split ? LB : L;
+                if (split) {
                     // counted with the same r as the evaluation forms
                     for (int j = 0; j < L; j += TQ) {
                         const int idx = j + qi;
@@ -754,7 +766,7 @@ __device__ __forceinline__ bool tile_pass(const PairArgs &a, StageT<MODE, FD> *s
                         ls_terms(wgt, kr1, kr2, kr3, kr4, a11, a12, a13, a22, a.ls_literal, t);
                     }
                 }
-                if (!two_lists) n_pairs += npe;
+                if (!split) n_pairs += npe;
                 npe = 0;
                 __syncwarp();   // the list and staged points are reused by the next chunk
             }
