@@ -41,15 +41,15 @@ UNIT = "pair-evals/s"
 FLOP_PER_PAIR = 76          # FP32 flops (FMA = 2) of one pair evaluation
 FLOP_PER_PAIR_EXACT = 232   # the G-CVO-E pass: the 76 above plus y, Sigma'y, u, K and the S_yy, S_B sums
 # DRAM bytes per active point (source + target) of one launch of the pair
-# kernel's evaluation pass: 92.45 MB over 1,201,176 points in one ncu
-# capture of the first iteration of the 64-problem batch (16 points per
+# kernel's evaluation pass: 97.33 MB over 1,201,176 points in one ncu
+# capture of the first iteration of the 64-problem batch (8 points per
 # sub-tile in that capture), from the kernel whose source (PAIR_KERNEL_FILES)
 # hashes to PAIR_KERNEL_SHA.  The pass reads every point of an active
 # problem once and writes one partial row per sub-tile, so its traffic grows
 # with the active points; the traffic is reported only while the source
 # still matches.
-PAIR_DRAM_BYTES_PER_POINT = 92.449792e6 / 1201176
-PAIR_KERNEL_SHA = "6c0a34b445574d1c"
+PAIR_DRAM_BYTES_PER_POINT = 97.334784e6 / 1201176
+PAIR_KERNEL_SHA = "01c419c83865a0c8"
 PAIR_KERNEL_FILES = ("tile.cuh", "tile.cu")
 EIG_MAX = 0.09              # (0.3 m)^2: eigenvalue bound for the 0.3 m voxel scans
 
@@ -356,7 +356,7 @@ def run_gcvo(args, rank, world):
     peak = sm_count * 128 * 2 * clock_ghz / 1e3      # FP32 TFLOP/s at the maximum SM clock
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": traffic,
-                "traffic_basis": "DRAM bytes per active point (77.0 B, ncu capture of the first iteration of the "
+                "traffic_basis": "DRAM bytes per active point (81.0 B, ncu capture of the first iteration of the "
                                  "64-problem batch) x mean active points per launch; null if the kernel source "
                                  "changed since the capture",
                 "active_points_per_launch": active_points / n_launch,
